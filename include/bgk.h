@@ -363,7 +363,7 @@ BGK_API bgk_status bgk_adjoint_lid_shear(bgk_solver* s, int64_t nsteps, int chec
  * fixed device-memory budget handed out by its host framework, or code on a
  * path where cudaMalloc's implicit device-wide synchronisation is not
  * allowed.  For them this call advances one state by one step using only
- * the buffers the caller passes plus a fixed 384 KiB scratch array compiled
+ * the buffers the caller passes plus a fixed 480 KiB scratch array compiled
  * into the library (held on every GPU that loads libbgk.so until the process
  * exits).  The scratch holds the per-velocity tables (about 120 bytes per
  * velocity) and the error flag, which limits this call to about 3260

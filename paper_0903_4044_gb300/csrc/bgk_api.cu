@@ -59,7 +59,10 @@ struct bgk_solver {
   double4_32a* mom_tmp = nullptr;   // scratch for bgk_moments(which = 0)
   double4_32a* flux_tmp = nullptr;  // scratch for bgk_wall_fluxes
   double* cx = nullptr;
-  double* cy = nullptr;  // [2 nvy]: centres, then their squares
+  double* cy = nullptr;  // [2 nvy]: centres, then the fixed-point y weights
+  uint64_t* wx = nullptr;  // [nvx] fixed-point x weights
+  double* sx = nullptr;     // [nvx] column scales
+  double2* ratio = nullptr;  // [nv]
   double4_32a* coef = nullptr;
   int* shift = nullptr;
   double2* cxy = nullptr;
@@ -83,11 +86,16 @@ struct bgk_solver {
   int64_t device_bytes = 0;
   double max_courant = 0.0;
 
+  uint64_t* y_weights() const { return reinterpret_cast<uint64_t*>(cy + P.nvy); }
   bgk::Tables tables() const {
     bgk::Tables T;
     T.cx = cx;
     T.cy = cy;
-    T.cy2 = cy + P.nvy;
+    T.grid = bgk::velocity_grid(P);
+    T.wx = wx;
+    T.wy = y_weights();
+    T.sx = sx;
+    T.ratio = ratio;
     T.coef = coef;
     T.shift = shift;
     T.cxy = cxy;
@@ -231,6 +239,7 @@ bgk_status validate(const bgk_config* c, bgk::Params* P, double* max_courant) {
     p.dt = c->cfl / (mx / p.dx + my / p.dy);
   }
   *max_courant = c->dim == 1 ? mx * p.dt / p.dx : mx * p.dt / p.dx + my * p.dt / p.dy;
+  if (c->dim == 2 && c->precision == BGK_F64) bgk::step_f64_plan(p, *max_courant);
 
   // cells per CTA: the caller's choice (checked here), else chosen in
   // bgk_create once the device's SM count is known
@@ -292,14 +301,22 @@ bgk_status validate(const bgk_config* c, bgk::Params* P, double* max_courant) {
 }
 
 // Largest tile (cells per CTA) that keeps two CTAs' shared memory within an
-// SM and still gives every SM at least two CTAs.  FP64 takes 8 cells per CTA
-// (4 CTAs per SM) only in 2D with at least three full waves of them: the
-// per-cell solve then serves 8 cells per warp instruction (measured 2.6 %
-// faster on 256^2 x 48^2, and 2.8 % on the gradient of the 128^2 x 32^2
-// cavity); on fewer cells the last wave leaves SMs idle (7 % slower on
-// 64^2 x 32^2), and 4 cells per CTA are kept.
+// SM and still gives every SM at least two CTAs.  The fixed-point FP64 step
+// runs 8 warps per CTA at every tile: 8 cells share one scalar solve, 4 or 2
+// cells split each over 2 or 4 warps.  Measured us per step (2 / 4 / 8 cells):
+// 16^2 x 16^2 19 / 21 / 25, 32^2 x 32^2 53 / 49 / 63, 64^2 x 32^2 130 / 105 /
+// 108, 64^2 x 48^2 233 / 211 / 244, 96^2 x 20^2 221 / 140 / 107, 128^2 x 32^2
+// 424 / 332 / 316, 256^2 x 48^2 3020 / 2630 / 2360: 8 from three full waves
+// (4 CTAs per SM) on, and from 40 cells per SM on grids of few velocities,
+// where the solve weighs more.
 int auto_tile(const bgk::Params& P, int prec, int sms) {
   const long long ncell = (long long)P.nx * P.ny;
+  if (prec == BGK_F64 && P.dim == 2 && P.lane_bits) {
+    if (ncell >= 96LL * sms || (P.nv <= 640 && ncell >= 40LL * sms)) return 8;
+    return ncell >= 5LL * sms ? 4 : 2;
+  }
+  // FP64-only form, 2D: 8 cells per CTA with at least three full waves (4 CTAs
+  // per SM)
   if (prec == BGK_F64 && P.dim == 2 && ncell >= 8LL * 4 * 3 * sms && step_smem(P, prec, 8) <= kAutoSmem) return 8;
   // FP32, 2D, at least 3 groups of 4 velocities per streaming thread: the
   // pipelined one-cell kernel (measured 9 % faster than 2 cells per CTA on
@@ -327,7 +344,7 @@ void release(bgk_solver* s) {
   for (auto& g : s->graph)
     if (g) cudaGraphExecDestroy(g);
   void* bufs[] = {s->f[0], s->f[1], s->stage, s->mom_step, s->mom_tmp, s->flux_tmp, s->cx, s->cy,
-                  s->coef, s->shift, s->cxy, s->vinfo, s->ghost, s->emitted, s->m_coef, s->m_cx,
+                  s->coef, s->shift, s->cxy, s->vinfo, s->ghost, s->emitted, s->wx, s->sx, s->ratio, s->m_coef, s->m_cx,
                   s->m_cy, s->m_ax, s->m_ay, s->m_ghost, s->m_mabs, s->m_sums, s->m_ctr, s->err};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -519,6 +536,9 @@ bgk_status bgk_create(const bgk_config* cfg, bgk_solver** out) {
   ALLOC(flux_tmp, nfc);
   ALLOC(cx, P.nvx);
   ALLOC(cy, 2 * (size_t)P.nvy);
+  ALLOC(wx, P.nvx);
+  ALLOC(sx, P.nvx);
+  ALLOC(ratio, P.nv);
   ALLOC(coef, P.nv);
   ALLOC(shift, P.nv);
   ALLOC(cxy, P.nv);
@@ -535,7 +555,7 @@ bgk_status bgk_create(const bgk_config* cfg, bgk_solver** out) {
   if (e == cudaSuccess && s->m_ctr) e = cudaMemsetAsync(s->m_ctr, 0, 2 * sizeof(unsigned), s->stream);
   if (e == cudaSuccess)
     e = bgk::launch_build_tables(P, s->cx, s->cy, s->coef, s->shift, s->cxy, s->vinfo, s->ghost,
-                                 s->emitted, s->stream);
+                                 s->emitted, s->wx, s->y_weights(), s->sx, s->ratio, s->stream);
   if (e == cudaSuccess && s->prec != bgk::PREC_F64) e = bgk::launch_build_mixed_tables(P, s->tables(), s->mtables(), s->stream);
   if (e == cudaSuccess) e = s->prec == bgk::PREC_F64 ? bgk::prepare_step_f64(P) : bgk::prepare_step_mixed(P, s->prec);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -798,9 +818,11 @@ bgk_status bgk_sync(bgk_solver* s) {
 namespace {
 
 constexpr size_t kNoAllocScratchBytes = 384 * 1024;  // about 120 bytes per velocity
+// behind it: x weights and scales (nvy >= 2), ratios
+constexpr size_t kNoAllocWeightBytes = (sizeof(uint64_t) + sizeof(double)) * bgk::kMaxNv / 2 + sizeof(double2) * bgk::kMaxNv;
 constexpr int kNoAllocMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + kNoAllocWeightBytes];
 
 std::mutex g_noalloc_mutex;
 void* g_noalloc_ptr[kNoAllocMaxDevices] = {};
@@ -844,14 +866,15 @@ extern "C" bgk_status bgk_step_noalloc(const bgk_config* cfg, const double* f_in
   if (a < b + elems * sizeof(double2) && b < a + elems * sizeof(double2))
     return fail(BGK_ERR_INVALID_ARG, "f_in and f_out overlap");
 
-  // scratch layout: tables then the error flag, each 256-byte aligned
+  // scratch layout: tables then the error flag, each 256-byte aligned; the
+  // x weights, scales and ratios follow at kNoAllocScratchBytes
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t at = off;
     off = align256(off + bytes);
     return at;
   };
-  const size_t o_cx = take(sizeof(double) * P.nvx), o_cy = take(sizeof(double) * 2 * P.nvy);
+  const size_t o_cx = take(sizeof(double) * P.nvx), o_cy = take((sizeof(double) + sizeof(uint64_t)) * P.nvy);
   const size_t o_coef = take(sizeof(double4_32a) * P.nv), o_shift = take(sizeof(int) * P.nv);
   const size_t o_cxy = take(sizeof(double2) * P.nv), o_vinfo = take(sizeof(int) * P.nv);
   const size_t o_ghost = take(sizeof(double2) * bgk::kFaces * P.nv);
@@ -884,9 +907,17 @@ extern "C" bgk_status bgk_step_noalloc(const bgk_config* cfg, const double* f_in
   double2* ghost = (double2*)(base + o_ghost);
   double* emitted = (double*)(base + o_emit);
   int* err = (int*)(base + o_err);
+  uint64_t* wx = (uint64_t*)(base + kNoAllocScratchBytes);
+  uint64_t* wy = (uint64_t*)(cy + P.nvy);
+  double* sx = (double*)(wx + bgk::kMaxNv / 2);
+  double2* ratio = (double2*)(sx + bgk::kMaxNv / 2);
   T.cx = cx;
   T.cy = cy;
-  T.cy2 = cy + P.nvy;
+  T.grid = bgk::velocity_grid(P);
+  T.wx = wx;
+  T.wy = wy;
+  T.sx = sx;
+  T.ratio = ratio;
   T.coef = coef;
   T.shift = shift;
   T.cxy = cxy;
@@ -896,7 +927,7 @@ extern "C" bgk_status bgk_step_noalloc(const bgk_config* cfg, const double* f_in
 
   cudaStream_t stream = (cudaStream_t)cfg->cuda_stream;
   e = cudaMemsetAsync(err, 0, sizeof(int), stream);
-  if (e == cudaSuccess) e = bgk::launch_build_tables(P, cx, cy, coef, shift, cxy, vinfo, ghost, emitted, stream);
+  if (e == cudaSuccess) e = bgk::launch_build_tables(P, cx, cy, coef, shift, cxy, vinfo, ghost, emitted, wx, wy, sx, ratio, stream);
   if (e == cudaSuccess) e = bgk::prepare_step_f64(P);
   if (e == cudaSuccess)
     e = bgk::launch_step_f64(P, T, (const double2*)f_in, (double2*)f_out, (double4_32a*)mom_out, err, stream);

@@ -13,7 +13,8 @@ __device__ __forceinline__ double centre(double vmin, int j, double dc) {
 
 // Per-velocity streaming weights and boundary Maxwellians.
 __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32a* coef, int* shift,
-                              double2* cxy, int* vinfo, double2* ghost) {
+                              double2* cxy, int* vinfo, double2* ghost, uint64_t* wx, uint64_t* wy, double* sx,
+                              double2* ratio) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= P.nv) return;
   const int jx = j % P.nvx, jy = j / P.nvx;
@@ -21,7 +22,6 @@ __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32
   const double cyj = (P.dim == 2) ? centre(P.vy_min, jy, P.dcy) : 0.0;
   if (jy == 0) cx[jx] = cxj;
   if (jx == 0) cy[jy] = cyj;
-  if (jx == 0) cy[P.nvy + jy] = __dmul_rn(cyj, cyj);  // c_y^2 after the centres
   const double c2 = __dadd_rn(__dmul_rn(cxj, cxj), __dmul_rn(cyj, cyj));
   cxy[j] = make_double2(cxj, cyj);
   const int sgx = cxj > 0.0 ? 1 : (cxj < 0.0 ? -1 : 0);
@@ -33,6 +33,19 @@ __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32
     const double ay = fabs(cyj) * P.dt / P.dy;
     coef[j] = make_double4_32a(1.0 - ax - ay, ax, ay, c2);
     shift[j] = 0;
+    // the weights as integers over 2^63; where rounding would make a sum of
+    // two exceed one (Courant number 1), the x weight gives way
+    const double one = 9223372036854775808.0;  // 2^63
+    const double cy_top = fmax(fabs(centre(P.vy_min, 0, P.dcy)), fabs(centre(P.vy_min, P.nvy - 1, P.dcy)));
+    const uint64_t wy_top = (uint64_t)(cy_top * P.dt / P.dy * one), rest = ((uint64_t)1 << 63) - wy_top;
+    const uint64_t w = (uint64_t)(ax * one);
+    if (jy == 0) wx[jx] = w < rest ? w : rest;
+    if (jx == 0) wy[jy] = (uint64_t)(ay * one) | (cyj < 0.0 ? (uint64_t)1 << 63 : 0);
+    // f~ / sx = f_upx + ratio.x f + ratio.y f_upy; where c_x = 0 the upwind
+    // value is f itself, whose weight a0 is split
+    const double s = ax > 0.0 ? ax : 0.5 * (1.0 - cy_top * P.dt / P.dy);
+    if (jy == 0) sx[jx] = s;
+    ratio[j] = make_double2((1.0 - ax - ay - (ax > 0.0 ? 0.0 : s)) / s, ay / s);
   } else {
     // Eq. (exact) shift by [C], then Eq. (upwind) with the remainder r
     const double C = cxj * P.dt / P.dx;
@@ -76,9 +89,9 @@ __global__ void __launch_bounds__(256) emitted_kernel(const Params P, const doub
 }
 
 cudaError_t launch_build_tables(const Params& P, double* cx, double* cy, double4_32a* coef, int* shift,
-                                double2* cxy, int* vinfo, double2* ghost, double* emitted,
-                                cudaStream_t stream) {
-  tables_kernel<<<(P.nv + 255) / 256, 256, 0, stream>>>(P, cx, cy, coef, shift, cxy, vinfo, ghost);
+                                double2* cxy, int* vinfo, double2* ghost, double* emitted, uint64_t* wx,
+                                uint64_t* wy, double* sx, double2* ratio, cudaStream_t stream) {
+  tables_kernel<<<(P.nv + 255) / 256, 256, 0, stream>>>(P, cx, cy, coef, shift, cxy, vinfo, ghost, wx, wy, sx, ratio);
   emitted_kernel<<<1, 256, 0, stream>>>(P, cx, cy, ghost, emitted);
   return cudaGetLastError();
 }

@@ -32,6 +32,8 @@ struct Params {
   int dim, nx, ny, nvx, nvy, nv;
   int tile;  // spatial cells per CTA of the step kernel (1, 2, 4 or 8)
   int mgl;   // reduced precisions: groups of 4 velocities per lane (2, 4 or 6)
+  int lane_bits;  // FP64 2D: log2 of the lanes per velocity row of the fixed-point step
+                  // (step_f64_plan); 0: FP64 loop
   int conservative, relax_exact;
   int bc_kind[kFaces];
   double dt, dx, dy, dcx, dcy, dv;
@@ -40,11 +42,28 @@ struct Params {
   double bc_state[kFaces][4];  // n, ux, uy, theta
 };
 
+// Numbers of the velocity grid that the fixed-point step uses (2D FP64).
+struct VelocityGrid {
+  double half_x, half_y, inv_half_x, inv_half_y;  // half velocity steps and their reciprocals
+  double mid_x, mid_y, dv_pi;                     // box centres, dv / pi
+};
+inline VelocityGrid velocity_grid(const Params& P) {
+  VelocityGrid g;
+  g.half_x = 0.5 * P.dcx;
+  g.half_y = 0.5 * P.dcy;
+  g.inv_half_x = 1.0 / g.half_x;
+  g.inv_half_y = 1.0 / g.half_y;
+  g.mid_x = P.vx_min + P.nvx * g.half_x;
+  g.mid_y = P.vy_min + P.nvy * g.half_y;
+  g.dv_pi = P.dv / 3.14159265358979323846;
+  return g;
+}
+
 // Per-velocity tables built once on the device (build_tables).
 struct Tables {
+  VelocityGrid grid;
   const double* cx;       // [nvx] velocity-cell centres
   const double* cy;       // [nvy] (dim 1: one entry, 0)
-  const double* cy2;      // [nvy] c_y^2 (stored right after cy)
   const double4_32a* coef;    // [nv] (a0, ax, ay, |c|^2): streaming weights, 2D
                           //      (w_near, w_far, 0, c_x^2): 1D
   const int* shift;       // [nv] 1D integer Courant shift [C] (0 in 2D)
@@ -53,6 +72,10 @@ struct Tables {
   const double2* ghost;   // [kFaces][nv] inflow Maxwellian, or the unit-density
                           //   wall Maxwellian for diffuse faces
   const double* emitted;  // [kFaces] sum_{c_n>0} c_n G_W(n=1) dv (diffuse)
+  const uint64_t* wx;     // [nvx] 2D streaming weight |c_x| dt / dx as an integer over 2^63
+  const uint64_t* wy;     // [nvy] |c_y| dt / dy likewise, top bit set for c_y < 0; wx + wy <= 2^63
+  const double* sx;       // [nvx] 2D scale of a column: |c_x| dt / dx (c_x = 0: a value below its a0)
+  const double2* ratio;   // [nv] 2D (a0 / sx, ay / sx), for c_x = 0 (a0 / sx - 1, ay / sx)
 };
 
 // FP32 tables of the reduced-precision step (bgk_mixed.cu).
@@ -80,8 +103,10 @@ struct MixedTables {
 cudaError_t launch_step_f64(const Params& P, const Tables& T, const double2* fin, double2* fout,
                             double4_32a* mom, int* err, cudaStream_t stream, double4_32a* par = nullptr);
 cudaError_t launch_build_tables(const Params& P, double* cx, double* cy, double4_32a* coef, int* shift,
-                                double2* cxy, int* vinfo, double2* ghost, double* emitted,
-                                cudaStream_t stream);
+                                double2* cxy, int* vinfo, double2* ghost, double* emitted, uint64_t* wx,
+                                uint64_t* wy, double* sx, double2* ratio, cudaStream_t stream);
+// Fills P.lane_bits (2D FP64) from the grid and the Courant number.
+void step_f64_plan(Params& P, double max_courant);
 size_t step_f64_smem_bytes(const Params& P, int tile);
 cudaError_t prepare_step_f64(const Params& P);
 cudaError_t launch_init_step(const Params& P, double2* f, double x_split, const double left[4],

@@ -1,8 +1,8 @@
 // bgk_step.cu - the fused FP64 BGK phase-space step.
 //
-// A CTA owns G spatial cells, one warp per cell; lanes stride over the
-// velocity index v = jy*nvx + jx with 16-byte (g, h) pairs.  Per step:
-//   phase 1 (each warp, its cell)
+// A CTA owns G spatial cells; the velocities are v = jy*nvx + jx with 16-byte
+// (g, h) pairs.  Per step:
+//   phase 1 (each warp, its cell or its rows of one)
 //     A0  diffuse-wall densities n_W of the faces the cell touches, from the
 //         cell's own f^n (zero net mass flux, below Eq. bc_cavity);
 //     A1  streaming: f~ = a0 f + ax f_(upwind x) + ay f_(upwind y) (2D
@@ -10,19 +10,33 @@
 //         (1D, Eq. upwind after the integer shift of Eq. exact); upwind
 //         neighbours come from L2, boundary values from the ghost tables;
 //         f~ is parked in the cell's output slots until phase 3;
-//     A2  FP64 velocity sums of f~ for Eq. (macroscopic), one warp reduction;
-//   phase 2 (warp 0, the G cells in lanes; in 2D warp 1 takes the y axis of
-//            the Gaussian sums and factors)
+//     A2  velocity sums of f~ for Eq. (macroscopic);
+//   phase 2
 //     A3  moments, nu = n theta^(1-omega), relaxation weights and the
-//         effective Maxwellian parameters (one set of exponentials per cell,
-//         linearised updates), separable factors written to shared memory;
-//   phase 3 (each warp, its cell)
+//         effective Maxwellian parameters, separable factors in shared memory;
+//   phase 3 (each warp, as phase 1)
 //     A4  f^{n+1} = b f~ + a Phi (Eq. relaxation: b = e^{-nu dt}, a = 1 - b;
 //         Euler: a = nu dt, b = 1 - a), stored to HBM.
-// The FP64 pipe of sm_103 charges every warp instruction in full whatever the
-// number of active lanes, so the per-cell scalar work of phase 2 runs with
-// cells in lanes (G cells per instruction) and sign tests use integer tables.
+//
+// The FP64 pipe of sm_103 takes 64 to 76 cycles for a warp instruction,
+// whatever the number of active lanes; an integer instruction takes 1 to 5.
+// So the 2D step (step_fixed_kernel) gives half of its per-velocity work and
+// nearly all of its per-cell work to the integer pipe as fixed-point
+// arithmetic (bgk_fixed.cuh) that rounds less than the FP64 form: g streams
+// and h relaxes on the integer pipe while h streams and g relaxes on the FP64
+// pipe (2 FP64 operations per velocity and phase), the moment sums are exact
+// integers, and the Gaussians are evaluated directly; 5 FP64 operations per
+// velocity in all instead of 15 to 19.  Measured against the FP64-only form:
+// 256^2 x 48^2 4.11 -> 2.36 ms, 64^2 x 32^2 167 -> 105 us, 157 x 83 cells x 20
+// x 28 velocities 320 -> 185 us a step; error of a 20-step run against exact
+// 64-bit sums 8.8e-16 -> 2.9e-16.  What bounds it now: 300 instructions per
+// warp and velocity (46 % of the issue slots), upwind loads and the parked f~
+// that L2 does not hold (82 B of DRAM traffic per update).
+//
+// step_f64_kernel is the FP64-only form: 1D grids, and 2D grids that
+// step_f64_plan leaves to it.
 #include "bgk_device.cuh"
+#include "bgk_fixed.cuh"
 
 namespace bgk {
 
@@ -50,199 +64,395 @@ __device__ __forceinline__ double2 ghost_at(const Params& P, const Tables& T, in
 }
 
 // ---- phase 1 ---------------------------------------------------------------
-// Interior cell of a 2D grid whose velocity rows hold NM x 16 columns (NM 3
-// or 4): lane
-// 16 h + l takes the rows jy = h, h + 2, ... and in each row the columns
-// jx = l + 16 m (m < NM).  A lane's columns never change, so sum c_x g and
-// the c_x^2 part of sum |c|^2 g follow from its column sums after the loop,
-// and sum c_y g and the c_y^2 part (c_y^2 from a table) from its row sum once
-// per row: per point one FP64 add into the column sum, one into the row sum
-// (NM - 1 per row) and one for h, plus two per row: 10/3 at NM = 3 instead
-// of 5.
-template <int NM>
-__device__ __forceinline__ void stream_interior_rows(const Params& P, const Tables& T,
-                                                     const double2* __restrict__ fc, ptrdiff_t row,
-                                                     double2* __restrict__ tile, double& s0, double& sx,
-                                                     double& sy, double& se) {
-  const int lane = threadIdx.x & 31, l = lane & 15;
-  const int nv = P.nv, nvx = P.nvx;
-  int offx[NM];
-  double col[NM];
-#pragma unroll
-  for (int m = 0; m < NM; ++m) {
-    offx[m] = -vi_sx(T.vinfo[l + 16 * m]) * nv;  // upwind in x: ix - sgn c_x
-    col[m] = 0.0;
-  }
-  double sh = 0.0, syy = 0.0;
-#pragma unroll 1
-  for (int jy = lane >> 4; jy < P.nvy; jy += 2) {
-    const int j0 = jy * nvx + l;
-    const ptrdiff_t offy = -(ptrdiff_t)vi_sy(T.vinfo[j0]) * row;
-    const double cy = T.cy[jy], cy2 = T.cy2[jy];
-    double rg = 0.0;
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      const int j = j0 + 16 * m;
-      const double2 f0 = fc[j];
-      const double2 fx = fc[j + offx[m]];
-      const double2 fy = fc[j + offy];
-      const double4_32a co = T.coef[j];
-      double2 ft;
-      ft.x = fma(co.z, fy.x, fma(co.y, fx.x, co.x * f0.x));
-      ft.y = fma(co.z, fy.y, fma(co.y, fx.y, co.x * f0.y));
-      tile[j] = ft;
-      col[m] += ft.x;
-      rg = m == 0 ? ft.x : rg + ft.x;
-      sh += ft.y;
-    }
-    sy = fma(cy, rg, sy);
-    syy = fma(cy2, rg, syy);
-  }
-  double sxx = 0.0;
-#pragma unroll
-  for (int m = 0; m < NM; ++m) {
-    const double cx = T.cx[l + 16 * m];
-    s0 += col[m];
-    sx = fma(cx, col[m], sx);
-    sxx = fma(cx * cx, col[m], sxx);
-  }
-  se = sxx + syy + sh;
-}
+// What a cell's sums (kSums doubles in shared memory) hold: the four velocity
+// sums (sum g, sum c_x g, sum c_y g, sum |c|^2 g + h), or the sums over the
+// integer velocity indices k = 2 j + 1 - n of the fixed-point path:
+// (sum g, sum k_x g, sum k_x^2 g, sum k_y g, sum k_y^2 g, sum h).
+constexpr int kSums = 6;
+enum { SUMS_VELOCITY = 0, SUMS_INDEX = 1 };
 
+// The faces the warp's cell touches and n_W of its diffuse ones.
+struct CellEdge {
+  bool xlo, xhi, ylo, yhi;
+  double nw[4];
+};
+
+// A0: n_W for each diffuse face the cell touches (warp-uniform branch).
 template <int DIM>
-__device__ __forceinline__ void stream_cell(const Params& P, const Tables& T,
-                                            const double2* __restrict__ fin, int cell,
-                                            double2* __restrict__ tile, double* __restrict__ sums) {
+__device__ __forceinline__ CellEdge cell_edge(const Params& P, const Tables& T, const double2* __restrict__ fc,
+                                              int ix, int iy) {
   const int lane = threadIdx.x & 31;
-  const int nv = P.nv, nx = P.nx;
-  const int ix = cell % nx, iy = cell / nx;
-  const double2* __restrict__ fc = fin + (size_t)cell * nv;
-  const bool bxlo = ix == 0, bxhi = ix == nx - 1;
-  const bool bylo = DIM == 2 && iy == 0, byhi = DIM == 2 && iy == P.ny - 1;
-
-  // A0: n_W for each diffuse face this cell touches (warp-uniform branch)
+  CellEdge C;
+  C.xlo = ix == 0;
+  C.xhi = ix == P.nx - 1;
+  C.ylo = DIM == 2 && iy == 0;
+  C.yhi = DIM == 2 && iy == P.ny - 1;
   unsigned diff = 0;
-  if (bxlo && P.bc_kind[XLO] == BC_DIFFUSE) diff |= 1u;
-  if (bxhi && P.bc_kind[XHI] == BC_DIFFUSE) diff |= 2u;
-  if (bylo && P.bc_kind[YLO] == BC_DIFFUSE) diff |= 4u;
-  if (byhi && P.bc_kind[YHI] == BC_DIFFUSE) diff |= 8u;
-  double nw[4] = {0.0, 0.0, 0.0, 0.0};
+  if (C.xlo && P.bc_kind[XLO] == BC_DIFFUSE) diff |= 1u;
+  if (C.xhi && P.bc_kind[XHI] == BC_DIFFUSE) diff |= 2u;
+  if (C.ylo && P.bc_kind[YLO] == BC_DIFFUSE) diff |= 4u;
+  if (C.yhi && P.bc_kind[YHI] == BC_DIFFUSE) diff |= 8u;
+#pragma unroll
+  for (int f = 0; f < 4; ++f) C.nw[f] = 0.0;
   if (diff) {
     double inc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int j = lane; j < nv; j += 32) {
+    for (int j = lane; j < P.nv; j += 32) {
       const int vi = T.vinfo[j];
       const double2 cxy = T.cxy[j];
       const double g = fc[j].x;
       const int sx = vi_sx(vi), sy = vi_sy(vi);
-      if (sx < 0) inc[0] = fma(-cxy.x, g, inc[0]);
-      if (sx > 0) inc[1] = fma(cxy.x, g, inc[1]);
-      if (sy < 0) inc[2] = fma(-cxy.y, g, inc[2]);
-      if (sy > 0) inc[3] = fma(cxy.y, g, inc[3]);
+      if ((diff & 1u) && sx < 0) inc[0] = fma(-cxy.x, g, inc[0]);
+      if ((diff & 2u) && sx > 0) inc[1] = fma(cxy.x, g, inc[1]);
+      if ((diff & 4u) && sy < 0) inc[2] = fma(-cxy.y, g, inc[2]);
+      if ((diff & 8u) && sy > 0) inc[3] = fma(cxy.y, g, inc[3]);
     }
     const double w = warp_reduce4(inc[0], inc[1], inc[2], inc[3]);
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const double tot = __shfl_sync(0xffffffffu, w, 8 * f);
-      nw[f] = (diff >> f & 1u) ? tot * P.dv / T.emitted[f] : 0.0;
+      C.nw[f] = (diff >> f & 1u) ? tot * P.dv / T.emitted[f] : 0.0;
     }
   }
+  return C;
+}
 
-  double s0 = 0.0, sx = 0.0, sy = 0.0, se = 0.0;
-  if (DIM == 2) {
-    const ptrdiff_t row = (ptrdiff_t)nx * nv;
-    const bool interior = !(bxlo || bxhi || bylo || byhi);
-    if (interior && P.nvx == 48) {
-      stream_interior_rows<3>(P, T, fc, row, tile, s0, sx, sy, se);
-    } else if (interior && P.nvx == 64) {
-      stream_interior_rows<4>(P, T, fc, row, tile, s0, sx, sy, se);
-    } else if (interior && P.nvx == 32) {
-      // 32 columns: lane = jx for every j = lane + 32 k, so sum c_x g =
-      // c_x[lane] sum g is taken once after the loop (4 operations per point,
-      // as many as the row mapping needs with two columns per lane)
-#pragma unroll 4
-      for (int j = lane; j < nv; j += 32) {
-        const int vi = T.vinfo[j];
-        const double2 f0 = fc[j];
-        const double2 fx = fc[j - vi_sx(vi) * nv];
-        const double2 fy = fc[j - vi_sy(vi) * row];
-        const double4_32a co = T.coef[j];
-        const double cyj = T.cxy[j].y;
-        double2 ft;
-        ft.x = fma(co.z, fy.x, fma(co.y, fx.x, co.x * f0.x));
-        ft.y = fma(co.z, fy.y, fma(co.y, fx.y, co.x * f0.y));
-        tile[j] = ft;
-        s0 += ft.x;
-        sy = fma(cyj, ft.x, sy);
-        se = fma(co.w, ft.x, se) + ft.y;
+// Sum over the warp of eight 96-bit values per lane (recursive halving as in
+// warp_reduce8): lane L ends with value (L >> 2) & 7.
+__device__ __forceinline__ fx::i96 shfl96(fx::i96 v, int from) {
+  return {__shfl_sync(0xffffffffu, v.a0, from), __shfl_sync(0xffffffffu, v.a1, from),
+          __shfl_sync(0xffffffffu, v.a2, from)};
+}
+__device__ __forceinline__ fx::i96 xor_add96(fx::i96 keep, fx::i96 send, int mask) {
+  const fx::i96 got = {__shfl_xor_sync(0xffffffffu, send.a0, mask), __shfl_xor_sync(0xffffffffu, send.a1, mask),
+                       __shfl_xor_sync(0xffffffffu, send.a2, mask)};
+  return fx::add(keep, got);
+}
+__device__ __forceinline__ fx::i96 pick(bool c, fx::i96 x, fx::i96 y) {
+  return {c ? x.a0 : y.a0, c ? x.a1 : y.a1, c ? x.a2 : y.a2};
+}
+__device__ __forceinline__ fx::i96 warp_reduce8_96(const fx::i96 (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  fx::i96 a[4], b[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) a[k] = xor_add96(pick(b4, v[k + 4], v[k]), pick(b4, v[k], v[k + 4]), 16);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) b[k] = xor_add96(pick(b3, a[k + 2], a[k]), pick(b3, a[k], a[k + 2]), 8);
+  fx::i96 x = xor_add96(pick(b2, b[1], b[0]), pick(b2, b[0], b[1]), 4);
+  x = xor_add96(x, x, 2);
+  return xor_add96(x, x, 1);
+}
+
+// g of f~ from its own and upwind values, in fixed point; `top` keeps the
+// largest exponent seen (a sign bit counts as a large one).  `ok` turns false
+// when the values are too small, or their weighted sum is far below the
+// largest of them.
+__device__ __forceinline__ double combine_fast(double f0, double fxv, double fyv, unsigned long long w0,
+                                               unsigned long long wx, unsigned long long wy, unsigned eref,
+                                               unsigned& top, bool& ok, unsigned long long& units) {
+  const unsigned h0 = (unsigned)__double2hiint(f0), hx = (unsigned)__double2hiint(fxv),
+                 hy = (unsigned)__double2hiint(fyv);
+  const unsigned emax = max(max(h0, hx), hy) >> 20;
+  const unsigned long long r =
+      fx::combine(w0, fx::align(h0, (unsigned)__double2loint(f0), emax), wx,
+                  fx::align(hx, (unsigned)__double2loint(fxv), emax), wy,
+                  fx::align(hy, (unsigned)__double2loint(fyv), emax));
+  top = max(top, emax);
+  ok = emax >= fx::kExpMin && fx::combine_ok(r);
+  units = fx::to_units(r, emax, eref);
+  unsigned hi, lo;
+  fx::to_words(r, emax, hi, lo);
+  return __hiloint2double((int)hi, (int)lo);
+}
+
+// The same in FP64 (a call: inlined, its conversions would be scheduled ahead
+// of the branch).
+__device__ __noinline__ double combine_slow(double f0, double fxv, double fyv, unsigned long long w0,
+                                            unsigned long long wx, unsigned long long wy, unsigned eref,
+                                            unsigned long long& units) {
+  const double s = 1.0 / 9223372036854775808.0;  // 2^-63
+  const double v = fma((double)wy * s, fyv, fma((double)wx * s, fxv, (double)w0 * s * f0));
+  units = fx::double_to_units((unsigned)__double2hiint(v), (unsigned)__double2loint(v), eref);
+  return v;
+}
+
+// Own and upwind values of velocity j = (jx, jy) of a cell at the edge.
+__device__ __forceinline__ void load_point(const Params& P, const Tables& T, const double2* __restrict__ fc,
+                                           ptrdiff_t row, const CellEdge& C, int j, int jx, int jy, int sgx, int sgy,
+                                           double2& f0, double2& fxv, double2& fyv) {
+  f0 = fc[j];
+  fxv = fyv = f0;
+  if (sgx > 0) fxv = C.xlo ? ghost_at(P, T, XLO, j, jx, jy, C.nw[XLO], fc) : fc[j - P.nv];
+  else if (sgx < 0) fxv = C.xhi ? ghost_at(P, T, XHI, j, jx, jy, C.nw[XHI], fc) : fc[j + P.nv];
+  if (sgy > 0) fyv = C.ylo ? ghost_at(P, T, YLO, j, jx, jy, C.nw[YLO], fc) : fc[j - row];
+  else if (sgy < 0) fyv = C.yhi ? ghost_at(P, T, YHI, j, jx, jy, C.nw[YHI], fc) : fc[j + row];
+}
+
+// The velocities of a lane in the fixed-point kernels: 2^lane_bits lanes share
+// a row, the rows of the cell's W warps advance together, and a lane takes its
+// columns jx = l + m 2^lane_bits one after the other, each over its rows
+// jy = row0 + r step.
+template <int W>
+struct LaneMap {
+  int l, width, row0, step, rows;
+  __device__ __forceinline__ LaneMap(const Params& P, int wi) {
+    const int lane = threadIdx.x & 31, lb = P.lane_bits;
+    width = 1 << lb;
+    l = lane & (width - 1);
+    row0 = wi * (32 >> lb) + (lane >> lb);
+    step = W * (32 >> lb);
+    rows = (P.nvy + step - 1) / step;
+  }
+};
+
+// Rows ahead that a lane asks into L1: with 8 warps per sub-partition at 64
+// registers the next row's values cannot wait in registers (256^2 x 48^2:
+// 2.57 ms without, 2.36 ms with 1 to 4 rows).
+constexpr int kAhead = 2;
+__device__ __forceinline__ void prefetch_l1(const double2* p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
+// A1 + A2 of a warp's rows of a 2D cell, g on the integer pipe and h on the
+// FP64 pipe, which run side by side (measured per 256^2 x 48^2 step: both on
+// the FP64 pipe 2.64 ms, both on the integer pipe 3.18 ms, this 2.36 ms); a
+// column's weights and running sums stay in registers.
+//  g: fixed point.  The running sums of first, second and third order over a
+//     column's rows give sum g, sum j_y g and sum j_y^2 g as exact integers,
+//     and times j_x the x sums.
+//  h: parked divided by the column's scale s (= |c_x| dt / dx), so that f~/s
+//     = f_x + (a0/s) f + (ay/s) f_y takes two FMAs; summed as integers per
+//     column, the scale applied to the column's sum.
+// eg, eh: largest exponents of g and h that the sums' units are cut for.  On
+// return they are the largest exponents seen; the sums are valid when these
+// do not exceed the ones passed in and the result is true (no lane's sum ran
+// over 63 bits).
+template <int W, bool EDGE>
+__device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables& T, const double2* __restrict__ fc,
+                                                  ptrdiff_t row, const CellEdge& C, int wi,
+                                                  double2* __restrict__ tile, double* __restrict__ sums, int& eg,
+                                                  int& eh) {
+  typedef unsigned long long u64;
+  const int lane = threadIdx.x & 31, nvx = P.nvx, nvy = P.nvy;
+  const LaneMap<W> L(P, wi);
+  const int h = L.row0, rpw = L.step, rows = L.rows;
+  unsigned topg = 0, over = 0;
+  int toph = 0;
+  double hs = 0.0;
+  const fx::i96 zero = {0u, 0u, 0u};
+  fx::i96 n0 = zero, x1 = zero, x2 = zero, i1 = zero, i2 = zero;
+#pragma unroll 1
+  for (int jl = L.l; jl - L.l < nvx; jl += L.width) {
+    const bool in = jl < nvx;
+    const int jx = in ? jl : nvx - 1;  // a column past the row repeats its last one and is not counted
+    const int sgx = vi_sx(T.vinfo[jx]);
+    const int offx = EDGE ? sgx : -sgx * P.nv;  // upwind in x: ix - sgn c_x
+    const u64 wx = T.wx[jx], rest = ((u64)1 << fx::kWeightBits) - wx;
+    const double s = T.sx[jx];
+    const int shift = 1023 - (__double2hiint(s) >> 20), ehc = eh + shift;
+    u64 s1 = 0, hsum = 0;
+    fx::i96 s2 = zero, s3 = zero;
+#pragma unroll 1
+    for (int r = 0; r < rows; ++r) {
+      const int jr = h + r * rpw, jy = min(jr, nvy - 1), j = jy * nvx + jx;
+      const u64 wys = T.wy[jy], wy = wys & ~((u64)1 << 63);  // top bit: c_y < 0
+      const double2 ra = T.ratio[j];
+      double2 f0, fxv, fyv, ft;
+      if (EDGE) {
+        load_point(P, T, fc, row, C, j, jx, jy, offx, vi_sy(T.vinfo[jy * nvx]), f0, fxv, fyv);
+      } else {
+        const double2* p = fc + j;
+        const ptrdiff_t offy = (long long)wys < 0 ? row : -row;  // c_y = 0: any value, its weight is 0
+        f0 = p[0];
+        fxv = p[offx];
+        fyv = p[offy];
+        if (jr + kAhead * rpw < nvy) {
+          const double2* a = p + kAhead * rpw * nvx;
+          prefetch_l1(a);
+          prefetch_l1(a + offx);
+          prefetch_l1(a + offy);
+        }
       }
-      sx = T.cx[lane] * s0;
-    } else if (interior) {
-      // interior cell: every upwind neighbour is a cell of the grid
-#pragma unroll 4
-      for (int j = lane; j < nv; j += 32) {
-        const int vi = T.vinfo[j];
-        const double2 f0 = fc[j];
-        const double2 fx = fc[j - vi_sx(vi) * nv];
-        const double2 fy = fc[j - vi_sy(vi) * row];
-        const double4_32a co = T.coef[j];
-        const double2 cxy = T.cxy[j];
-        double2 ft;
-        ft.x = fma(co.z, fy.x, fma(co.y, fx.x, co.x * f0.x));
-        ft.y = fma(co.z, fy.y, fma(co.y, fx.y, co.x * f0.y));
+      u64 ug;
+      bool ok;
+      ft.x = combine_fast(f0.x, fxv.x, fyv.x, rest - wy, wx, wy, (unsigned)eg, topg, ok, ug);
+      ft.y = fma(ra.y, fyv.y, fma(ra.x, f0.y, fxv.y));
+      const bool valid = in && jr < nvy;
+      if (valid) {
+        const unsigned hh = (unsigned)__double2hiint(ft.y);
         tile[j] = ft;
-        s0 += ft.x;
-        sx = fma(cxy.x, ft.x, sx);
-        sy = fma(cxy.y, ft.x, sy);
-        se = fma(co.w, ft.x, se) + ft.y;
+        s1 += ok ? ug : 0;
+        hsum += fx::double_to_units(hh, (unsigned)__double2loint(ft.y), (unsigned)ehc);
+        toph = max(toph, (int)(hh >> 20) - shift);
       }
-    } else {
-      for (int j = lane; j < nv; j += 32) {
-        const int vi = T.vinfo[j];
-        const int jx = vi_jx(vi), jy = vi_jy(vi), sgx = vi_sx(vi), sgy = vi_sy(vi);
-        const double2 f0 = fc[j];
-        double2 fx = f0, fy = f0;
-        if (sgx > 0) fx = bxlo ? ghost_at(P, T, XLO, j, jx, jy, nw[XLO], fc) : fc[j - nv];
-        else if (sgx < 0) fx = bxhi ? ghost_at(P, T, XHI, j, jx, jy, nw[XHI], fc) : fc[j + nv];
-        if (sgy > 0) fy = bylo ? ghost_at(P, T, YLO, j, jx, jy, nw[YLO], fc) : fc[j - row];
-        else if (sgy < 0) fy = byhi ? ghost_at(P, T, YHI, j, jx, jy, nw[YHI], fc) : fc[j + row];
-        const double4_32a co = T.coef[j];
-        const double2 cxy = T.cxy[j];
-        double2 ft;
-        ft.x = fma(co.z, fy.x, fma(co.y, fx.x, co.x * f0.x));
-        ft.y = fma(co.z, fy.y, fma(co.y, fx.y, co.x * f0.y));
-        tile[j] = ft;
-        s0 += ft.x;
-        sx = fma(cxy.x, ft.x, sx);
-        sy = fma(cxy.y, ft.x, sy);
-        se = fma(co.w, ft.x, se) + ft.y;
+      if (valid && !ok) {  // rare: values near the smallest doubles, or fronts steeper than the weights
+        tile[j].x = combine_slow(f0.x, fxv.x, fyv.x, rest - wy, wx, wy, (unsigned)eg, ug);
+        s1 += ug;
       }
+      s2 = fx::add(s2, fx::wide(s1));
+      s3 = fx::add(s3, s2);
+      over |= (unsigned)((s1 | hsum) >> 32);  // an addend is at most 2^59: the top bit shows before a sum wraps
     }
-  } else {
-    for (int j = lane; j < nv; j += 32) {
-      const int vi = T.vinfo[j];
-      const int sgx = vi_sx(vi);
-      const int s = T.shift[j];
-      const int i1 = ix - s, i2 = ix - s - sgx;
-      double2 f1, f2;
-      if (i1 < 0) f1 = ghost_at(P, T, XLO, j, j, 0, nw[XLO], fc);
-      else if (i1 >= nx) f1 = ghost_at(P, T, XHI, j, j, 0, nw[XHI], fc);
-      else f1 = fin[(size_t)i1 * nv + j];
-      if (i2 < 0) f2 = ghost_at(P, T, XLO, j, j, 0, nw[XLO], fc);
-      else if (i2 >= nx) f2 = ghost_at(P, T, XHI, j, j, 0, nw[XHI], fc);
-      else f2 = fin[(size_t)i2 * nv + j];
+    n0 = fx::add(n0, fx::wide(s1));
+    i1 = fx::add(i1, s2);
+    i2 = fx::add(i2, s3);
+    x1 = fx::add(x1, fx::mul(fx::wide(s1), (unsigned)jx));
+    x2 = fx::add(x2, fx::mul(fx::wide(s1), (unsigned)(jx * jx)));
+    // the column's unit times its scale: s 2^(ehc - 1081)
+    hs = fma((double)hsum, __hiloint2double(__double2hiint(s) + (ehc - 1081) * (1 << 20), __double2loint(s)), hs);
+  }
+  topg = __reduce_max_sync(0xffffffffu, topg);
+  toph = __reduce_max_sync(0xffffffffu, toph);
+  const bool valid = (int)topg <= eg && toph <= eh && !__any_sync(0xffffffffu, (int)over < 0);
+  if (valid) {
+    // j_y of row r: A - rpw (rows - r); i1 = sum (rows - r) g, i2 = sum (rows - r)(rows - r + 1) / 2 g
+    const unsigned A = (unsigned)(h + rpw * rows), B = (unsigned)rpw;
+    const fx::i96 b1 = fx::mul(i1, B);
+    fx::i96 v[8] = {n0, x1, x2, fx::add(fx::mul(n0, A), fx::neg(b1)),
+                    fx::add(fx::add(fx::mul(n0, A * A), fx::neg(fx::mul(b1, 2u * A + B))), fx::mul(i2, 2u * B * B)),
+                    zero, zero, zero};
+    const fx::i96 t = warp_reduce8_96(v);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) hs += __shfl_xor_sync(0xffffffffu, hs, m);
+    // from j to k = 2 j + 1 - n: lane group q holds value q of (1, j_x, j_x^2, j_y, j_y^2) sums
+    const int q = lane >> 2, n = 1 - (q <= 2 ? nvx : nvy);
+    const fx::i96 first = shfl96(t, 0), prev = shfl96(t, max(lane - 4, 0));
+    const bool lin = q == 1 || q == 3, quad = q == 2 || q == 4;
+    const fx::i96 k = lin ? fx::add(fx::mul(t, 2u), fx::muls(first, n))
+                          : quad ? fx::add(fx::add(fx::mul(t, 4u), fx::muls(prev, 4 * n)), fx::mul(first, (unsigned)(n * n)))
+                                 : t;
+    if ((lane & 3) == 0 && q < 5) {
+      unsigned hi, lo;
+      fx::wide_to_words(k, (unsigned)eg, hi, lo);
+      sums[q] = __hiloint2double((int)hi, (int)lo);
+    }
+    if (lane == 0) sums[5] = hs;
+  }
+  eg = (int)topg;
+  eh = toph;
+  return valid;
+}
+
+// Largest exponent fields of g and h over 128 samples of the cell, spread
+// over both axes by an odd stride (nv >= 128), plus the headroom.
+__device__ __forceinline__ void sample_range(const double2* __restrict__ fc, int nv, int& eg, int& eh) {
+  const int lane = threadIdx.x & 31;
+  unsigned sg = 0, sh = 0;
+  const int stride = (nv >> 7) | 1;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int at = (4 * lane + s) * stride;  // below 2 nv
+    const double2 v = fc[at < nv ? at : at - nv];
+    sg = max(sg, (unsigned)__double2hiint(v.x));
+    sh = max(sh, (unsigned)__double2hiint(v.y));
+  }
+  eg = (int)((__reduce_max_sync(0xffffffffu, sg) >> 20) + fx::kHeadroom);
+  eh = (int)((__reduce_max_sync(0xffffffffu, sh) >> 20) + fx::kHeadroom);
+}
+
+// The same rows in FP64, for any values.
+template <int W>
+__device__ __noinline__ void stream_rows_f64(const Params& P, const Tables& T, const double2* __restrict__ fc,
+                                             ptrdiff_t row, const CellEdge& C, int wi, double2* __restrict__ tile,
+                                             double* __restrict__ sums) {
+  const LaneMap<W> L(P, wi);
+  const int lane = threadIdx.x & 31;
+  double s0 = 0.0, sx = 0.0, sy = 0.0, se = 0.0;
+  for (int jx = L.l; jx < P.nvx; jx += L.width)
+    for (int jy = L.row0; jy < P.nvy; jy += L.step) {
+      const int j = jy * P.nvx + jx, vi = T.vinfo[j];
       const double4_32a co = T.coef[j];
-      const double cx = T.cxy[j].x;
-      double2 ft;
-      ft.x = fma(co.y, f2.x, co.x * f1.x);
-      ft.y = fma(co.y, f2.y, co.x * f1.y);
+      const double2 cxy = T.cxy[j];
+      double2 f0, fx, fy, ft;
+      load_point(P, T, fc, row, C, j, jx, jy, vi_sx(vi), vi_sy(vi), f0, fx, fy);
+      ft.x = fma(co.z, fy.x, fma(co.y, fx.x, co.x * f0.x));
+      ft.y = fma(co.z, fy.y, fma(co.y, fx.y, co.x * f0.y));
       tile[j] = ft;
       s0 += ft.x;
-      sx = fma(cx, ft.x, sx);
+      sx = fma(cxy.x, ft.x, sx);
+      sy = fma(cxy.y, ft.x, sy);
       se = fma(co.w, ft.x, se) + ft.y;
     }
+  const double w = warp_reduce4(s0, sx, sy, se);
+  if ((lane & 7) == 0) sums[lane >> 3] = w;
+}
+
+// A0 to A2 of a warp's rows; returns the kind of its sums.
+template <int W>
+__device__ __forceinline__ int stream_rows(const Params& P, const Tables& T, const double2* __restrict__ fin, int cell,
+                                           int wi, double2* __restrict__ tile, double* __restrict__ sums) {
+  const int ix = cell % P.nx, iy = cell / P.nx;
+  const double2* __restrict__ fc = fin + (size_t)cell * P.nv;
+  const ptrdiff_t row = (ptrdiff_t)P.nx * P.nv;
+  const CellEdge C = cell_edge<2>(P, T, fc, ix, iy);
+  int eg, eh;
+  sample_range(fc, P.nv, eg, eh);
+  const bool edge = C.xlo || C.xhi || C.ylo || C.yhi;
+  // a second pass takes the largest exponents of the first as its range
+  for (int pass = 0; pass < 2; ++pass) {
+    if (min(eg, eh) < (int)fx::kExpMin || max(eg, eh) > (int)fx::kExpMax) break;
+    if (edge ? stream_rows_fixed<W, true>(P, T, fc, row, C, wi, tile, sums, eg, eh)
+             : stream_rows_fixed<W, false>(P, T, fc, row, C, wi, tile, sums, eg, eh))
+      return SUMS_INDEX;
+  }
+  stream_rows_f64<W>(P, T, fc, row, C, wi, tile, sums);
+  return SUMS_VELOCITY;
+}
+
+// A1 + A2 in FP64 for any grid and any values.
+template <int DIM>
+__device__ __forceinline__ void stream_cell_f64(const Params& P, const Tables& T, const double2* __restrict__ fin,
+                                                const double2* __restrict__ fc, int ix, ptrdiff_t row,
+                                                const CellEdge& C, double2* __restrict__ tile,
+                                                double* __restrict__ sums) {
+  const int lane = threadIdx.x & 31;
+  const int nv = P.nv, nx = P.nx;
+  double s0 = 0.0, sx = 0.0, sy = 0.0, se = 0.0;
+  for (int j = lane; j < nv; j += 32) {
+    const int vi = T.vinfo[j];
+    const int sgx = vi_sx(vi);
+    const double4_32a co = T.coef[j];
+    const double2 cxy = T.cxy[j];
+    double2 ft;
+    if (DIM == 2) {
+      const int jx = vi_jx(vi), jy = vi_jy(vi), sgy = vi_sy(vi);
+      const double2 f0 = fc[j];
+      double2 fx = f0, fy = f0;
+      if (sgx > 0) fx = C.xlo ? ghost_at(P, T, XLO, j, jx, jy, C.nw[XLO], fc) : fc[j - nv];
+      else if (sgx < 0) fx = C.xhi ? ghost_at(P, T, XHI, j, jx, jy, C.nw[XHI], fc) : fc[j + nv];
+      if (sgy > 0) fy = C.ylo ? ghost_at(P, T, YLO, j, jx, jy, C.nw[YLO], fc) : fc[j - row];
+      else if (sgy < 0) fy = C.yhi ? ghost_at(P, T, YHI, j, jx, jy, C.nw[YHI], fc) : fc[j + row];
+      ft.x = fma(co.z, fy.x, fma(co.y, fx.x, co.x * f0.x));
+      ft.y = fma(co.z, fy.y, fma(co.y, fx.y, co.x * f0.y));
+      sy = fma(cxy.y, ft.x, sy);
+    } else {
+      const int i1 = ix - T.shift[j], i2 = i1 - sgx;
+      double2 f1, f2;
+      if (i1 < 0) f1 = ghost_at(P, T, XLO, j, j, 0, C.nw[XLO], fc);
+      else if (i1 >= nx) f1 = ghost_at(P, T, XHI, j, j, 0, C.nw[XHI], fc);
+      else f1 = fin[(size_t)i1 * nv + j];
+      if (i2 < 0) f2 = ghost_at(P, T, XLO, j, j, 0, C.nw[XLO], fc);
+      else if (i2 >= nx) f2 = ghost_at(P, T, XHI, j, j, 0, C.nw[XHI], fc);
+      else f2 = fin[(size_t)i2 * nv + j];
+      ft.x = fma(co.y, f2.x, co.x * f1.x);
+      ft.y = fma(co.y, f2.y, co.x * f1.y);
+    }
+    tile[j] = ft;
+    s0 += ft.x;
+    sx = fma(cxy.x, ft.x, sx);
+    se = fma(co.w, ft.x, se) + ft.y;
   }
   const double w = warp_reduce4(s0, sx, sy, se);
   if ((lane & 7) == 0) sums[lane >> 3] = w;
+}
+
+template <int DIM>
+__device__ __forceinline__ void stream_cell(const Params& P, const Tables& T, const double2* __restrict__ fin,
+                                            int cell, double2* __restrict__ tile, double* __restrict__ sums) {
+  const int ix = cell % P.nx, iy = cell / P.nx;
+  const double2* __restrict__ fc = fin + (size_t)cell * P.nv;
+  const CellEdge C = cell_edge<DIM>(P, T, fc, ix, iy);
+  stream_cell_f64<DIM>(P, T, fin, fc, ix, (ptrdiff_t)P.nx * P.nv, C, tile, sums);
 }
 
 // ---- phase 2 ---------------------------------------------------------------
@@ -353,8 +563,41 @@ __device__ __forceinline__ void axis_sums(const double* __restrict__ c, int n, d
   M[4] = m4;
 }
 
-template <int DIM, int G>
-__device__ void maxwellian_cells(const Params& P, const Tables& T, int cell0, const double (*sums)[4],
+// The cell's moments from the sums of its W warps, of either kind; k -> c is
+// affine on the uniform grid: c = mid + half k.
+template <int W>
+__device__ __forceinline__ void cell_moments(const Params& P, const VelocityGrid& V, const double (*sums)[kSums],
+                                             const int* kind, double q[4]) {
+  double t[4] = {0.0, 0.0, 0.0, 0.0}, u[kSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  bool index = false;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    if (kind[w] == SUMS_VELOCITY) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) t[k] += sums[w][k];
+    } else {
+      index = true;
+#pragma unroll
+      for (int k = 0; k < kSums; ++k) u[k] += sums[w][k];
+    }
+  }
+  if (index) {
+    const double tx = V.half_x * u[1], ty = V.half_y * u[3];
+    const double sx = fma(V.mid_x, u[0], tx), sy = fma(V.mid_y, u[0], ty);
+    // sum c^2 g = mid (sum c g + half sum k g) + half^2 sum k^2 g per axis
+    const double ex = fma(V.half_x * V.half_x, u[2], V.mid_x * (sx + tx));
+    const double ey = fma(V.half_y * V.half_y, u[4], V.mid_y * (sy + ty));
+    t[0] += u[0];
+    t[1] += sx;
+    t[2] += sy;
+    t[3] += (ex + ey) + u[5];
+  }
+  moments_from_sums(t[0], t[1], t[2], t[3], P.dv, q);
+}
+
+template <int DIM, int G, int W = 1>
+__device__ void maxwellian_cells(const Params& P, const Tables& T, int cell0, const double (*sums)[kSums],
+                                 const int* kind,
                                  double* __restrict__ phx, double* __restrict__ phy, double* sb,
                                  double* sk, int* sok, double4_32a* __restrict__ mom,
                                  double4_32a* __restrict__ par, int* __restrict__ err) {
@@ -363,7 +606,7 @@ __device__ void maxwellian_cells(const Params& P, const Tables& T, int cell0, co
   const int cell = cell0 + c;
   const bool live = cell < P.nx * P.ny;
   double qm[4] = {1.0, 0.0, 0.0, 1.0};  // moments of f~ (Eq. macroscopic)
-  if (live) moments_from_sums(sums[c][0], sums[c][1], sums[c][2], sums[c][3], P.dv, qm);
+  if (live) cell_moments<W>(P, T.grid, sums + c * W, kind + c * W, qm);
   bool ok = live && moments_ok(qm);
   // a failed cell keeps its lanes busy on a harmless stand-in state
   const double q[4] = {ok ? qm[0] : 1.0, ok ? qm[1] : 0.0, ok ? qm[2] : 0.0, ok ? qm[3] : 1.0};
@@ -441,7 +684,8 @@ struct SolveXchg {
 __device__ __forceinline__ void pair_barrier() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
 
 template <int G>
-__device__ void maxwellian_cells_2w(const Params& P, const Tables& T, int cell0, const double (*sums)[4],
+__device__ void maxwellian_cells_2w(const Params& P, const Tables& T, int cell0, const double (*sums)[kSums],
+                                    const int* kind,
                                     double* __restrict__ phx, double* __restrict__ phy, double* sb, double* sk,
                                     int* sok, double4_32a* __restrict__ mom, double4_32a* __restrict__ par,
                                     int* __restrict__ err, SolveXchg<G>& X) {
@@ -473,7 +717,7 @@ __device__ void maxwellian_cells_2w(const Params& P, const Tables& T, int cell0,
   const int cell = cell0 + c;
   const bool live = cell < P.nx * P.ny;
   double qm[4] = {1.0, 0.0, 0.0, 1.0};  // moments of f~ (Eq. macroscopic)
-  if (live) moments_from_sums(sums[c][0], sums[c][1], sums[c][2], sums[c][3], P.dv, qm);
+  if (live) cell_moments<1>(P, T.grid, sums + c, kind + c, qm);
   bool ok = live && moments_ok(qm);
   const double q[4] = {ok ? qm[0] : 1.0, ok ? qm[1] : 0.0, ok ? qm[2] : 0.0, ok ? qm[3] : 1.0};
   double* px = phx + c * P.nvx;
@@ -536,93 +780,485 @@ __device__ void maxwellian_cells_2w(const Params& P, const Tables& T, int cell0,
   }
 }
 
+// Phase 2 of the fixed-point kernels: the Gaussians of a cell on its own warp
+// and on the integer pipe, the scalar solve with cells in lanes on one warp.
+// A rounding-free index form of the central sums: with integers k' = k - k0,
+// k0 next to the mean, c - u = half k' + delta.
+__device__ const unsigned long long kExp2[32] = BGK_EXP2_TABLE;
+
+constexpr int kMaxIndexShift = 1024;  // |k0|: keeps sum k'^2 e within 95 bits
+
+template <int G>
+struct CellSolve {
+  // base point of the Gaussians per axis, (c_k - u) sqrt(log2 e / theta) = a k - c in units of 2^-58
+  long long a[G][2], c[G][2];
+  int k0[G][2];
+  double sums[G][2][3];  // sum e, sum k' e, sum k'^2 e
+  double ap[G];          // a n / (pi theta)
+  int need[G];
+  int go;  // 1: sums wanted, 0: factors wanted, -1: a cell is out of range (FP64 path)
+};
+
+// 1/x and 1/sqrt(x) of positive normal x by one third-order (Householder)
+// step from the FP32 approximation of relative error e0 < 2^-21: three and
+// five FP64 operations, error e0^3 beside the roundings (an FP64 division or
+// square root costs ten or more).
+__device__ __forceinline__ float to_float_bits(double x) {  // truncated, exponent kept in range by the caller
+  return __uint_as_float((((unsigned)__double2hiint(x) - 0x38000000u) << 3) | ((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double to_double_bits(float y) {
+  const unsigned u = __float_as_uint(y);
+  return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
+__device__ __forceinline__ double rcp3(double x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_bits(x)));
+  const double d = to_double_bits(y), e = fma(-x, d, 1.0);
+  return fma(d, fma(e, e, e), d);
+}
+__device__ __forceinline__ double rsqrt3(double x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_bits(x)));
+  const double d = to_double_bits(y), e = fma(-x * d, d, 1.0);
+  return fma(d, e * fma(0.375, e, 0.5), d);
+}
+// Whether x is positive, finite and well inside the FP32 exponent range.
+__device__ __forceinline__ bool in_range(double x) {
+  const unsigned h = (unsigned)__double2hiint(x);
+  return h - 0x3a000000u < 0x0c000000u;  // 2^-95 to 2^97
+}
+__device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// A cell's solve: moments q, parameters p (the base point of the Gaussians),
+// ith = 1 / theta, isq = 1 / sqrt(theta) of p.
+struct FixedSolve {
+  double q[4], p[4];
+  double ith, isq;
+  double iq0, iq3, ivs;  // 1 / n, 1 / theta, 1 / sqrt(theta) of q
+  int it;
+  bool conv, fail;
+};
+
+// Publishes the base point of a cell; false when it or a velocity lies too
+// far out for the fixed-point Gaussian.
+template <int G>
+__device__ __forceinline__ bool publish_base(const Params& P, const VelocityGrid& V, const FixedSolve& E, int c, CellSolve<G>& X) {
+  const double gamma = E.isq * 1.2011224087864498;  // sqrt(log2 e)
+  bool fit = true;
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int n = x == 0 ? P.nvx : P.nvy;
+    const double half = x == 0 ? V.half_x : V.half_y;
+    const double off = E.p[1 + x] - (x == 0 ? V.mid_x : V.mid_y);
+    const double a = half * gamma, s = off * gamma;
+    const double r = fma(off, x == 0 ? V.inv_half_x : V.inv_half_y, 6755399441055744.0);  // 1.5 2^52: rounds to an integer
+    const int k0 = __double2loint(r);
+    // |s| + a n < 31.9, |off| below 1024 half steps (words: the exponent decides)
+    const double reach = fma(a, (double)n, fabs(s));
+    fit = fit && abs_hi(reach) < 0x403fe666u && abs_hi(r) == 0x43380000u - (k0 < 0 ? 1u : 0u) &&
+          (unsigned)(k0 + kMaxIndexShift) < 2u * kMaxIndexShift;
+    X.a[c][x] = fx::to_fix58((unsigned)__double2hiint(a), (unsigned)__double2loint(a));
+    X.c[c][x] = fx::to_fix58((unsigned)__double2hiint(s), (unsigned)__double2loint(s));
+    X.k0[c][x] = k0;
+  }
+  return fit;
+}
+
+// nu = n theta^(1-omega) and the relaxation weights, exp(-nu dt) on the
+// integer pipe where its argument allows.
+__device__ __forceinline__ void relax_weights_fixed(const Params& P, const FixedSolve& E, double& a, double& b) {
+  const double nu = E.q[0] * (P.omega == 0.5 ? E.q[3] * E.ivs : pow(E.q[3], 1.0 - P.omega));
+  const double x = nu * P.dt;
+  if (!P.relax_exact) {
+    a = x;
+    b = 1.0 - a;
+    return;
+  }
+  const double t = x * 1.4426950408889634;  // log2 e
+  if (abs_hi(t) < 0x40400000u) {             // below 32
+    const unsigned long long f = (unsigned long long)fx::to_fix58((unsigned)__double2hiint(t), (unsigned)__double2loint(t));
+    unsigned hi, lo;
+    fx::gauss_words(fx::exp2_neg(f << 6, (const fx::u64*)kExp2), (unsigned)(f >> 58), hi, lo);
+    b = __hiloint2double((int)hi, (int)lo);
+  } else {
+    b = exp(-x);
+  }
+  a = 1.0 - b;
+}
+
+// One update p <- p + (q - D(p)) (A3) from the central sums M_m of both axes
+// at p, with the stopping rules of eff_iterate.
+__device__ __forceinline__ void eff_update(const VelocityGrid& V, const double (&Mx)[3], const double (&My)[3],
+                                           FixedSolve& E) {
+  ++E.it;
+  const double rxy = rcp3(Mx[0] * My[0]);
+  const double rx = My[0] * rxy, ry = Mx[0] * rxy;
+  const double mux = Mx[1] * rx, muy = My[1] * ry;
+  double d[4];
+  d[0] = (E.p[0] * E.ith) * V.dv_pi * (Mx[0] * My[0]);
+  d[1] = E.p[1] + mux;
+  d[2] = E.p[2] + muy;
+  const double var = fma(Mx[2], rx, -mux * mux) + fma(My[2], ry, -muy * muy);
+  d[3] = (2.0 / 3.0) * fma(0.5, E.p[3], var);
+  unsigned r = 0;  // high word of the largest scaled update
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double delta = E.q[k] - d[k];
+    E.p[k] += delta;
+    r = max(r, abs_hi(delta * (k == 0 ? E.iq0 : k == 3 ? E.iq3 : E.ivs)));
+  }
+  // the high words of kEffTol = 1e-13, sqrt(kEffTol / 100) = 3.16e-8 and kEffFail = 1e-9
+  if (!in_range(E.p[0]) || !in_range(E.p[3]) || r >= 0x7ff00000u) E.fail = true;
+  else if (r < 0x3d3c25c2u || (E.it == 1 && r < 0x3e60fa33u)) E.conv = true;
+  else if (E.it >= kEffMaxIt) (r < 0x3e112e0bu ? E.conv : E.fail) = true;
+  E.isq = rsqrt3(E.p[3]);
+  E.ith = E.isq * E.isq;
+}
+
+// Which axis of its cell a warp works on, with which lane of how many: half a
+// warp per axis when the cell has one warp, a warp per axis when it has more
+// (the others none, x = 2).
+template <int W>
+struct AxisMap {
+  static constexpr int kLanes = W == 1 ? 16 : 32;
+  int x, i;
+  __device__ __forceinline__ AxisMap(int wi) {
+    const int lane = threadIdx.x & 31;
+    x = W == 1 ? lane >> 4 : min(wi, 2);
+    i = lane & (kLanes - 1);
+  }
+};
+
+// Sums of cell c's Gaussians at the base point, along the warp's axis.
+template <int G, int W>
+__device__ __forceinline__ void gauss_sums(const Params& P, int c, int wi, CellSolve<G>& X) {
+  const AxisMap<W> A(wi);
+  if (W > 2 && A.x > 1) return;  // the whole warp
+  const int n = A.x == 0 ? P.nvx : P.nvy, k0 = X.k0[c][A.x];
+  const long long a = X.a[c][A.x], off = X.c[c][A.x];
+  fx::i96 s[3] = {{0u, 0u, 0u}, {0u, 0u, 0u}, {0u, 0u, 0u}};
+#pragma unroll 1
+  for (int j = A.i; j < n; j += A.kLanes) {
+    const int k = 2 * j + 1 - n, kk = k - k0;
+    unsigned q2;
+    const unsigned long long q = fx::gauss(a * k - off, (const fx::u64*)kExp2, q2);
+    const fx::i96 e = fx::wide(q2 < 62u ? q >> (q2 + 1u) : 0);  // units of 2^-62
+    s[0] = fx::add(s[0], e);
+    s[1] = fx::add(s[1], fx::muls(e, kk));
+    s[2] = fx::add(s[2], fx::mul(e, (unsigned)(kk * kk)));
+  }
+#pragma unroll
+  for (int m = A.kLanes / 2; m > 0; m >>= 1)
+#pragma unroll
+    for (int p = 0; p < 3; ++p) s[p] = xor_add96(s[p], s[p], m);
+  if (A.i < 3) {
+    unsigned hi, lo;
+    fx::wide_to_words(A.i == 0 ? s[0] : A.i == 1 ? s[1] : s[2], 1081u - 62u, hi, lo);
+    X.sums[c][A.x][A.i] = __hiloint2double((int)hi, (int)lo);
+  }
+}
+
+// Cell c's a Phi factors at the final parameters, along the warp's axis.
+template <int G, int W>
+__device__ __forceinline__ void gauss_factors(const Params& P, int c, int wi, const CellSolve<G>& X,
+                                              double* __restrict__ px, double* __restrict__ py) {
+  const AxisMap<W> A(wi);
+  if (W > 2 && A.x > 1) return;
+  const int n = A.x == 0 ? P.nvx : P.nvy;
+  const long long a = X.a[c][A.x], off = X.c[c][A.x];
+  const double scale = X.ap[c];
+  double* out = A.x == 0 ? px : py;
+#pragma unroll 1
+  for (int j = A.i; j < n; j += A.kLanes) {
+    unsigned q2, hi, lo;
+    const unsigned long long q = fx::gauss(a * (2 * j + 1 - n) - off, (const fx::u64*)kExp2, q2);
+    fx::gauss_words(q, q2, hi, lo);
+    const double e = __hiloint2double((int)hi, (int)lo);
+    out[j] = A.x == 0 ? scale * e : e;
+  }
+}
+
+// All threads of the CTA.  Leaves factors, weights and ok of every cell; false
+// when they come from maxwellian_cells.
+template <int G, int W>
+__device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Tables& T, int cell0,
+                                                       const double (*sums)[kSums], const int* kind,
+                                                       double* __restrict__ phx, double* __restrict__ phy, double* sb,
+                                                       double* sk, int* sok, double4_32a* __restrict__ mom,
+                                                       double4_32a* __restrict__ par, int* __restrict__ err,
+                                                       CellSolve<G>& X) {
+  const VelocityGrid& V = T.grid;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mine = warp / W, wi = warp % W;
+  // the solving warp varies from CTA to CTA, so that the FP64 work of the
+  // solves is spread over the SM's four sub-partitions
+  const int solver = (int)((blockIdx.x * 0x9E3779B1u) >> 16) % (G * W);
+  const bool solving = warp == solver;
+  const int c = lane % G, cell = cell0 + c;
+  const bool live = cell < P.nx * P.ny, wr = lane < G;
+  double qm[4] = {1.0, 0.0, 0.0, 1.0}, a = 0.0, b = 0.0;
+  bool ok = false;
+  FixedSolve E;
+  if (solving) {
+    if (live) cell_moments<W>(P, T.grid, sums + c * W, kind + c * W, qm);
+    ok = live && moments_ok(qm);
+    bool fit = !ok || (in_range(qm[0]) && in_range(qm[3]));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) E.q[k] = E.p[k] = ok && fit ? qm[k] : (k == 0 || k == 3) ? 1.0 : 0.0;
+    E.ivs = E.isq = rsqrt3(E.q[3]);
+    E.iq3 = E.ith = E.isq * E.isq;
+    E.iq0 = rcp3(E.q[0]);
+    E.it = 0;
+    E.conv = P.conservative == 0 || !ok;
+    E.fail = false;
+    if (wr) {
+      const bool reach = publish_base(P, V, E, c, X);
+      fit = fit && (reach || !ok);
+      X.need[c] = !E.conv;
+    }
+    const bool all = __all_sync(0xffffffffu, fit);
+    const bool any = __any_sync(0xffffffffu, wr && !E.conv);
+    if (lane == 0) X.go = !all ? -1 : any ? 1 : 0;
+  }
+  __syncthreads();
+  bool weighted = false;
+  while (X.go > 0) {
+    if (solving && !weighted) {
+      relax_weights_fixed(P, E, a, b);
+      weighted = true;
+    }
+    if (X.need[mine]) gauss_sums<G, W>(P, mine, wi, X);
+    __syncthreads();
+    if (solving) {
+      bool fit = true;
+      if (!E.conv && !E.fail) {
+        double M[2][3];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const double half = x == 0 ? V.half_x : V.half_y;
+          const double d = fma((double)X.k0[c][x], half, x == 0 ? V.mid_x : V.mid_y) - E.p[1 + x];
+          const double m0 = X.sums[c][x][0], t1 = half * X.sums[c][x][1];
+          M[x][0] = m0;
+          M[x][1] = fma(d, m0, t1);
+          M[x][2] = fma(half * half, X.sums[c][x][2], d * (t1 + M[x][1]));
+        }
+        eff_update(V, M[0], M[1], E);
+        if (wr) fit = publish_base(P, V, E, c, X) || E.fail;
+      }
+      if (wr) X.need[c] = !E.conv && !E.fail;
+      const bool all = __all_sync(0xffffffffu, fit);
+      const bool any = __any_sync(0xffffffffu, wr && !E.conv && !E.fail);
+      if (lane == 0) X.go = !all ? -1 : any ? 1 : 0;
+    }
+    __syncthreads();
+  }
+  if (X.go < 0) {
+    if (warp == 0) maxwellian_cells<2, G, W>(P, T, cell0, sums, kind, phx, phy, sb, sk, sok, mom, par, err);
+    __syncthreads();
+    return false;
+  }
+  if (solving) {
+    if (E.fail) ok = false;
+    if (!weighted) relax_weights_fixed(P, E, a, b);
+    if (wr) {
+      X.ap[c] = a * (E.p[0] * E.ith) * 0.31830988618379067;  // 1 / pi
+      sb[c] = b;
+      sk[c] = 0.5 * E.p[3];
+      sok[c] = ok ? 1 : 0;
+      if (live) {
+        mom[cell] = make_double4_32a(qm[0], qm[1], qm[2], qm[3]);
+        if (par) par[cell] = make_double4_32a(E.p[0], E.p[1], E.p[2], E.p[3]);
+        if (!ok) atomicOr(err, E.fail ? ERR_EFFECTIVE : ERR_MOMENT);
+      }
+    }
+  }
+  __syncthreads();
+  if (sok[mine]) gauss_factors<G, W>(P, mine, wi, X, phx + mine * P.nvx, phy + mine * P.nvy);
+  if (W == 1) __syncwarp();
+  else __syncthreads();
+  return true;
+}
+
 // ---- phase 3 ---------------------------------------------------------------
 // A4 for the warp's cell: f^{n+1} = b f~ + a Phi from the f~ parked in the
 // cell's output slots, a Phi_g = px[jx] py[jy], a Phi_h = kappa a Phi_g.
 template <int DIM>
-__device__ __forceinline__ void relax_cell(const Params& P, const Tables& T, double2* __restrict__ fout, int cell,
+__device__ __forceinline__ void relax_cell(const Params& P, const Tables& T, double2* __restrict__ fo,
                                            const double* __restrict__ px, const double* __restrict__ py, double b,
-                                           double kappa, bool ok) {
+                                           double kappa) {
   const int lane = threadIdx.x & 31;
-  const int nv = P.nv;
-  double2* __restrict__ fo = fout + (size_t)cell * nv;
-  const double2* tile = fo;
-  if (DIM == 2 && ok && (P.nvx == 48 || P.nvx == 64)) {
-    // rows jy = h, h + 2, ..., columns jx = l + 16 m of lane 16 h + l, as
-    // in stream_interior_rows: a Phi = px[jx] py[jy] from shared memory
-    const int l = lane & 15;
-    for (int jy = lane >> 4; jy < P.nvy; jy += 2) {
-      const double pyv = py[jy];
 #pragma unroll 4
-      for (int jx = l; jx < P.nvx; jx += 16) {
-        const int j = jy * P.nvx + jx;
-        const double2 ft = tile[j];
-        const double aphi = px[jx] * pyv;
-        fo[j] = make_double2(fma(b, ft.x, aphi), fma(b, ft.y, kappa * aphi));
+  for (int j = lane; j < P.nv; j += 32) {
+    const double2 ft = fo[j];
+    double aphi;
+    if (DIM == 2) {
+      const int vi = T.vinfo[j];
+      aphi = px[vi_jx(vi)] * py[vi_jy(vi)];
+    } else {
+      aphi = px[j];
+    }
+    fo[j] = make_double2(fma(b, ft.x, aphi), fma(b, ft.y, kappa * aphi));
+  }
+}
+
+// h of one value in FP64 (a call, see combine_slow).
+__device__ __noinline__ double relax_slow(double h, double aphi, double b, double kappa) {
+  return fma(b, h, kappa * aphi);
+}
+
+// The same for a cell streamed by stream_rows_fixed (rows and columns of a
+// lane as there; h parked divided by the column's scale): g in two FP64
+// operations, h on the integer pipe beside them, as two products of 63-bit
+// significands aligned, added and rounded once (error half an ulp plus about
+// 2^-58).  Values that are not positive normals well inside the range take
+// FP64.
+template <int W>
+__device__ __forceinline__ void relax_rows_fixed(const Params& P, const Tables& T, int wi, double2* __restrict__ fo,
+                                                 const double* __restrict__ px, const double* __restrict__ py,
+                                                 double b, double kappa) {
+  typedef unsigned long long u64;
+  constexpr int kRows = 4;
+  const LaneMap<W> L(P, wi);
+  const int rpw = L.step, nvx = P.nvx, nvy = P.nvy;
+  const unsigned hk = (unsigned)__double2hiint(kappa);
+  const u64 wk = fx::top63(hk, (unsigned)__double2loint(kappa));
+  const int ek = (int)(hk >> 20) - 1022;
+#pragma unroll 1
+  for (int jx = L.l; jx < nvx; jx += L.width) {
+    const double xv = px[jx], bs = b * T.sx[jx];
+    // weights as 63-bit significands and exponents; a or b not positive (Euler
+    // form, steps beyond the collision time): every value takes FP64
+    const unsigned hb = (unsigned)__double2hiint(bs);
+    const bool fit = min(hb, hk) >= (400u << 20) && max(hb, hk) < (1600u << 20);
+    const u64 wb = fx::top63(hb, (unsigned)__double2loint(bs));
+    const int eb = (int)(hb >> 20) - 1022;
+#pragma unroll 1
+    for (int j0 = L.row0; j0 < nvy; j0 += kRows * rpw) {
+      double2 ft[kRows];
+      double2* __restrict__ p = fo + j0 * nvx + jx;
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) ft[u] = j0 + u * rpw < nvy ? p[u * rpw * nvx] : make_double2(1.0, 1.0);
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        if (j0 + u * rpw < nvy) {
+          const double aphi = xv * py[j0 + u * rpw];
+          const unsigned ha = (unsigned)__double2hiint(aphi);
+          int e;
+          const u64 m = fx::mulhi(fx::top63(ha, (unsigned)__double2loint(aphi)), wk);
+          const u64 r = fx::relax((unsigned)__double2hiint(ft[u].y), (unsigned)__double2loint(ft[u].y), wb, eb, m,
+                                  (int)(ha >> 20) + ek, e);
+          unsigned hi, lo;
+          fx::to_words(r, (unsigned)e, hi, lo);
+          double2 o = make_double2(fma(b, ft[u].x, aphi), __hiloint2double((int)hi, (int)lo));
+          if (!fit || e < (int)fx::kExpMin || e > (int)fx::kExpMax) o.y = relax_slow(ft[u].y, aphi, bs, kappa);
+          p[u * rpw * nvx] = o;
+        }
       }
     }
-    return;
   }
-#pragma unroll 4
-  for (int j = lane; j < nv; j += 32) {
-    const double2 ft = tile[j];
-    double2 r = ft;
-    if (ok) {
-      double aphi;
-      if (DIM == 2) {
-        const int vi = T.vinfo[j];
-        aphi = px[vi_jx(vi)] * py[vi_jy(vi)];
-      } else {
-        aphi = px[j];
-      }
-      r.x = fma(b, ft.x, aphi);
-      r.y = fma(b, ft.y, kappa * aphi);
+}
+
+// h of rows streamed by stream_rows_fixed, back from their columns' scales.
+template <int W>
+__device__ __noinline__ void unscale_rows(const Params& P, const Tables& T, int wi, double2* __restrict__ fo) {
+  const LaneMap<W> L(P, wi);
+  for (int jx = L.l; jx < P.nvx; jx += L.width)
+    for (int jy = L.row0; jy < P.nvy; jy += L.step) fo[jy * P.nvx + jx].y *= T.sx[jx];
+}
+
+// A4 of a warp's rows in FP64, f~ unscaled.
+template <int W>
+__device__ __noinline__ void relax_rows_f64(const Params& P, int wi, double2* __restrict__ fo,
+                                            const double* __restrict__ px, const double* __restrict__ py, double b,
+                                            double kappa) {
+  const LaneMap<W> L(P, wi);
+  for (int jx = L.l; jx < P.nvx; jx += L.width)
+    for (int jy = L.row0; jy < P.nvy; jy += L.step) {
+      double2* p = fo + jy * P.nvx + jx;
+      const double2 ft = *p;
+      const double aphi = px[jx] * py[jy];
+      *p = make_double2(fma(b, ft.x, aphi), fma(b, ft.y, kappa * aphi));
     }
-    fo[j] = r;
-  }
 }
 
 }  // namespace
 
-// 4 cells per CTA runs 8 CTAs per SM at 64 registers: spilling a little
-// beats 4 CTAs at 124 registers (measured: 204 -> 191 us on 64^2 x 32^2,
-// 5.14 -> 4.84 ms on 256^2 x 48^2; 5 and 6 CTAs were slower); 8 cells per
-// CTA run 4 CTAs per SM at 64 registers (the choice for large 2D grids).
+// Resident CTAs per SM that the register budget is cut for (FP64 kernel).
+__host__ __device__ constexpr int step_min_ctas(int G) { return G == 4 ? 8 : (G == 8 ? 4 : 1); }
+
 template <int DIM, int G>
-__global__ void __launch_bounds__(32 * G, G == 4 ? 8 : (G == 8 ? 4 : 1))
+__global__ void __launch_bounds__(32 * G, step_min_ctas(G))
     step_f64_kernel(const double2* __restrict__ fin, double2* __restrict__ fout,
                     double4_32a* __restrict__ mom, double4_32a* __restrict__ par, const Params P,
                     const Tables T, int* __restrict__ err) {
   extern __shared__ double4_32a smem4[];
   double* phx = reinterpret_cast<double*>(smem4);
   double* phy = phx + G * P.nvx;
-  __shared__ double s_sum[G][4];
+  __shared__ double s_sum[G][kSums];
+  __shared__ int s_kind[G];
   __shared__ double s_b[G], s_k[G];
   __shared__ int s_ok[G];
 
   const int warp = threadIdx.x >> 5;
-  const int nv = P.nv;
   const int cell = blockIdx.x * G + warp;
   const bool live = cell < P.nx * P.ny;
   // f~ of the warp's cell is parked in the cell's own output slots between
-  // the passes (each lane rereads only what it wrote; the values come back
-  // from L2): staging it in shared memory (16 B per velocity) held an SM to
-  // 3 CTAs, measured 21 % (64^2 x 32^2) and 40 % (256^2 x 48^2) slower
-  double2* tile = fout + (size_t)cell * nv;
+  // the passes (the values come back from L2): staging it in shared memory
+  // (16 B per velocity) held an SM to 3 CTAs, measured 21 % (64^2 x 32^2) and
+  // 40 % (256^2 x 48^2) slower
+  double2* tile = fout + (size_t)cell * P.nv;
 
   if (live) stream_cell<DIM>(P, T, fin, cell, tile, s_sum[warp]);
+  if ((threadIdx.x & 31) == 0) s_kind[warp] = SUMS_VELOCITY;
   __syncthreads();
-  if (DIM == 2 && G >= 2) {
+  if constexpr (DIM == 2 && G >= 2) {
     __shared__ SolveXchg<G> s_x;
-    if (warp < 2) maxwellian_cells_2w<G>(P, T, blockIdx.x * G, s_sum, phx, phy, s_b, s_k, s_ok, mom, par, err, s_x);
+    if (warp < 2)
+      maxwellian_cells_2w<G>(P, T, blockIdx.x * G, s_sum, s_kind, phx, phy, s_b, s_k, s_ok, mom, par, err, s_x);
   } else if (warp == 0) {
-    maxwellian_cells<DIM, G>(P, T, blockIdx.x * G, s_sum, phx, phy, s_b, s_k, s_ok, mom, par, err);
+    maxwellian_cells<DIM, G>(P, T, blockIdx.x * G, s_sum, s_kind, phx, phy, s_b, s_k, s_ok, mom, par, err);
   }
   __syncthreads();
-  if (!live) return;
+  // a failed cell keeps f^{n+1} = f~ (flagged)
+  if (live && s_ok[warp])
+    relax_cell<DIM>(P, T, tile, phx + warp * P.nvx, phy + warp * P.nvy, s_b[warp], s_k[warp]);
+}
 
-  relax_cell<DIM>(P, T, fout, cell, phx + warp * P.nvx, phy + warp * P.nvy, s_b[warp], s_k[warp],
-                  s_ok[warp] != 0);
+// The 2D step with the work split over the integer and the FP64 pipe: 8
+// warps, G cells of W = 8 / G warps each.
+template <int G>
+__global__ void __launch_bounds__(256, 4)
+    step_fixed_kernel(const double2* __restrict__ fin, double2* __restrict__ fout, double4_32a* __restrict__ mom,
+                      double4_32a* __restrict__ par, const Params P, const Tables T, int* __restrict__ err) {
+  constexpr int W = 8 / G;
+  extern __shared__ double4_32a smem4[];
+  double* phx = reinterpret_cast<double*>(smem4);
+  double* phy = phx + G * P.nvx;
+  __shared__ double s_sum[8][kSums];
+  __shared__ int s_kind[8];
+  __shared__ double s_b[G], s_k[G];
+  __shared__ int s_ok[G];
+  __shared__ CellSolve<G> s_x;
+
+  const int warp = threadIdx.x >> 5, mine = warp / W, wi = warp % W;
+  const int cell = blockIdx.x * G + mine;
+  const bool live = cell < P.nx * P.ny;
+  double2* tile = fout + (size_t)cell * P.nv;  // f~ is parked in the output slots
+  int kind = SUMS_VELOCITY;
+  if (live) kind = stream_rows<W>(P, T, fin, cell, wi, tile, s_sum[warp]);
+  if ((threadIdx.x & 31) == 0) s_kind[warp] = kind;
+  __syncthreads();
+  const bool fixed =
+      maxwellian_cells_fixed<G, W>(P, T, blockIdx.x * G, s_sum, s_kind, phx, phy, s_b, s_k, s_ok, mom, par, err, s_x);
+  if (!live) return;
+  const double *px = phx + mine * P.nvx, *py = phy + mine * P.nvy;
+  const bool ok = s_ok[mine] != 0;
+  if (kind == SUMS_INDEX && fixed && ok) {
+    relax_rows_fixed<W>(P, T, wi, tile, px, py, s_b[mine], s_k[mine]);
+    return;
+  }
+  // a failed cell keeps f^{n+1} = f~ (flagged)
+  if (kind == SUMS_INDEX) unscale_rows<W>(P, T, wi, tile);
+  if (ok) relax_rows_f64<W>(P, wi, tile, px, py, s_b[mine], s_k[mine]);
 }
 
 namespace {
@@ -631,66 +1267,83 @@ size_t step_smem(const Params& P, int G) {
   return sizeof(double) * (size_t)G * (P.nvx + P.nvy);
 }
 
-template <int DIM, int G>
-cudaError_t launch_g(const Params& P, const Tables& T, const double2* fin, double2* fout,
-                     double4_32a* mom, double4_32a* par, int* err, cudaStream_t stream) {
-  const int ncell = P.nx * P.ny;
-  const unsigned grid = (unsigned)((ncell + G - 1) / G);
-  step_f64_kernel<DIM, G><<<grid, 32 * G, step_smem(P, G), stream>>>(fin, fout, mom, par, P, T, err);
-  return cudaGetLastError();
-}
+typedef void (*StepKernel)(const double2*, double2*, double4_32a*, double4_32a*, const Params, const Tables, int*);
 
-// The attribute belongs to the kernel, not to a solver: set it to the
-// largest dynamic shared memory any solver may request (what the device
-// allows a CTA beside the kernel's static shared memory) so that solvers
-// with different grids sharing an instantiation never shrink it.
-template <int DIM, int G>
-cudaError_t prepare_g(const Params&) {
-  int dev = 0, optin = 0;
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, step_f64_kernel<DIM, G>);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(step_f64_kernel<DIM, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              optin - (int)fa.sharedSizeBytes);
-}
-
-template <int DIM>
-cudaError_t dispatch(const Params& P, const Tables& T, const double2* fin, double2* fout,
-                     double4_32a* mom, double4_32a* par, int* err, cudaStream_t stream) {
+// The problem's kernel and its threads per CTA; null for an unknown tile.
+StepKernel step_kernel(const Params& P, unsigned* threads) {
+  *threads = 32u * (unsigned)P.tile;
+  if (P.dim == 1) switch (P.tile) {
+      case 1: return step_f64_kernel<1, 1>;
+      case 2: return step_f64_kernel<1, 2>;
+      case 4: return step_f64_kernel<1, 4>;
+      case 8: return step_f64_kernel<1, 8>;
+      default: return nullptr;
+    }
+  if (P.lane_bits == 0) switch (P.tile) {
+      case 1: return step_f64_kernel<2, 1>;
+      case 2: return step_f64_kernel<2, 2>;
+      case 4: return step_f64_kernel<2, 4>;
+      case 8: return step_f64_kernel<2, 8>;
+      default: return nullptr;
+    }
+  *threads = 256u;
   switch (P.tile) {
-    case 1: return launch_g<DIM, 1>(P, T, fin, fout, mom, par, err, stream);
-    case 2: return launch_g<DIM, 2>(P, T, fin, fout, mom, par, err, stream);
-    case 4: return launch_g<DIM, 4>(P, T, fin, fout, mom, par, err, stream);
-    case 8: return launch_g<DIM, 8>(P, T, fin, fout, mom, par, err, stream);
+    case 1: return step_fixed_kernel<1>;
+    case 2: return step_fixed_kernel<2>;
+    case 4: return step_fixed_kernel<4>;
+    case 8: return step_fixed_kernel<8>;
+    default: return nullptr;
   }
-  return cudaErrorInvalidValue;
-}
-
-template <int DIM>
-cudaError_t prepare_dim(const Params& P) {
-  switch (P.tile) {
-    case 1: return prepare_g<DIM, 1>(P);
-    case 2: return prepare_g<DIM, 2>(P);
-    case 4: return prepare_g<DIM, 4>(P);
-    case 8: return prepare_g<DIM, 8>(P);
-  }
-  return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
 size_t step_f64_smem_bytes(const Params& P, int tile) { return step_smem(P, tile); }
 
+// Lanes per velocity row of the fixed-point kernels: the 4, 8, 16 or 32 that
+// leave the fewest lanes idle (more lanes on a tie, for wider accesses).  They
+// need weights that sum to one (Courant number at most 1), 128 velocities to
+// sample, and index sums within 95 bits (at most 512 velocities per axis).
+void step_f64_plan(Params& P, double max_courant) {
+  P.lane_bits = 0;
+  if (P.dim != 2 || P.nv < 128 || P.nvx > 512 || P.nvy > 512 || max_courant > 1.0 + 4e-15) return;
+  double best = 0.0;
+  for (int lb = 5; lb >= 2; --lb) {
+    const int lw = 1 << lb, rpw = 32 >> lb;
+    const int width = (P.nvx + lw - 1) / lw * lw, rows = (P.nvy + rpw - 1) / rpw * rpw;
+    const double use = (double)P.nv / ((double)width * rows);
+    if (use > best + 1e-9) {
+      best = use;
+      P.lane_bits = lb;
+    }
+  }
+}
+
+// The attribute belongs to the kernel, not to a solver: set it to the
+// largest dynamic shared memory any solver may request (what the device
+// allows a CTA beside the kernel's static shared memory) so that solvers
+// with different grids sharing an instantiation never shrink it.
 cudaError_t prepare_step_f64(const Params& P) {
-  return P.dim == 1 ? prepare_dim<1>(P) : prepare_dim<2>(P);
+  unsigned threads = 0;
+  const StepKernel k = step_kernel(P, &threads);
+  if (!k) return cudaErrorInvalidValue;
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
 cudaError_t launch_step_f64(const Params& P, const Tables& T, const double2* fin, double2* fout,
                             double4_32a* mom, int* err, cudaStream_t stream, double4_32a* par) {
-  return P.dim == 1 ? dispatch<1>(P, T, fin, fout, mom, par, err, stream)
-                    : dispatch<2>(P, T, fin, fout, mom, par, err, stream);
+  unsigned threads = 0;
+  const StepKernel k = step_kernel(P, &threads);
+  if (!k) return cudaErrorInvalidValue;
+  const unsigned grid = (unsigned)((P.nx * P.ny + P.tile - 1) / P.tile);
+  k<<<grid, threads, step_smem(P, P.tile), stream>>>(fin, fout, mom, par, P, T, err);
+  return cudaGetLastError();
 }
 
 }  // namespace bgk

@@ -1,0 +1,119 @@
+"""The 2D FP64 step's fixed-point kernels against the FP64 CPU oracle where
+they can go wrong: velocity rows that fill no lane count, columns and rows
+past the grid, c = 0, Courant number 1, boxes off centre, every number of
+warps per cell, and states that leave the fixed-point range (negative and
+zero values, steep fronts, densities far from one, relaxation weights beyond
+one), for which the kernels fall back to FP64.
+
+Tolerances as in test_gpu_parity.py: 1e-13 of the largest value and 1e-12 of
+each value per step.  Each rounds at most five times a step (streaming 2,
+relaxation 1, parameters), each to half an ulp of a sum of positive terms.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0903_4044_gb300 import bgk as B
+from paper_0903_4044_gb300 import build, solver
+from paper_0903_4044_gb300 import workloads as W
+from test_gpu_parity import assert_moments_close, assert_state_close
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    oracle.build()
+    B.lib()
+
+
+def pair(nx, ny, nvx, nvy, *, tile=0, vx=(-4.0, 4.0), vy=(-4.5, 4.5), cfl=0.6, cons=1, exact=1, kinds=(1, 1, 1, 1),
+         omega=0.5, n=1.0, length=0.5):
+    rest, lid = (n, 0.0, 0.0, 1.0), (n, 0.05, 0.0, 1.0)
+    kw = dict(dim=2, nx=nx, ny=ny, lx=nx * length, ly=ny * length, nvx=nvx, nvy=nvy, vx=vx, vy=vy, cfl=cfl,
+              conservative=cons, relax_exact=exact, omega=omega)
+    cfg = B.make_config(**kw, bc=[(k, *s) for k, s in zip(kinds, (rest, rest, rest, lid))], tile_cells=tile)
+    prob = oracle.Problem(oracle.make_config(**kw, bc_kind=kinds, bc_state=(rest, rest, rest, lid)))
+    xi = W.perturbation(3, prob.ncell, prob.nv)
+    g, h = oracle.init_uniform(prob, rest, xi, 1e-2)
+    return solver.Solver(cfg), prob, g, h
+
+
+def run(s, prob, g, h, steps=3):
+    s.set_state(np.ascontiguousarray(np.stack([g, h], -1)))
+    s.step(steps)
+    g1, h1, mom = oracle.step(prob, g, h, steps)
+    return s.get_state(), s.moments(which=1), g1, h1, mom
+
+
+@pytest.mark.parametrize("tile", [1, 2, 4, 8])
+@pytest.mark.parametrize("nvx,nvy", [(12, 11), (13, 17), (21, 20), (33, 12), (48, 16), (65, 20), (128, 9)])
+def test_velocity_grids(nvx, nvy, tile):
+    s, prob, g, h = pair(5, 4, nvx, nvy, tile=tile)
+    st, m, g1, h1, mom = run(s, prob, g, h)
+    assert_state_close(st, g1, h1)
+    assert_moments_close(m, mom, vscale=0.05)
+    s.close()
+
+
+@pytest.mark.parametrize("case", [
+    dict(cfl=1.0), dict(cfl=1.0, vx=(-4.2, 4.2), vy=(-3.9, 3.9)), dict(vx=(-4.0, 6.0), vy=(-5.0, 4.0), kinds=(0, 0, 1, 1)),
+    dict(kinds=(2, 2, 2, 2)), dict(omega=0.74), dict(cons=0), dict(exact=0), dict(n=1e60), dict(n=1e-60),
+    dict(n=40.0, exact=0), dict(n=3000.0), dict(vx=(-40.0, 40.0), vy=(-40.0, 40.0), cons=0)])
+def test_options(case):
+    # nvx and nvy odd: a zero velocity per axis; n = 40 with the Euler form
+    # makes the relaxation weight of f~ negative, n = 3000 makes it tiny; the
+    # box of +-40 underflows to zeros at its corners
+    s, prob, g, h = pair(6, 5, 21, 25, **case)
+    steps = 1 if case.get("n") == 40.0 else 3
+    st, m, g1, h1, mom = run(s, prob, g, h, steps)
+    if case.get("n") == 40.0:  # f~ and Phi subtract: no bound relative to each value
+        assert np.abs(st[..., 0] - g1).max() <= 1e-13 * np.abs(g1).max()
+        assert np.abs(st[..., 1] - h1).max() <= 1e-13 * np.abs(h1).max()
+    elif "vx" in case and case["vx"][1] == 40.0:
+        # values below 2.2e-308 are spaced 4.9e-324 apart whatever their size:
+        # four spacings (two products and two roundings) beside the 1e-12
+        for a, b in ((st[..., 0], g1), (st[..., 1], h1)):
+            assert (np.abs(a - b) <= 1e-12 * np.abs(b) + 2e-323).all()
+    else:
+        assert_state_close(st, g1, h1)
+    assert_moments_close(m, mom, vscale=0.05)
+    s.close()
+
+
+@pytest.mark.parametrize("what", ["negative", "zero", "front", "fast"])
+def test_states_out_of_range(what):
+    s, prob, g, h = pair(6, 5, 24, 20, cons=0, kinds=(2, 2, 2, 2))
+    j = np.arange(prob.nv)
+    if what == "negative":
+        g[7, j % 13 == 0] *= -0.01
+        h[11, j % 7 == 0] *= -0.01
+    elif what == "zero":
+        g[7, j % 3 == 0] = 0.0
+        h[8] = 0.0
+        h[14, ::2] = 0.0
+    elif what == "front":
+        g[12:18] *= 1e9
+        h[12:18] *= 1e9
+    else:  # a beam in a few velocities between the sampled ones
+        g[9, 37] += 1e5 * g.max()
+        h[9, 38] += 1e5 * h.max()
+    st, m, g1, h1, mom = run(s, prob, g, h, 1)
+    for a, b in ((st[..., 0], g1), (st[..., 1], h1)):
+        assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
+        if what != "negative":
+            assert (np.abs(a - b) <= 1e-12 * np.abs(b)).all()
+    assert_moments_close(m, mom, vscale=0.05)
+    s.close()
+
+
+def test_nan_is_flagged():
+    s, prob, g, h = pair(6, 5, 24, 20)
+    g[9, 5] = np.nan
+    s.set_state(np.ascontiguousarray(np.stack([g, h], -1)))
+    s.step(1)
+    with pytest.raises(B.BgkError) as e:
+        s.sync()
+    assert e.value.status == B.BGK_ERR_NUMERIC
+    s.close()
