@@ -1639,6 +1639,7 @@ bgk_status validate3v(const bgk3v_config* c, bgk::Params3v& p, double* max_coura
   } else {
     return fail(BGK_ERR_INVALID_ARG, "need dt > 0, or dt = 0 and cfl > 0");
   }
+  bgk::plan3v(p);
   *max_courant = mx * p.dt / p.dx;
   if (*max_courant > 1e6) return fail(BGK_ERR_UNSUPPORTED, "Courant number %.3g is too large", *max_courant);
   return BGK_OK;

@@ -136,6 +136,15 @@ BGK_HD u64 double_to_units(u32 hi, u32 lo, u32 eref) {
   return shr64(m << 8, d + 2u) + ((u32)shr64(m << 8, d + 1u) & 1u);
 }
 
+// The same in the unit 2^(eref - 1097), truncated: below 2^75 for an exponent
+// field of at most eref.
+BGK_HD i96 double_to_units96(u32 hi, u32 lo, u32 eref) {
+  const u64 m = ((u64)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 8;
+  const u32 e = eref - (hi >> 20) + 2u;  // m 2^(16 - e)
+  const u64 top = shr64(m, e + 16u);
+  return {e >= 16u ? (u32)shr64(m, e - 16u) : (u32)m << ((16u - e) & 31u), (u32)top, (u32)(top >> 32)};
+}
+
 // The double nearest to v in units of 2^(eref - 1081), |v| < 2^95 (words).
 BGK_HD void wide_to_words(i96 v, u32 eref, u32& hi, u32& lo) {
   const bool minus = v.a2 >> 31;

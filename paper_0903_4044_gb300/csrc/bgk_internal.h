@@ -158,9 +158,12 @@ cudaError_t launch_persistent(int ninst, int total_units, int nsteps, GridBarrie
 // Full 3D velocity grid, one spatial dimension (bgk_step3v.cu).
 struct Params3v {
   int nx, nvx, nvy, nvz, nv;
+  int lane_bits, zw_bits;  // fixed-point kernel: log2 of the lanes per velocity row and of the warps
+                           // along z (plan3v); lane_bits = 0: FP64 kernel
   int conservative, relax_exact;
   double x0, dx, dt, dv, omega;
   double dc[3], vmin[3];
+  double half[3], inv_half[3], mid[3];  // half velocity steps, their reciprocals, box centres (plan3v)
 };
 struct Tables3v {
   const double* c[3];    // [nvx], [nvy], [nvz] velocity-cell centres
@@ -175,6 +178,8 @@ struct Inflow3v {
 };
 cudaError_t launch_tables3v(const Params3v& P, double* c0, double* c1, double* c2, double* cc, int* shift,
                             int* upwind, double* rem, double* ghost, const Inflow3v& inflow, cudaStream_t stream);
+// Fills P.lane_bits, P.zw_bits and P.half .. P.mid from the velocity grid.
+void plan3v(Params3v& P);
 cudaError_t launch_init3v(const Params3v& P, const Tables3v& T, double x_split, const Inflow3v& lr, double* f,
                           cudaStream_t stream);
 cudaError_t launch_step3v(const Params3v& P, const Tables3v& T, const double* fin, double* fout, double* mom,

@@ -36,7 +36,7 @@
 // step_f64_kernel is the FP64-only form: 1D grids, and 2D grids that
 // step_f64_plan leaves to it.
 #include "bgk_device.cuh"
-#include "bgk_fixed.cuh"
+#include "bgk_solve.cuh"
 
 namespace bgk {
 
@@ -121,11 +121,6 @@ __device__ __forceinline__ CellEdge cell_edge(const Params& P, const Tables& T, 
 __device__ __forceinline__ fx::i96 shfl96(fx::i96 v, int from) {
   return {__shfl_sync(0xffffffffu, v.a0, from), __shfl_sync(0xffffffffu, v.a1, from),
           __shfl_sync(0xffffffffu, v.a2, from)};
-}
-__device__ __forceinline__ fx::i96 xor_add96(fx::i96 keep, fx::i96 send, int mask) {
-  const fx::i96 got = {__shfl_xor_sync(0xffffffffu, send.a0, mask), __shfl_xor_sync(0xffffffffu, send.a1, mask),
-                       __shfl_xor_sync(0xffffffffu, send.a2, mask)};
-  return fx::add(keep, got);
 }
 __device__ __forceinline__ fx::i96 pick(bool c, fx::i96 x, fx::i96 y) {
   return {c ? x.a0 : y.a0, c ? x.a1 : y.a1, c ? x.a2 : y.a2};
@@ -782,52 +777,14 @@ __device__ void maxwellian_cells_2w(const Params& P, const Tables& T, int cell0,
 
 // Phase 2 of the fixed-point kernels: the Gaussians of a cell on its own warp
 // and on the integer pipe, the scalar solve with cells in lanes on one warp.
-// A rounding-free index form of the central sums: with integers k' = k - k0,
-// k0 next to the mean, c - u = half k' + delta.
-__device__ const unsigned long long kExp2[32] = BGK_EXP2_TABLE;
-
-constexpr int kMaxIndexShift = 1024;  // |k0|: keeps sum k'^2 e within 95 bits
-
 template <int G>
 struct CellSolve {
-  // base point of the Gaussians per axis, (c_k - u) sqrt(log2 e / theta) = a k - c in units of 2^-58
-  long long a[G][2], c[G][2];
-  int k0[G][2];
+  AxisBase base[G][2];
   double sums[G][2][3];  // sum e, sum k' e, sum k'^2 e
   double ap[G];          // a n / (pi theta)
   int need[G];
   int go;  // 1: sums wanted, 0: factors wanted, -1: a cell is out of range (FP64 path)
 };
-
-// 1/x and 1/sqrt(x) of positive normal x by one third-order (Householder)
-// step from the FP32 approximation of relative error e0 < 2^-21: three and
-// five FP64 operations, error e0^3 beside the roundings (an FP64 division or
-// square root costs ten or more).
-__device__ __forceinline__ float to_float_bits(double x) {  // truncated, exponent kept in range by the caller
-  return __uint_as_float((((unsigned)__double2hiint(x) - 0x38000000u) << 3) | ((unsigned)__double2loint(x) >> 29));
-}
-__device__ __forceinline__ double to_double_bits(float y) {
-  const unsigned u = __float_as_uint(y);
-  return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
-}
-__device__ __forceinline__ double rcp3(double x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_bits(x)));
-  const double d = to_double_bits(y), e = fma(-x, d, 1.0);
-  return fma(d, fma(e, e, e), d);
-}
-__device__ __forceinline__ double rsqrt3(double x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_bits(x)));
-  const double d = to_double_bits(y), e = fma(-x * d, d, 1.0);
-  return fma(d, e * fma(0.375, e, 0.5), d);
-}
-// Whether x is positive, finite and well inside the FP32 exponent range.
-__device__ __forceinline__ bool in_range(double x) {
-  const unsigned h = (unsigned)__double2hiint(x);
-  return h - 0x3a000000u < 0x0c000000u;  // 2^-95 to 2^97
-}
-__device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
 // A cell's solve: moments q, parameters p (the base point of the Gaussians),
 // ith = 1 / theta, isq = 1 / sqrt(theta) of p.
@@ -844,45 +801,25 @@ struct FixedSolve {
 template <int G>
 __device__ __forceinline__ bool publish_base(const Params& P, const VelocityGrid& V, const FixedSolve& E, int c, CellSolve<G>& X) {
   const double gamma = E.isq * 1.2011224087864498;  // sqrt(log2 e)
-  bool fit = true;
-#pragma unroll
-  for (int x = 0; x < 2; ++x) {
-    const int n = x == 0 ? P.nvx : P.nvy;
-    const double half = x == 0 ? V.half_x : V.half_y;
-    const double off = E.p[1 + x] - (x == 0 ? V.mid_x : V.mid_y);
-    const double a = half * gamma, s = off * gamma;
-    const double r = fma(off, x == 0 ? V.inv_half_x : V.inv_half_y, 6755399441055744.0);  // 1.5 2^52: rounds to an integer
-    const int k0 = __double2loint(r);
-    // |s| + a n < 31.9, |off| below 1024 half steps (words: the exponent decides)
-    const double reach = fma(a, (double)n, fabs(s));
-    fit = fit && abs_hi(reach) < 0x403fe666u && abs_hi(r) == 0x43380000u - (k0 < 0 ? 1u : 0u) &&
-          (unsigned)(k0 + kMaxIndexShift) < 2u * kMaxIndexShift;
-    X.a[c][x] = fx::to_fix58((unsigned)__double2hiint(a), (unsigned)__double2loint(a));
-    X.c[c][x] = fx::to_fix58((unsigned)__double2hiint(s), (unsigned)__double2loint(s));
-    X.k0[c][x] = k0;
-  }
-  return fit;
+  AxisBase x, y;
+  const bool fx = axis_base(P.nvx, V.half_x, V.inv_half_x, V.mid_x, E.p[1], gamma, x);
+  const bool fy = axis_base(P.nvy, V.half_y, V.inv_half_y, V.mid_y, E.p[2], gamma, y);
+  X.base[c][0] = x;
+  X.base[c][1] = y;
+  return fx && fy;
 }
 
 // nu = n theta^(1-omega) and the relaxation weights, exp(-nu dt) on the
 // integer pipe where its argument allows.
 __device__ __forceinline__ void relax_weights_fixed(const Params& P, const FixedSolve& E, double& a, double& b) {
-  const double nu = E.q[0] * (P.omega == 0.5 ? E.q[3] * E.ivs : pow(E.q[3], 1.0 - P.omega));
+  const double nu = E.q[0] * (P.omega == 0.5 ? E.q[3] * E.ivs : pow_fixed(E.q[3], 1.0 - P.omega));
   const double x = nu * P.dt;
   if (!P.relax_exact) {
     a = x;
     b = 1.0 - a;
     return;
   }
-  const double t = x * 1.4426950408889634;  // log2 e
-  if (abs_hi(t) < 0x40400000u) {             // below 32
-    const unsigned long long f = (unsigned long long)fx::to_fix58((unsigned)__double2hiint(t), (unsigned)__double2loint(t));
-    unsigned hi, lo;
-    fx::gauss_words(fx::exp2_neg(f << 6, (const fx::u64*)kExp2), (unsigned)(f >> 58), hi, lo);
-    b = __hiloint2double((int)hi, (int)lo);
-  } else {
-    b = exp(-x);
-  }
+  b = exp_neg_fixed(x);
   a = 1.0 - b;
 }
 
@@ -934,28 +871,8 @@ template <int G, int W>
 __device__ __forceinline__ void gauss_sums(const Params& P, int c, int wi, CellSolve<G>& X) {
   const AxisMap<W> A(wi);
   if (W > 2 && A.x > 1) return;  // the whole warp
-  const int n = A.x == 0 ? P.nvx : P.nvy, k0 = X.k0[c][A.x];
-  const long long a = X.a[c][A.x], off = X.c[c][A.x];
-  fx::i96 s[3] = {{0u, 0u, 0u}, {0u, 0u, 0u}, {0u, 0u, 0u}};
-#pragma unroll 1
-  for (int j = A.i; j < n; j += A.kLanes) {
-    const int k = 2 * j + 1 - n, kk = k - k0;
-    unsigned q2;
-    const unsigned long long q = fx::gauss(a * k - off, (const fx::u64*)kExp2, q2);
-    const fx::i96 e = fx::wide(q2 < 62u ? q >> (q2 + 1u) : 0);  // units of 2^-62
-    s[0] = fx::add(s[0], e);
-    s[1] = fx::add(s[1], fx::muls(e, kk));
-    s[2] = fx::add(s[2], fx::mul(e, (unsigned)(kk * kk)));
-  }
-#pragma unroll
-  for (int m = A.kLanes / 2; m > 0; m >>= 1)
-#pragma unroll
-    for (int p = 0; p < 3; ++p) s[p] = xor_add96(s[p], s[p], m);
-  if (A.i < 3) {
-    unsigned hi, lo;
-    fx::wide_to_words(A.i == 0 ? s[0] : A.i == 1 ? s[1] : s[2], 1081u - 62u, hi, lo);
-    X.sums[c][A.x][A.i] = __hiloint2double((int)hi, (int)lo);
-  }
+  const double t = axis_index_sums<AxisMap<W>::kLanes>(A.x == 0 ? P.nvx : P.nvy, X.base[c][A.x], A.i);
+  if (A.i < 3) X.sums[c][A.x][A.i] = t;
 }
 
 // Cell c's a Phi factors at the final parameters, along the warp's axis.
@@ -965,13 +882,13 @@ __device__ __forceinline__ void gauss_factors(const Params& P, int c, int wi, co
   const AxisMap<W> A(wi);
   if (W > 2 && A.x > 1) return;
   const int n = A.x == 0 ? P.nvx : P.nvy;
-  const long long a = X.a[c][A.x], off = X.c[c][A.x];
+  const AxisBase B = X.base[c][A.x];
   const double scale = X.ap[c];
   double* out = A.x == 0 ? px : py;
 #pragma unroll 1
   for (int j = A.i; j < n; j += A.kLanes) {
     unsigned q2, hi, lo;
-    const unsigned long long q = fx::gauss(a * (2 * j + 1 - n) - off, (const fx::u64*)kExp2, q2);
+    const unsigned long long q = fx::gauss(B.a * (2 * j + 1 - n) - B.c, (const fx::u64*)kExp2, q2);
     fx::gauss_words(q, q2, hi, lo);
     const double e = __hiloint2double((int)hi, (int)lo);
     out[j] = A.x == 0 ? scale * e : e;
@@ -1032,15 +949,8 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
       bool fit = true;
       if (!E.conv && !E.fail) {
         double M[2][3];
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-          const double half = x == 0 ? V.half_x : V.half_y;
-          const double d = fma((double)X.k0[c][x], half, x == 0 ? V.mid_x : V.mid_y) - E.p[1 + x];
-          const double m0 = X.sums[c][x][0], t1 = half * X.sums[c][x][1];
-          M[x][0] = m0;
-          M[x][1] = fma(d, m0, t1);
-          M[x][2] = fma(half * half, X.sums[c][x][2], d * (t1 + M[x][1]));
-        }
+        central_sums(X.sums[c][0], X.base[c][0].k0, V.half_x, V.mid_x, E.p[1], M[0]);
+        central_sums(X.sums[c][1], X.base[c][1].k0, V.half_y, V.mid_y, E.p[2], M[1]);
         eff_update(V, M[0], M[1], E);
         if (wr) fit = publish_base(P, V, E, c, X) || E.fail;
       }

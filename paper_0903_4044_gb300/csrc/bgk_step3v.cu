@@ -17,7 +17,7 @@
 //   pass 2  f^{n+1} = b f~ + a Phi, Phi = px[jx] py[jy] pz[jz], on the f~
 //           values pass 1 parked in the cell's output slots (each thread
 //           rereads its own writes, from L2).
-#include "bgk_device.cuh"
+#include "bgk_solve.cuh"
 
 namespace bgk {
 
@@ -68,7 +68,7 @@ __device__ __forceinline__ void bar_axes() { asm volatile("bar.sync 1, 96;" ::: 
 // Warp `a` (0..2): 1D Gaussian e_j = exp(-(c_j - u)^2 / theta) of its axis
 // at p; returns the warp totals (sum e, sum d e, sum d^2 e) in every lane and
 // leaves e_j in fac (when not null).
-__device__ __forceinline__ void axis_sums(const Params3v& P, const Tables3v& T, int a, double u, double inv_th,
+__device__ __forceinline__ void axis_sums3v(const Params3v& P, const Tables3v& T, int a, double u, double inv_th,
                                           double* fac, double (&s)[3]) {
   const int lane = threadIdx.x & 31;
   s[0] = s[1] = s[2] = 0.0;
@@ -84,17 +84,21 @@ __device__ __forceinline__ void axis_sums(const Params3v& P, const Tables3v& T, 
     for (int m = 16; m > 0; m >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], m);
 }
 
-}  // namespace
+// Scratch of a CTA.
+struct Shared3v {
+  double red[kW * 8], tot[8];
+  double ax[3][3];  // per axis: sum e, sum d e, sum d^2 e (fixed point: index sums)
+  double ab[2];     // relaxation weights a (on Phi; fixed point: its factor), b (on f~)
+  AxisBase base[3];
+  int ok, go, valid[kW];
+};
 
-__global__ void __launch_bounds__(kT) step3v_kernel(const Params3v P, const Tables3v T,
-                                                    const double* __restrict__ fin, double* __restrict__ fout,
-                                                    double* __restrict__ mom, int* __restrict__ err) {
-  extern __shared__ double fac[];  // px[nvx], py[nvy], pz[nvz]
-  __shared__ double red[kW * 8], tot[8];
-  __shared__ double s_ax[3][3];   // per axis: sum e, sum d e, sum d^2 e
-  __shared__ double s_ab[2];      // relaxation weights a (on Phi), b (on f~)
-  __shared__ int s_ok;
-  const int i = blockIdx.x;
+// The step of cell i in FP64, for any grid and any values (all threads).
+__device__ __noinline__ void cell3v_f64(const Params3v& P, const Tables3v& T, const double* __restrict__ fin,
+                                        double* __restrict__ fout, double* __restrict__ mom, int* __restrict__ err,
+                                        int i, double* fac, Shared3v& S) {
+  double *red = S.red, *tot = S.tot, (*s_ax)[3] = S.ax, *s_ab = S.ab;
+  int& s_ok = S.ok;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // pass 1: stream (f~ parked in the cell's output slots) and the five sums
@@ -133,7 +137,7 @@ __global__ void __launch_bounds__(kT) step3v_kernel(const Params3v P, const Tabl
       const double vs = sqrt(q[4]);
       for (int it = 1; it <= kEffMaxIt; ++it) {
         double s[3];
-        axis_sums(P, T, warp, p[1 + warp], 1.0 / p[4], nullptr, s);
+        axis_sums3v(P, T, warp, p[1 + warp], 1.0 / p[4], nullptr, s);
         if (lane == 0)
           for (int m = 0; m < 3; ++m) s_ax[warp][m] = s[m];
         bar_axes();
@@ -169,7 +173,7 @@ __global__ void __launch_bounds__(kT) step3v_kernel(const Params3v P, const Tabl
     const double b = !ok ? 1.0 : P.relax_exact ? exp(-nu * P.dt) : 1.0 - a;
     double* fw = fac + (warp == 0 ? 0 : warp == 1 ? P.nvx : P.nvx + P.nvy);
     double s[3];
-    axis_sums(P, T, warp, p[1 + warp], 1.0 / p[4], fw, s);
+    axis_sums3v(P, T, warp, p[1 + warp], 1.0 / p[4], fw, s);
     if (warp == 0) {
       __syncwarp();
       const double scale = a * p[0] / (kPi() * p[4] * sqrt(kPi() * p[4]));
@@ -198,6 +202,366 @@ __global__ void __launch_bounds__(kT) step3v_kernel(const Params3v P, const Tabl
   for (int j = threadIdx.x; j < P.nv; j += kT) {
     const Idx3 k = split3(P, j);
     fo[j] = fma(b, fo[j], px[k.jx] * py[k.jy] * pz[k.jz]);
+  }
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kT) step3v_kernel(const Params3v P, const Tables3v T,
+                                                    const double* __restrict__ fin, double* __restrict__ fout,
+                                                    double* __restrict__ mom, int* __restrict__ err) {
+  extern __shared__ double fac[];  // px[nvx], py[nvy], pz[nvz]
+  __shared__ Shared3v S;
+  cell3v_f64(P, T, fin, fout, mom, err, blockIdx.x, fac, S);
+}
+
+namespace {
+
+// ---- fixed-point kernel -------------------------------------------------------
+// The FP64 pipe takes 64 to 76 cycles per warp instruction and bounded the
+// step (12.1 operations per velocity).  Here four remain, two to stream and
+// two to relax; the moment sums are exact integers, the Gaussians and the
+// relaxation weight come from the integer pipe.  2048 x 30^3: 1.24 -> 0.63 ms a
+// step, 512 x 16^3: 126 -> 50 us.  What bounds it now: pass 1 (half of the
+// time) by its loads, each lane's column comes from another cell (8 of each 32
+// bytes are used); the solve of a 16^3 cell takes as long as its passes.
+//
+// 2^lane_bits lanes share a velocity row (fixed jy, jz); the 8 warps split z
+// 2^zw_bits ways and y the rest.  A lane takes its columns jx one after the
+// other over its rows, y inside z.
+struct Map3v {
+  int l, width, y0, ystep, yrows, z0, zstep, zrows;
+  __device__ __forceinline__ explicit Map3v(const Params3v& P) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lb = P.lane_bits, zb = P.zw_bits;
+    width = 1 << lb;
+    l = lane & (width - 1);
+    z0 = warp & ((1 << zb) - 1);
+    zstep = 1 << zb;
+    ystep = (kW >> zb) * (32 >> lb);
+    y0 = (warp >> zb) * (32 >> lb) + (lane >> lb);
+    yrows = (P.nvy + ystep - 1) / ystep;
+    zrows = (P.nvz + zstep - 1) / zstep;
+  }
+};
+
+// Sources of a column of cell i: the shifted cell and its upwind neighbour,
+// or the inflow Maxwellian beyond an end.
+__device__ __forceinline__ const double* column_source(const Params3v& P, const Tables3v& T,
+                                                       const double* __restrict__ fin, int i) {
+  return i < 0 ? T.ghost : i >= P.nx ? T.ghost + P.nv : fin + (size_t)i * P.nv;
+}
+
+// Integer sums of weight (first + step k) along an axis of `rows` rows from
+// the running sums r0 = sum g, r1 = sum (rows - k) g, r2 = sum (rows - k)
+// (rows - k + 1) / 2 g: sum w g and sum w^2 g with w = 2 j + 1 - n.
+__device__ __forceinline__ void axis_weights(fx::i96 r0, fx::i96 r1, fx::i96 r2, int first, int step, int rows, int n,
+                                             fx::i96& w1, fx::i96& w2) {
+  const int A = 2 * (first + step * rows) + 1 - n, B = 2 * step;
+  const fx::i96 b1 = fx::mul(r1, (unsigned)B);
+  w1 = fx::add(fx::muls(r0, A), fx::neg(b1));
+  w2 = fx::add(fx::add(fx::mul(r0, (unsigned)(A * A)), fx::neg(fx::muls(b1, 2 * A + B))),
+               fx::mul(r2, (unsigned)(2 * B * B)));
+}
+
+// Rows whose values are loaded together (2048 x 30^3: 0.77 ms a step with 4,
+// 0.71 with 8).
+constexpr int kAhead3 = 8;
+
+// Pass 1 of the warp's rows: f~ into fo, the sums of (1, k_x, k_x^2,
+// k_y, k_y^2, k_z, k_z^2) f~ into sums.  eg: largest exponent the units are
+// cut for; on return the largest seen.  False when the sums are not valid.
+__device__ __forceinline__ bool stream3v_fixed(const Params3v& P, const Tables3v& T, const double* __restrict__ fin,
+                                               double* __restrict__ fo, int i, int& eg, double* sums) {
+  const Map3v L(P);
+  const int nvx = P.nvx, nvy = P.nvy, nvz = P.nvz;
+  const fx::i96 zero = {0u, 0u, 0u};
+  double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  int top = 0;
+  unsigned over = 0;
+#pragma unroll 1
+  for (int jl = L.l; jl - L.l < nvx; jl += L.width) {
+    const bool in = jl < nvx;
+    const int jx = in ? jl : nvx - 1;  // a column past the row repeats its last one and is not counted
+    const int i1 = i - T.shift[jx];
+    const double* p1 = column_source(P, T, fin, i1);
+    const double* p2 = column_source(P, T, fin, i1 - T.upwind[jx]);
+    const double rem = T.rem[jx];
+    fx::i96 n0 = zero, y1 = zero, y2 = zero, z1 = zero, z2 = zero;
+#pragma unroll 1
+    for (int kz = 0; kz < L.zrows; ++kz) {
+      const int jz = L.z0 + kz * L.zstep;
+      const bool zin = in && jz < nvz;
+      const int jb = min(jz, nvz - 1) * nvy * nvx + jx;
+      fx::i96 t1 = zero, t2 = zero, t3 = zero;
+#pragma unroll 1
+      for (int k0 = 0; k0 < L.yrows; k0 += kAhead3) {
+        double f1[kAhead3], f2[kAhead3];
+#pragma unroll
+        for (int u = 0; u < kAhead3; ++u) {
+          const int j = jb + min(L.y0 + (k0 + u) * L.ystep, nvy - 1) * nvx;
+          f1[u] = p1[j];
+          f2[u] = p2[j];
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead3; ++u) {
+          const int jy = L.y0 + (k0 + u) * L.ystep;
+          const double ft = fma(rem, f2[u] - f1[u], f1[u]);
+          if (zin && jy < nvy) {
+            const unsigned hi = (unsigned)__double2hiint(ft);
+            fo[jb + jy * nvx] = ft;
+            top = max(top, (int)(hi >> 20));
+            t1 = fx::add(t1, fx::double_to_units96(hi, (unsigned)__double2loint(ft), (unsigned)eg));
+          }
+          if (k0 + u < L.yrows) {
+            t2 = fx::add(t2, t1);
+            t3 = fx::add(t3, t2);
+          }
+        }
+      }
+      n0 = fx::add(n0, t1);
+      y1 = fx::add(y1, t2);
+      y2 = fx::add(y2, t3);
+      z1 = fx::add(z1, n0);
+      z2 = fx::add(z2, z1);
+    }
+    over |= n0.a2 >> 16;  // 2^12 rows of 2^75 do not wrap; below 2^80 the squared indices fit too
+    fx::i96 a1, a2, b1, b2;
+    axis_weights(n0, y1, y2, L.y0, L.ystep, L.yrows, nvy, a1, a2);
+    axis_weights(n0, z1, z2, L.z0, L.zstep, L.zrows, nvz, b1, b2);
+    const double sn = unit_value(n0, eg - 16), kx = (double)(2 * jx + 1 - nvx), kn = kx * sn;
+    v[0] += sn;
+    v[1] += kn;
+    v[2] = fma(kx, kn, v[2]);
+    v[3] += unit_value(a1, eg - 16);
+    v[4] += unit_value(a2, eg - 16);
+    v[5] += unit_value(b1, eg - 16);
+    v[6] += unit_value(b2, eg - 16);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  const bool valid = top <= eg && !__any_sync(0xffffffffu, over != 0);
+  const int lane = threadIdx.x & 31;
+  const double t = warp_reduce8(v);  // lane 4 k + r holds total k
+  if ((lane & 3) == 0) sums[lane >> 2] = t;
+  eg = top;
+  return valid;
+}
+
+// Largest exponent of the cell's own state along the x lines through the
+// middle of the (y, z) box, plus the headroom: the peak of a flow along x
+// with little transverse motion lies there.
+__device__ __forceinline__ int sample3v(const Params3v& P, const double* __restrict__ f) {
+  const int lane = threadIdx.x & 31;
+  unsigned m = 0;
+  for (int jx = lane; jx < P.nvx; jx += 32) {
+    const int j = ((P.nvz >> 1) * P.nvy + (P.nvy >> 1)) * P.nvx + jx;
+    const int k = ((max(P.nvz - 1, 0) >> 1) * P.nvy + (max(P.nvy - 1, 0) >> 1)) * P.nvx + jx;
+    m = max(m, max((unsigned)__double2hiint(f[j]), (unsigned)__double2hiint(f[k])));
+  }
+  return (int)((__reduce_max_sync(0xffffffffu, m) >> 20) + fx::kHeadroom);
+}
+
+// Warps 0 to 2 (an axis each) and 3 (the relaxation weight).
+__device__ __forceinline__ void bar_solve() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
+
+// The cell's parameters on warps 0 to 3, from the totals in S.tot.  Leaves
+// S.ok, S.ab, the factors in fac and returns true, or false (S.ok = -1) when
+// the cell needs FP64.
+__device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v& S, double* fac,
+                                              double* __restrict__ mom, int* __restrict__ err) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n3[3] = {P.nvx, P.nvy, P.nvz};
+  double half[3], mid[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    half[a] = P.half[a];
+    mid[a] = P.mid[a];
+  }
+  double q[5], p[5], ith = 1.0, isq = 1.0, iq0 = 1.0, iq4 = 1.0, ivs = 1.0;
+  bool ok = false, conv = true, fail = false;
+  if (warp == 0) {  // all lanes alike
+    const double* t = S.tot;
+    bool fit = in_range(t[0]);
+    const double in = rcp3(fit ? t[0] : 1.0);
+    q[0] = t[0] * P.dv;
+    double e = 0.0, uu = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const double m1 = half[a] * t[1 + 2 * a] * in;  // mean of c - mid
+      const double u = mid[a] + m1;
+      q[1 + a] = u;
+      // mean of c^2 less u^2, both about mid
+      e += fma(half[a] * half[a], t[2 + 2 * a] * in, -m1 * m1);
+      uu += u;
+    }
+    q[4] = (2.0 / 3.0) * e;
+    ok = q[0] > 0.0 && q[4] > 0.0 && isfinite(q[0]) && isfinite(q[4]) && isfinite(uu);
+    fit = fit && ok && in_range(q[0]) && in_range(q[4]);
+    if (fit) {
+      ivs = isq = rsqrt3(q[4]);
+      iq4 = ith = isq * isq;
+      iq0 = rcp3(q[0]);
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) p[k] = fit ? q[k] : (k == 0 || k == 4) ? 1.0 : 0.0;
+    if (fit) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        AxisBase B;
+        fit = axis_base(n3[a], half[a], P.inv_half[a], mid[a], p[1 + a], isq * 1.2011224087864498, B) && fit;
+        if (lane == 0) S.base[a] = B;
+      }
+    }
+    conv = P.conservative == 0;
+    if (lane == 0) {
+      S.go = !fit ? -1 : conv ? 0 : 1;
+      S.tot[7] = q[4];
+    }
+  }
+  bar_solve();
+  if (S.go < 0) return;
+  if (warp == 3) {  // nu = n theta^(1 - omega), the weights
+    const double x = S.tot[0] * P.dv * pow_fixed(S.tot[7], 1.0 - P.omega) * P.dt;  // nu dt
+    const double b = P.relax_exact ? exp_neg_fixed(x) : 1.0 - x;
+    if (lane == 0) {
+      S.ab[0] = P.relax_exact ? 1.0 - b : x;
+      S.ab[1] = b;
+    }
+  }
+  int it = 0;
+  while (S.go > 0) {
+    if (warp < 3) {
+      const double t = axis_index_sums<32>(n3[warp], S.base[warp], lane);
+      if (lane < 3) S.ax[warp][lane] = t;
+    }
+    bar_solve();
+    if (warp == 0) {
+      ++it;
+      double M[3][3], d[5];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) central_sums(S.ax[a], S.base[a].k0, half[a], mid[a], p[1 + a], M[a]);
+      const double pi15 = 5.568327996831708;  // pi^(3/2)
+      d[0] = p[0] * (ith * isq) * (P.dv / pi15) * (M[0][0] * M[1][0] * M[2][0]);
+      double var = 0.0;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const double r = rcp3(M[a][0]), mu = M[a][1] * r;
+        d[1 + a] = p[1 + a] + mu;
+        var += fma(M[a][2], r, -mu * mu);
+      }
+      d[4] = (2.0 / 3.0) * var;
+      unsigned r = 0;  // high word of the largest scaled update
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const double delta = q[k] - d[k];
+        p[k] += delta;
+        r = max(r, abs_hi(delta * (k == 0 ? iq0 : k == 4 ? iq4 : ivs)));
+      }
+      // the high words of kEffTol = 1e-13 and kEffFail = 1e-9 (no early stop: on
+      // coarse grids, 16^3 on the paper's box, the contraction is 20 times the
+      // first update, and the skipped one would show at 1e-14)
+      if (!in_range(p[0]) || !in_range(p[4]) || r >= 0x7ff00000u) fail = true;
+      else if (r < 0x3d3c25c2u) conv = true;
+      else if (it >= kEffMaxIt) (r < 0x3e112e0bu ? conv : fail) = true;
+      bool fit = true;
+      if (!fail) {
+        isq = rsqrt3(p[4]);
+        ith = isq * isq;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          AxisBase B;
+          fit = axis_base(n3[a], half[a], P.inv_half[a], mid[a], p[1 + a], isq * 1.2011224087864498, B) && fit;
+          if (lane == 0) S.base[a] = B;
+        }
+      }
+      if (lane == 0) S.go = !fit ? -1 : conv || fail ? 0 : 1;
+    }
+    bar_solve();
+  }
+  if (S.go < 0) return;
+  bar_solve();  // the weights of warp 3, when there was no round
+  if (warp == 0) {
+    if (fail) ok = false;
+    if (lane == 0) {
+      S.ok = ok ? 1 : 0;
+      S.tot[6] = S.ab[0] * p[0] * (ith * isq) * (1.0 / 5.568327996831708);
+      for (int k = 0; k < 5; ++k) mom[(size_t)i * 5 + k] = q[k];
+      if (!ok) atomicOr(err, fail ? ERR_EFFECTIVE : ERR_MOMENT);
+    }
+  }
+  bar_solve();
+  if (warp < 3) {
+    const AxisBase B = S.base[warp];
+    const double scale = warp == 0 ? S.tot[6] : 1.0;
+    double* fw = fac + (warp == 0 ? 0 : warp == 1 ? P.nvx : P.nvx + P.nvy);
+    for (int j = lane; j < n3[warp]; j += 32) {
+      unsigned q2, hi, lo;
+      const unsigned long long g = fx::gauss(B.a * (2 * j + 1 - n3[warp]) - B.c, (const fx::u64*)kExp2, q2);
+      fx::gauss_words(g, q2, hi, lo);
+      fw[j] = scale * __hiloint2double((int)hi, (int)lo);
+    }
+  }
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kT, 4) step3v_fixed_kernel(const Params3v P, const Tables3v T,
+                                                             const double* __restrict__ fin, double* __restrict__ fout,
+                                                             double* __restrict__ mom, int* __restrict__ err) {
+  extern __shared__ double fac[];  // px[nvx], py[nvy], pz[nvz]
+  __shared__ Shared3v S;
+  const int i = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* fo = fout + (size_t)i * P.nv;
+  bool valid = false;
+  int eg = sample3v(P, fin + (size_t)i * P.nv);
+  // a second pass takes the largest exponent of the first as its range
+  for (int pass = 0; pass < 2 && !valid; ++pass) {
+    if (eg < (int)fx::kExpMin || eg > (int)fx::kExpMax) break;
+    valid = stream3v_fixed(P, T, fin, fo, i, eg, S.red + warp * 8);
+  }
+  if (lane == 0) S.valid[warp] = valid ? 1 : 0;
+  __syncthreads();
+  bool all = true;
+  for (int w = 0; w < kW; ++w) all = all && S.valid[w];
+  if (all) {
+    if (warp == 0) {
+      double t = 0.0;
+      if (lane < 7)
+        for (int w = 0; w < kW; ++w) t += S.red[w * 8 + lane];
+      if (lane < 7) S.tot[lane] = t;
+      __syncwarp();
+    }
+    if (warp < 4) solve3v_fixed(P, i, S, fac, mom, err);
+    __syncthreads();
+    all = S.go >= 0;
+  }
+  if (!all) {
+    __syncthreads();
+    cell3v_f64(P, T, fin, fout, mom, err, i, fac, S);
+    return;
+  }
+  if (!S.ok) return;  // a failed cell keeps f~ (flagged)
+  // pass 2: f^{n+1} = b f~ + a Phi on the rows of pass 1
+  const Map3v L(P);
+  const int nvx = P.nvx, nvy = P.nvy, ys = L.ystep * nvx;
+  const double b = S.ab[1];
+  const double *py = fac + nvx, *pz = py + nvy;
+#pragma unroll 1
+  for (int jx = L.l; jx < nvx; jx += L.width) {
+    const double x = fac[jx];
+#pragma unroll 1
+    for (int jz = L.z0; jz < P.nvz; jz += L.zstep) {
+      const double xz = x * pz[jz];
+      double* p = fo + (jz * nvy + L.y0) * nvx + jx;
+#pragma unroll 1
+      for (int jy = L.y0; jy < nvy; jy += kAhead3 * L.ystep, p += kAhead3 * ys) {
+        double ft[kAhead3];
+#pragma unroll
+        for (int u = 0; u < kAhead3; ++u) ft[u] = jy + u * L.ystep < nvy ? p[u * ys] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kAhead3; ++u)
+          if (jy + u * L.ystep < nvy) p[u * ys] = fma(b, ft[u], xz * py[jy + u * L.ystep]);
+      }
+    }
   }
 }
 
@@ -292,10 +656,39 @@ cudaError_t launch_init3v(const Params3v& P, const Tables3v& T, double x_split, 
   return cudaGetLastError();
 }
 
+// Lanes per row and warps along z that leave the fewest lanes idle (more
+// lanes per row, then more warps along z, on a tie).  The fixed-point kernel
+// takes at most 64 velocities per axis (its squared indices and sums then stay
+// within 95 bits).
+void plan3v(Params3v& P) {
+  const int n3[3] = {P.nvx, P.nvy, P.nvz};
+  for (int a = 0; a < 3; ++a) {
+    P.half[a] = 0.5 * P.dc[a];
+    P.inv_half[a] = 1.0 / P.half[a];
+    P.mid[a] = P.vmin[a] + n3[a] * P.half[a];
+  }
+  P.lane_bits = P.zw_bits = 0;
+  if (P.nvx > 64 || P.nvy > 64 || P.nvz > 64) return;
+  double best = 0.0;
+  for (int lb = 5; lb >= 2; --lb)
+    for (int zb = 3; zb >= 0; --zb) {
+      const int lw = 1 << lb, ys = (kW >> zb) * (32 >> lb), zs = 1 << zb;
+      const double width = (P.nvx + lw - 1) / lw * lw, y = (P.nvy + ys - 1) / ys * ys, z = (P.nvz + zs - 1) / zs * zs;
+      const double use = (double)P.nv / (width * y * z);
+      if (use > best + 1e-9) {
+        best = use;
+        P.lane_bits = lb;
+        P.zw_bits = zb;
+      }
+    }
+  if (best < 0.5) P.lane_bits = 0;
+}
+
 cudaError_t launch_step3v(const Params3v& P, const Tables3v& T, const double* fin, double* fout, double* mom,
                           int* err, cudaStream_t stream) {
   const size_t smem = sizeof(double) * (size_t)(P.nvx + P.nvy + P.nvz);
-  step3v_kernel<<<P.nx, kT, smem, stream>>>(P, T, fin, fout, mom, err);
+  if (P.lane_bits) step3v_fixed_kernel<<<P.nx, kT, smem, stream>>>(P, T, fin, fout, mom, err);
+  else step3v_kernel<<<P.nx, kT, smem, stream>>>(P, T, fin, fout, mom, err);
   return cudaGetLastError();
 }
 

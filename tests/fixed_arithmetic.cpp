@@ -25,7 +25,7 @@ static const u64 kTable[32] = BGK_EXP2_TABLE;
 int main() {
   std::mt19937_64 g(1);
   std::uniform_real_distribution<double> U(0, 1);
-  long double worst[5] = {0, 0, 0, 0, 0};
+  long double worst[6] = {0, 0, 0, 0, 0, 0};
   auto keep = [&](int k, long double got, long double want) {
     worst[k] = std::fmax(worst[k], std::fabs((got - want) / want));
   };
@@ -46,6 +46,10 @@ int main() {
     // units: at most half of one off
     const long double unit = std::ldexp(1.0L, (int)(em + 2) - 1081);
     worst[1] = std::fmax(worst[1], std::fabs(double_to_units(hi, lo, em + 2) - value(hi, lo) / unit));
+    const u32 up = em + 2 + (u32)(40 * U(g));
+    const i96 w96 = double_to_units96(hi, lo, up);
+    const long double fine = std::ldexp(1.0L, (int)up - 1097), v96 = ((long double)w96.a2 * 0x1p32L + w96.a1) * 0x1p32L + w96.a0;
+    worst[5] = std::fmax(worst[5], std::fabs(v96 - std::floor(value(hi, lo) / fine)));
     // Gaussian and relaxation
     const double x = 8 * (2 * U(g) - 1), y = 8 * (2 * U(g) - 1);
     words(x, a, b);
