@@ -239,7 +239,6 @@ bgk_status validate(const bgk_config* c, bgk::Params* P, double* max_courant) {
     p.dt = c->cfl / (mx / p.dx + my / p.dy);
   }
   *max_courant = c->dim == 1 ? mx * p.dt / p.dx : mx * p.dt / p.dx + my * p.dt / p.dy;
-  if (c->dim == 2 && c->precision == BGK_F64) bgk::step_f64_plan(p, *max_courant);
 
   // cells per CTA: the caller's choice (checked here), else chosen in
   // bgk_create once the device's SM count is known
@@ -292,6 +291,7 @@ bgk_status validate(const bgk_config* c, bgk::Params* P, double* max_courant) {
         return fail(BGK_ERR_INVALID_ARG, "face %d: unknown boundary kind %d", face, b.kind);
     }
   }
+  if (c->precision == BGK_F64) bgk::step_f64_plan(p, *max_courant);
   if (c->dim == 2 && *max_courant > 1.0 + 1e-12)
     return fail(BGK_ERR_UNSUPPORTED, "2D donor cell needs (max|cx|/dx + max|cy|/dy) dt <= 1 (got %.6g)",
                 *max_courant);

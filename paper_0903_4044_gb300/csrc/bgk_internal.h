@@ -32,8 +32,8 @@ struct Params {
   int dim, nx, ny, nvx, nvy, nv;
   int tile;  // spatial cells per CTA of the step kernel (1, 2, 4 or 8)
   int mgl;   // reduced precisions: groups of 4 velocities per lane (2, 4 or 6)
-  int lane_bits;  // FP64 2D: log2 of the lanes per velocity row of the fixed-point step
-                  // (step_f64_plan); 0: FP64 loop
+  int lane_bits;  // FP64: log2 of the lanes per velocity row of the fixed-point step
+                  // (step_f64_plan); 0: FP64-only form
   int conservative, relax_exact;
   int bc_kind[kFaces];
   double dt, dx, dy, dcx, dcy, dv;
@@ -42,7 +42,7 @@ struct Params {
   double bc_state[kFaces][4];  // n, ux, uy, theta
 };
 
-// Numbers of the velocity grid that the fixed-point step uses (2D FP64).
+// Numbers of the velocity grid that the fixed-point step uses (FP64).
 struct VelocityGrid {
   double half_x, half_y, inv_half_x, inv_half_y;  // half velocity steps and their reciprocals
   double mid_x, mid_y, dv_pi;                     // box centres, dv / pi
@@ -105,7 +105,7 @@ cudaError_t launch_step_f64(const Params& P, const Tables& T, const double2* fin
 cudaError_t launch_build_tables(const Params& P, double* cx, double* cy, double4_32a* coef, int* shift,
                                 double2* cxy, int* vinfo, double2* ghost, double* emitted, uint64_t* wx,
                                 uint64_t* wy, double* sx, double2* ratio, cudaStream_t stream);
-// Fills P.lane_bits (2D FP64) from the grid and the Courant number.
+// Fills P.lane_bits (FP64) from the grid, the boundaries and the Courant number.
 void step_f64_plan(Params& P, double max_courant);
 size_t step_f64_smem_bytes(const Params& P, int tile);
 cudaError_t prepare_step_f64(const Params& P);

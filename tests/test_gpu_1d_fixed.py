@@ -1,0 +1,87 @@
+"""The 1D FP64 step that keeps a cell on one warp against the FP64 CPU oracle:
+every number of velocities per lane and its remainders, grids it leaves to the
+FP64-only kernel, shifts, options, and states out of its range.  Tolerances as
+in test_gpu_fixed.py."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0903_4044_gb300 import bgk as B
+from paper_0903_4044_gb300 import build, solver
+from paper_0903_4044_gb300 import workloads as W
+from test_gpu_parity import assert_moments_close, assert_state_close
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    oracle.build()
+    B.lib()
+
+
+def pair(**over):
+    w = W.scaled(W.SHOCK_M2, **{**dict(nx=23, length=8.0), **over})
+    s = solver.make_shock(w)
+    prob, g, h = oracle.shock_problem(**w)
+    rng = np.random.default_rng(2)
+    return s, prob, g * (1.0 + 0.01 * rng.uniform(-1, 1, g.shape)), h * (1.0 + 0.01 * rng.uniform(-1, 1, h.shape))
+
+
+def run(s, prob, g, h, steps=3):
+    s.set_state(np.ascontiguousarray(np.stack([g, h], -1)))
+    s.step(steps)
+    g1, h1, mom = oracle.step(prob, g, h, steps)
+    return s.get_state(), s.moments(which=1), g1, h1, mom
+
+
+@pytest.mark.parametrize("nvx,vbox", [(24, 6.0), (31, 6.0), (32, 6.0), (33, 7.0), (64, 8.0), (65, 8.0), (97, 9.0), (128, 9.0),
+                                      (129, 10.0), (160, 10.0), (161, 10.0), (200, 10.0)])
+def test_velocity_counts(nvx, vbox):
+    s, prob, g, h = pair(nvx=nvx, vx=(-vbox, vbox + 1.0), tile_cells=(1, 2, 4, 8)[nvx % 4])
+    st, m, g1, h1, mom = run(s, prob, g, h)
+    assert_state_close(st, g1, h1)
+    assert_moments_close(m, mom, vscale=1.0)
+    s.close()
+
+
+@pytest.mark.parametrize("over", [dict(cfl=2.6), dict(omega=0.74), dict(omega=0.74, mach=5.0, nvx=96, vx=(-19.0, 19.0)),
+                                  dict(conservative=0), dict(relax_exact=0), dict(nx=1), dict(length=4000.0)])
+def test_options(over):
+    s, prob, g, h = pair(**over)
+    st, m, g1, h1, mom = run(s, prob, g, h)
+    if "length" in over or "mach" in over:
+        # the effective parameters stop within 1e-13 of each other and a value
+        # moves |c - U|^2 / theta times as much (64 and 555 at the box's end)
+        bound = 7e-12 if "length" in over else 6e-11
+        assert (np.abs(st[..., 0] - g1) <= bound * np.abs(g1)).all()
+    else:
+        assert_state_close(st, g1, h1)
+    assert_moments_close(m, mom, vscale=1.0)
+    s.close()
+
+
+@pytest.mark.parametrize("what", ["negative", "zero", "front", "scale"])
+def test_states_out_of_range(what):
+    s, prob, g, h = pair(conservative=0)
+    j = np.arange(prob.nv)
+    if what == "negative":
+        g[9, j % 13 == 0] *= -0.01
+        h[12, j % 7 == 0] *= -0.01
+    elif what == "zero":
+        g[9, j % 3 == 0] = 0.0
+        h[13] = 0.0
+    elif what == "front":
+        g[12:] *= 1e9
+        h[12:] *= 1e9
+    else:
+        g[8:15] *= 1e60
+        h[8:15] *= 1e60
+    st, m, g1, h1, mom = run(s, prob, g, h, 1)
+    for a, b in ((st[..., 0], g1), (st[..., 1], h1)):
+        assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
+        if what != "negative":
+            assert (np.abs(a - b) <= 1e-12 * np.abs(b)).all()
+    assert_moments_close(m, mom, vscale=1.0)
+    s.close()
