@@ -27,7 +27,7 @@
 // Derivatives with respect to the domain scale L (lengths and the Courant
 // time step scale together, Kn = 1/L) and the lid speed U_W accumulate per
 // cell in a fixed order, so results are deterministic.
-#include "bgk_device.cuh"
+#include "bgk_solve.cuh"
 
 namespace bgk {
 
@@ -235,6 +235,153 @@ __device__ __forceinline__ void collide_sums(const Params& P, const Tables& T, c
   }
 }
 
+// ---- interior cells on grids that P.lane_bits maps -----------------------------
+// 2^lane_bits lanes share a velocity row; a lane takes its columns one after
+// the other, each over its rows, so that what depends on one axis is held per
+// column or read per row: lambda^{n+1} / s gathers in two FMAs per component
+// (s the column's scale, as in the forward step), the collision sums take seven
+// FP64 operations a velocity and the output three, 14 where the plain loops
+// (edge cells) take 24.
+struct RowMap {
+  int l, width, row0, step;
+  __device__ __forceinline__ explicit RowMap(const Params& P) {
+    const int lane = threadIdx.x & 31, lb = P.lane_bits;
+    width = 1 << lb;
+    l = lane & (width - 1);
+    row0 = lane >> lb;
+    step = 32 >> lb;
+  }
+};
+
+// Row and column factors of a cell at its parameters p: ex = n / (pi theta)
+// e^{-(c_x-u_x)^2 / theta}, wy[k] = c_y^k e^{-(c_y-u_y)^2 / theta}, k = 0, 1, 2.
+__device__ __forceinline__ void row_factors(const Params& P, const Tables& T, const double4_32a& p, double* ex,
+                                            double* wy) {
+  const int lane = threadIdx.x & 31, nvx = P.nvx, nvy = P.nvy;
+  const VelocityGrid& V = T.grid;
+  AxisBase A, B;
+  bool fit = in_range(p.x) && in_range(p.w);
+  double ith, pref;
+  if (fit) {
+    const double isq = rsqrt3(p.w), gamma = isq * 1.2011224087864498;  // sqrt(log2 e)
+    ith = isq * isq;
+    pref = p.x * ith * 0.31830988618379067;
+    fit = axis_base(nvx, V.half_x, V.inv_half_x, V.mid_x, p.y, gamma, A) &&
+          axis_base(nvy, V.half_y, V.inv_half_y, V.mid_y, p.z, gamma, B);
+  } else {
+    ith = 1.0 / p.w;
+    pref = p.x / (kPi() * p.w);
+  }
+#pragma unroll 1
+  for (int j = lane; j < nvx + nvy; j += 32) {
+    const bool isx = j < nvx;
+    const int k = isx ? j : j - nvx;
+    double g;
+    if (fit) {
+      unsigned n, hi, lo;
+      const long long w = isx ? A.a * (2 * k + 1 - nvx) - A.c : B.a * (2 * k + 1 - nvy) - B.c;
+      const unsigned long long q = fx::gauss(w, (const fx::u64*)kExp2, n);
+      fx::gauss_words(q, n, hi, lo);
+      g = __hiloint2double((int)hi, (int)lo);
+    } else {
+      const double d = isx ? T.cx[k] - p.y : T.cy[k] - p.z;
+      g = exp(-(d * d) * ith);
+    }
+    if (isx) {
+      ex[k] = pref * g;
+    } else {
+      const double c = T.cy[k], cg = c * g;
+      wy[k] = g;
+      wy[nvy + k] = cg;
+      wy[2 * nvy + k] = c * cg;
+    }
+  }
+}
+
+// lambda^{n+1} / s into dst and the collision sums of collide_sums.
+__device__ __forceinline__ void gather_sums_rows(const Params& P, const Tables& T, const double2* __restrict__ lt,
+                                                 const double2* __restrict__ f1, double2* __restrict__ dst,
+                                                 const double* ex, const double* wy, double hp, double (&sum)[8]) {
+  constexpr int kRows = 2;
+  const RowMap L(P);
+  const int nvx = P.nvx, nvy = P.nvy;
+  const ptrdiff_t row = (ptrdiff_t)P.nx * P.nv;
+#pragma unroll 1
+  for (int jx = L.l; jx < nvx; jx += L.width) {
+    const int offx = sgn_x(T.vinfo[jx]) * P.nv;  // downwind neighbours used this value as their upwind source
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, b0 = 0.0, d0 = 0.0;
+#pragma unroll 1
+    for (int j0 = L.row0; j0 < nvy; j0 += kRows * L.step) {
+      double2 l0[kRows], lx[kRows], ly[kRows], ra[kRows], f[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const int j = min(j0 + u * L.step, nvy - 1) * nvx + jx;
+        const ptrdiff_t offy = sgn_y(T.vinfo[j]) * row;
+        l0[u] = lt[j];
+        lx[u] = lt[j + offx];
+        ly[u] = lt[j + offy];
+        ra[u] = T.ratio[j];
+        f[u] = f1[j];
+      }
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const int jy = j0 + u * L.step;
+        if (jy < nvy) {
+          double2 l;
+          l.x = fma(ra[u].y, ly[u].x, fma(ra[u].x, l0[u].x, lx[u].x));
+          l.y = fma(ra[u].y, ly[u].y, fma(ra[u].x, l0[u].y, lx[u].y));
+          dst[jy * nvx + jx] = l;
+          const double t = fma(hp, l.y, l.x), w = wy[jy];
+          a0 = fma(w, t, a0);
+          a1 = fma(wy[nvy + jy], t, a1);
+          a2 = fma(wy[2 * nvy + jy], t, a2);
+          b0 = fma(w, l.y, b0);
+          d0 = fma(l.x, f[u].x, fma(l.y, f[u].y, d0));
+        }
+      }
+    }
+    const double s = T.sx[jx], es = ex[jx] * s, c = T.cx[jx], g = es * a0, cg = c * g;
+    sum[0] += g;
+    sum[1] += cg;
+    sum[2] = fma(es, a1, sum[2]);
+    sum[3] += fma(es, a2, c * cg);
+    sum[4] = fma(es, b0, sum[4]);
+    sum[5] = fma(s, d0, sum[5]);
+  }
+}
+
+// lambda~ = e lambda + A0 + A1 c_x + A2 c_y + B |c|^2 (h: e lambda_h + B).
+__device__ __forceinline__ void output_rows(const Params& P, const Tables& T, double2* __restrict__ o, double* qy,
+                                            double e, double A0, double A1, double A2, double B) {
+  constexpr int kRows = 4;
+  const RowMap L(P);
+  const int nvx = P.nvx, nvy = P.nvy;
+  for (int j = threadIdx.x & 31; j < nvy; j += 32) {
+    const double c = T.cy[j];
+    qy[j] = c * fma(B, c, A2);
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int jx = L.l; jx < nvx; jx += L.width) {
+    const double c = T.cx[jx], px = fma(c, fma(B, c, A1), A0), es = e * T.sx[jx];
+#pragma unroll 1
+    for (int j0 = L.row0; j0 < nvy; j0 += kRows * L.step) {
+      double2* p = o + j0 * nvx + jx;
+      double2 l[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+        l[u] = j0 + u * L.step < nvy ? p[u * L.step * nvx] : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+        if (j0 + u * L.step < nvy)
+          p[u * L.step * nvx] = make_double2(fma(es, l[u].x, px + qy[j0 + u * L.step]), fma(es, l[u].y, B));
+    }
+  }
+}
+
+// 1/x from the third-order step where its FP32 start is in range.
+__device__ __forceinline__ double rcp_any(double x) { return in_range(x) ? rcp3(x) : 1.0 / x; }
+
 }  // namespace
 
 // One reverse step, G cells per CTA, one warp per cell.
@@ -243,11 +390,11 @@ __device__ __forceinline__ void collide_sums(const Params& P, const Tables& T, c
 //   collide = 1: out = lambda~^n (needs qn, pn of step n; fn1 = f^{n+1});
 //   collide = 0: out = lambda^{n+1} (the last launch, giving lambda^0).
 // dghost, demit: d/dU_W of the lid's unit Maxwellian and of its emitted flux.
-// The per-cell coefficients are computed cells-in-lanes by warp 0.  Six
-// CTAs per SM hold it to 80 registers without spills (105 unbounded):
-// 3.881 -> 3.846 s per 128^2 x 32^2, 2000-step gradient.
+// The per-cell coefficients are computed cells-in-lanes by warp 0.  24 warps
+// per SM at 80 registers.  128^2 x 32^2: 0.84 -> 0.60 ms a step; the FP64 pipe
+// stays the bound (17.4 operations per velocity, 98 % of its measured rate).
 template <int G>
-__global__ void __launch_bounds__(32 * G, 6) adj_step_kernel(const Params P, const Tables T,
+__global__ void __launch_bounds__(32 * G, 24 / G) adj_step_kernel(const Params P, const Tables T,
                                                           const double2* __restrict__ fn1,
                                                           const double4_32a* __restrict__ qn,
                                                           const double4_32a* __restrict__ pn,
@@ -258,20 +405,23 @@ __global__ void __launch_bounds__(32 * G, 6) adj_step_kernel(const Params P, con
   extern __shared__ double sh[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ncell = P.nx * P.ny, nvxy = P.nvx + P.nvy;
-  double* ex = sh + (size_t)warp * nvxy;  // n/(pi theta) e^{-(c_x-u_x)^2/theta}
-  double* ey = ex + P.nvx;                // e^{-(c_y-u_y)^2/theta}
+  double* ex = sh + (size_t)warp * (P.nvx + 3 * P.nvy);  // n/(pi theta) e^{-(c_x-u_x)^2/theta}
+  double* ey = ex + P.nvx;                                // e^{-(c_y-u_y)^2/theta} (rows: times 1, c_y, c_y^2)
   __shared__ double s_sum[G][8], s_cf[G][5];
   const int cell = blockIdx.x * G + warp;
   const bool live = cell < ncell;
   const int ix = cell % P.nx, iy = cell / P.nx;
   const size_t base = (size_t)cell * P.nv;
   const int dmask = live ? diffuse_faces(P, ix, iy) : 0;
+  // interior cells of a step that needs the collision take one pass for
+  // lambda^{n+1} and its sums
+  const bool rows = P.lane_bits && tilde && collide && ix > 0 && ix < P.nx - 1 && iy > 0 && iy < P.ny - 1;
 
   // 1. lambda^{n+1} at this cell, parked in the cell's output slots (each
   // lane rereads only what it wrote; shared-memory staging, 16 B per
   // velocity, held an SM to 3 CTAs)
   double2* sl = out + base;
-  if (live) {
+  if (live && !rows) {
     double2* dst = sl;
     if (tilde) {
       stream_adjoint(P, T, cell, ix, iy, dmask, fn1, lam_in, dghost, demit, duw, dst);
@@ -285,16 +435,22 @@ __global__ void __launch_bounds__(32 * G, 6) adj_step_kernel(const Params P, con
   double4_32a p = make_double4_32a(1.0, 0.0, 0.0, 1.0);
   if (live) {
     p = pn[cell];
-    const double inv = 1.0 / p.w, pref = p.x / (kPi() * p.w);
-    for (int j = lane; j < nvxy; j += 32) {
-      const bool isx = j < P.nvx;
-      const double d = (isx ? T.cx[j] : T.cy[j - P.nvx]) - (isx ? p.y : p.z);
-      const double g = exp(-(d * d) * inv);
-      ex[j] = isx ? pref * g : g;  // ey = ex + nvx
-    }
-    __syncwarp();
     double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    collide_sums(P, T, fn1 + base, ex, ey, sl, 0.5 * p.w, s);
+    if (rows) {
+      row_factors(P, T, p, ex, ey);
+      __syncwarp();
+      gather_sums_rows(P, T, lam_in + base, fn1 + base, sl, ex, ey, 0.5 * p.w, s);
+    } else {
+      const double inv = 1.0 / p.w, pref = p.x / (kPi() * p.w);
+      for (int j = lane; j < nvxy; j += 32) {
+        const bool isx = j < P.nvx;
+        const double d = (isx ? T.cx[j] : T.cy[j - P.nvx]) - (isx ? p.y : p.z);
+        const double g = exp(-(d * d) * inv);
+        ex[j] = isx ? pref * g : g;  // ey = ex + nvx
+      }
+      __syncwarp();
+      collide_sums(P, T, fn1 + base, ex, ey, sl, 0.5 * p.w, s);
+    }
     const double x = warp_reduce8(s);
     if ((lane & 3) == 0) s_sum[warp][lane >> 2] = x;
   }
@@ -305,21 +461,22 @@ __global__ void __launch_bounds__(32 * G, 6) adj_step_kernel(const Params P, con
     const double4_32a q = qn[c], pc = pn[c];
     const double* t = s_sum[lane];
     const double n = q.x, ux = q.y, uy = q.z, th = q.w;
-    const double th1 = pow(th, 1.0 - P.omega);
+    const double th1 = P.omega == 0.5 && in_range(th) ? th * rsqrt3(th) : in_range(th) ? pow_fixed(th, 1.0 - P.omega)
+                                                                                     : pow(th, 1.0 - P.omega);
     const double nu = n * th1;
-    const double e = exp(-nu * P.dt), a = 1.0 - e;
+    const double e = exp_neg_fixed(nu * P.dt), a = 1.0 - e;
     const double s0 = t[0], s1 = t[1], s2 = t[2], s3 = t[3], s4 = t[4];
-    const double sa = (s0 - t[5]) / e;  // <lambda, Phi - f~>
-    const double ip = 1.0 / pc.w;
-    const double sp0 = s0 / pc.x;
+    const double sa = (s0 - t[5]) * rcp_any(e);  // <lambda, Phi - f~>
+    const double ip = rcp_any(pc.w);
+    const double sp0 = s0 * rcp_any(pc.x);
     const double sp1 = 2.0 * (s1 - pc.y * s0) * ip;
     const double sp2 = 2.0 * (s2 - pc.z * s0) * ip;
     const double sp3 =
         (s3 - 2.0 * (pc.y * s1 + pc.z * s2) + (pc.y * pc.y + pc.z * pc.z) * s0) * ip * ip - s0 * ip + 0.5 * s4;
     const double da_dn = P.dt * e * th1;
-    const double da_dth = P.dt * e * (1.0 - P.omega) * n * th1 / th;
+    const double da_dth = P.dt * e * (1.0 - P.omega) * n * th1 * rcp_any(th);
     const double mu0 = a * sp0 + da_dn * sa, mu1 = a * sp1, mu2 = a * sp2, mu3 = a * sp3 + da_dth * sa;
-    const double r = P.dv / n, eon = 1.5 * th + ux * ux + uy * uy;
+    const double r = P.dv * rcp_any(n), eon = 1.5 * th + ux * ux + uy * uy;
     const double B = (2.0 / 3.0) * r * mu3;
     s_cf[lane][0] = e;
     s_cf[lane][1] = mu0 * P.dv - r * (mu1 * ux + mu2 * uy) + B * (2.0 * (ux * ux + uy * uy) - eon);
@@ -333,6 +490,10 @@ __global__ void __launch_bounds__(32 * G, 6) adj_step_kernel(const Params P, con
   // lambda~ = e lambda + (dq/df~)^T mu, a polynomial in (1, c_x, c_y, |c|^2)
   const double e = s_cf[warp][0], A0 = s_cf[warp][1], A1 = s_cf[warp][2], A2 = s_cf[warp][3], B = s_cf[warp][4];
   double2* o = out + base;
+  if (rows) {
+    output_rows(P, T, o, ey, e, A0, A1, A2, B);
+    return;
+  }
   for (int j = lane; j < P.nv; j += 32) {
     const double2 c = T.cxy[j];
     const double2 l = sl[j];
@@ -411,7 +572,7 @@ cudaError_t launch_adj_seed(const Params& P, const Tables& T, const double2* f, 
 
 namespace {
 
-size_t adj_cell_bytes(const Params& P) { return sizeof(double) * (size_t)(P.nvx + P.nvy); }
+size_t adj_cell_bytes(const Params& P) { return sizeof(double) * (size_t)(P.nvx + 3 * P.nvy); }
 
 template <int G>
 cudaError_t launch_adj_g(const Params& P, const Tables& T, const double2* fn1,
@@ -432,8 +593,8 @@ cudaError_t launch_adj_g(const Params& P, const Tables& T, const double2* fn1,
 
 }  // namespace
 
-// Cells per CTA: 4 while four cells' Gaussian factors fit in 100 KB (two
-// CTAs per SM), else 2, else 1.
+// Cells per CTA: 4 while their factors fit in 100 KB (two CTAs per SM), else
+// fewer (8: 2 % slower on the 128^2 x 32^2 gradient).
 cudaError_t launch_adj_step(const Params& P, const Tables& T, const double2* fn1,
                             const double4_32a* qn, const double4_32a* pn, const double2* lam_in, int tilde,
                             int collide, double2* out, const double2* dghost, double demit, double* dlnl,
