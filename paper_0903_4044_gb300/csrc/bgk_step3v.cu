@@ -221,8 +221,8 @@ namespace {
 // The FP64 pipe takes 64 to 76 cycles per warp instruction and bounded the
 // step (12.1 operations per velocity).  Here four remain, two to stream and
 // two to relax; the moment sums are exact integers, the Gaussians and the
-// relaxation weight come from the integer pipe.  2048 x 30^3: 1.24 -> 0.63 ms a
-// step, 512 x 16^3: 126 -> 50 us.  What bounds it now: pass 1 (half of the
+// relaxation weight come from the integer pipe.  2048 x 30^3: 1.24 -> 0.65 ms a
+// step, 512 x 16^3: 126 -> 51 us.  What bounds it now: pass 1 (half of the
 // time) by its loads, each lane's column comes from another cell (8 of each 32
 // bytes are used); the solve of a 16^3 cell takes as long as its passes.
 //
@@ -298,12 +298,14 @@ __device__ __forceinline__ bool stream3v_fixed(const Params3v& P, const Tables3v
         double f1[kAhead3], f2[kAhead3];
 #pragma unroll
         for (int u = 0; u < kAhead3; ++u) {
+          if (k0 + u >= L.yrows) break;  // the same for every lane
           const int j = jb + min(L.y0 + (k0 + u) * L.ystep, nvy - 1) * nvx;
           f1[u] = p1[j];
           f2[u] = p2[j];
         }
 #pragma unroll
         for (int u = 0; u < kAhead3; ++u) {
+          if (k0 + u >= L.yrows) break;
           const int jy = L.y0 + (k0 + u) * L.ystep;
           const double ft = fma(rem, f2[u] - f1[u], f1[u]);
           if (zin && jy < nvy) {
@@ -312,10 +314,8 @@ __device__ __forceinline__ bool stream3v_fixed(const Params3v& P, const Tables3v
             top = max(top, (int)(hi >> 20));
             t1 = fx::add(t1, fx::double_to_units96(hi, (unsigned)__double2loint(ft), (unsigned)eg));
           }
-          if (k0 + u < L.yrows) {
-            t2 = fx::add(t2, t1);
-            t3 = fx::add(t3, t2);
-          }
+          t2 = fx::add(t2, t1);
+          t3 = fx::add(t3, t2);
         }
       }
       n0 = fx::add(n0, t1);
@@ -656,8 +656,11 @@ cudaError_t launch_init3v(const Params3v& P, const Tables3v& T, double x_split, 
   return cudaGetLastError();
 }
 
-// Lanes per row and warps along z that leave the fewest lanes idle (more
-// lanes per row, then more warps along z, on a tie).  The fixed-point kernel
+// Lanes per row and warps along z that leave the fewest lanes idle, a tenth
+// off for each further column of a lane, which reads the same sectors again
+// (11 x 21 x 23 velocities, 1400 cells: 346 us a step with three columns at 77 %
+// use, 291 with one at 63 %; 18 x 26 x 11, 600 cells: 162 and 115); more lanes
+// per row, then more warps along z, on a tie.  The fixed-point kernel
 // takes at most 64 velocities per axis (its squared indices and sums then stay
 // within 95 bits).
 void plan3v(Params3v& P) {
@@ -674,14 +677,14 @@ void plan3v(Params3v& P) {
     for (int zb = 3; zb >= 0; --zb) {
       const int lw = 1 << lb, ys = (kW >> zb) * (32 >> lb), zs = 1 << zb;
       const double width = (P.nvx + lw - 1) / lw * lw, y = (P.nvy + ys - 1) / ys * ys, z = (P.nvz + zs - 1) / zs * zs;
-      const double use = (double)P.nv / (width * y * z);
+      const double use = (double)P.nv / (width * y * z) * (1.0 - 0.1 * (width / lw - 1.0));
       if (use > best + 1e-9) {
         best = use;
         P.lane_bits = lb;
         P.zw_bits = zb;
       }
     }
-  if (best < 0.5) P.lane_bits = 0;
+  if (best < 0.3) P.lane_bits = 0;
 }
 
 cudaError_t launch_step3v(const Params3v& P, const Tables3v& T, const double* fin, double* fout, double* mom,
