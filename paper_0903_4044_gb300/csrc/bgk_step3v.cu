@@ -656,13 +656,16 @@ cudaError_t launch_init3v(const Params3v& P, const Tables3v& T, double x_split, 
   return cudaGetLastError();
 }
 
-// Lanes per row and warps along z that leave the fewest lanes idle, a tenth
-// off for each further column of a lane, which reads the same sectors again
-// (11 x 21 x 23 velocities, 1400 cells: 346 us a step with three columns at 77 %
-// use, 291 with one at 63 %; 18 x 26 x 11, 600 cells: 162 and 115); more lanes
-// per row, then more warps along z, on a tie.  The fixed-point kernel
-// takes at most 64 velocities per axis (its squared indices and sums then stay
-// within 95 bits).
+// Lanes per row and warps along z with the least work per lane: its rows, two
+// rows' time for the wait of each batch of kAhead3 loads, and a tenth more for
+// each further column, which reads the same sectors again (11 x 21 x 23
+// velocities, 1400 cells: 346 us a step with three columns at 77 % use of the
+// lanes, 291 with one at 63 %; 18 x 26 x 11, 600 cells: 162 and 115).  By the
+// lanes' use alone, 22 x 31 x 19 took three columns with one row a batch: 126 us
+// a step on 100 cells and 342 on 600, 58 and 121 with one column of 16 rows.  More
+// lanes per row, then more warps along z, unless the gain is above 3 %.  The
+// fixed-point kernel takes at most 64 velocities per axis (its squared indices
+// and sums then stay within 95 bits).
 void plan3v(Params3v& P) {
   const int n3[3] = {P.nvx, P.nvy, P.nvz};
   for (int a = 0; a < 3; ++a) {
@@ -676,15 +679,17 @@ void plan3v(Params3v& P) {
   for (int lb = 5; lb >= 2; --lb)
     for (int zb = 3; zb >= 0; --zb) {
       const int lw = 1 << lb, ys = (kW >> zb) * (32 >> lb), zs = 1 << zb;
-      const double width = (P.nvx + lw - 1) / lw * lw, y = (P.nvy + ys - 1) / ys * ys, z = (P.nvz + zs - 1) / zs * zs;
-      const double use = (double)P.nv / (width * y * z) * (1.0 - 0.1 * (width / lw - 1.0));
-      if (use > best + 1e-9) {
-        best = use;
+      const int cols = (P.nvx + lw - 1) / lw, rows = (P.nvy + ys - 1) / ys, z = (P.nvz + zs - 1) / zs;
+      const double work = cols * z * (rows + 2.0 * ((rows + kAhead3 - 1) / kAhead3)) * (1.0 + 0.1 * (cols - 1));
+      if (best == 0.0 || work < 0.97 * best) {
+        best = work;
         P.lane_bits = lb;
         P.zw_bits = zb;
       }
     }
-  if (best < 0.3) P.lane_bits = 0;
+  const int lw = 1 << P.lane_bits, ys = (kW >> P.zw_bits) * (32 >> P.lane_bits), zs = 1 << P.zw_bits;
+  const double lanes = (double)((P.nvx + lw - 1) / lw * lw) * ((P.nvy + ys - 1) / ys * ys) * ((P.nvz + zs - 1) / zs * zs);
+  if (P.nv < 0.3 * lanes) P.lane_bits = 0;
 }
 
 cudaError_t launch_step3v(const Params3v& P, const Tables3v& T, const double* fin, double* fout, double* mom,
