@@ -47,7 +47,7 @@ def check(s, prob, f, steps=2, signed=False):
 
 
 @pytest.mark.parametrize("nv", [(16, 16, 16), (30, 30, 30), (13, 11, 9), (33, 10, 12), (64, 9, 10), (9, 64, 10), (10, 9, 17),
-                                (65, 9, 9), (12, 14, 1)])
+                                (65, 9, 9), (12, 14, 1), (22, 31, 19), (20, 31, 22), (13, 29, 19)])
 def test_velocity_grids(nv):
     check(*pair(nv, conservative=0 if min(nv) == 1 else 1))
 
