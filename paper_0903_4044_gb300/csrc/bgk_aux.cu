@@ -49,14 +49,14 @@ __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32
     const double ay = fabs(cyj) * P.dt / P.dy;
     coef[j] = make_double4_32a(1.0 - ax - ay, ax, ay, c2);
     shift[j] = 0;
-    // the weights as integers over 2^63; where rounding would make a sum of
-    // two exceed one (Courant number 1), the x weight gives way
+    // the weights as integers over 2^63, rounded; where that would make a sum
+    // of two exceed one (Courant number 1), the x weight gives way
     const double one = 9223372036854775808.0;  // 2^63
     const double cy_top = fmax(fabs(centre(P.vy_min, 0, P.dcy)), fabs(centre(P.vy_min, P.nvy - 1, P.dcy)));
-    const uint64_t wy_top = (uint64_t)(cy_top * P.dt / P.dy * one), rest = ((uint64_t)1 << 63) - wy_top;
-    const uint64_t w = (uint64_t)(ax * one);
+    const uint64_t wy_top = __double2ull_rn(cy_top * P.dt / P.dy * one), rest = ((uint64_t)1 << 63) - wy_top;
+    const uint64_t w = __double2ull_rn(ax * one);
     if (jy == 0) wx[jx] = w < rest ? w : rest;
-    if (jx == 0) wy[jy] = (uint64_t)(ay * one) | (cyj < 0.0 ? (uint64_t)1 << 63 : 0);
+    if (jx == 0) wy[jy] = __double2ull_rn(ay * one) | (cyj < 0.0 ? (uint64_t)1 << 63 : 0);
     // f~ / sx = f_upx + ratio.x f + ratio.y f_upy; where c_x = 0 the upwind
     // value is f itself, whose weight a0 is split
     const double s = ax > 0.0 ? ax : 0.5 * (1.0 - cy_top * P.dt / P.dy);

@@ -169,13 +169,13 @@ __device__ __forceinline__ double combine_fast(double f0, double fxv, double fyv
   return __hiloint2double((int)hi, (int)lo);
 }
 
-// The same in FP64 (a call: inlined, its conversions would be scheduled ahead
-// of the branch).
-__device__ __noinline__ double combine_slow(double f0, double fxv, double fyv, unsigned long long w0,
-                                            unsigned long long wx, unsigned long long wy, unsigned eref,
-                                            unsigned long long& units) {
-  const double s = 1.0 / 9223372036854775808.0;  // 2^-63
-  const double v = fma((double)wy * s, fyv, fma((double)wx * s, fxv, (double)w0 * s * f0));
+// The same in FP64 with the FP64 weights (integers over 2^63 keep fewer than
+// 53 bits of a weight below 2^-10, and beside a front that weight's error is
+// the result's).  A call: inlined, it would be scheduled ahead of the branch.
+__device__ __noinline__ double combine_slow(double f0, double fxv, double fyv, const double4_32a* __restrict__ coef,
+                                            unsigned eref, unsigned long long& units) {
+  const double4_32a co = *coef;
+  const double v = fma(co.z, fyv, fma(co.y, fxv, co.x * f0));
   units = fx::double_to_units((unsigned)__double2hiint(v), (unsigned)__double2loint(v), eref);
   return v;
 }
@@ -290,7 +290,7 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
         toph = max(toph, (int)(hh >> 20) - shift);
       }
       if (valid && !ok) {  // rare: values near the smallest doubles, or fronts steeper than the weights
-        tile[j].x = combine_slow(f0.x, fxv.x, fyv.x, rest - wy, wx, wy, (unsigned)eg, ug);
+        tile[j].x = combine_slow(f0.x, fxv.x, fyv.x, T.coef + j, (unsigned)eg, ug);
         s1 += ug;
       }
       s2 = fx::add(s2, fx::wide(s1));
