@@ -123,13 +123,8 @@ BGK_HD void to_words(u64 r, u32 emax, u32& hi, u32& lo) {
   hi = (u32)(m >> 32) + ((emax + 3u - lz) << 20);
 }
 
-// The same r in the cell's unit 2^(eref - 1081), rounded; at most 2^59 for emax <= eref.
-BGK_HD u64 to_units(u64 r, u32 emax, u32 eref) {
-  const u32 d = eref - emax;
-  return shr64(r, d + 1u) + ((u32)shr64(r, d) & 1u);
-}
-
-// A positive double (words hi, lo) in the cell's unit.
+// A positive double (words hi, lo) in the cell's unit 2^(eref - 1081), rounded;
+// at most 2^59 for an exponent field of at most eref.
 BGK_HD u64 double_to_units(u32 hi, u32 lo, u32 eref) {
   const u64 m = (u64)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
   const u32 d = eref - (hi >> 20);  // m 2^(6 - d)

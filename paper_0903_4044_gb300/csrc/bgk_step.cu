@@ -147,13 +147,11 @@ __device__ __forceinline__ fx::i96 warp_reduce8_96(const fx::i96 (&v)[8]) {
   return xor_add96(x, x, 1);
 }
 
-// g of f~ from its own and upwind values, in fixed point; `top` keeps the
-// largest exponent seen (a sign bit counts as a large one).  `ok` turns false
-// when the values are too small, or their weighted sum is far below the
-// largest of them.
+// g of f~ from its own and upwind values, in fixed point.  `ok` is false when
+// the largest of them is too small or too large (a sign bit counts as large),
+// or the weighted sum far below it.
 __device__ __forceinline__ double combine_fast(double f0, double fxv, double fyv, unsigned long long w0,
-                                               unsigned long long wx, unsigned long long wy, unsigned eref,
-                                               unsigned& top, bool& ok, unsigned long long& units) {
+                                               unsigned long long wx, unsigned long long wy, bool& ok) {
   const unsigned h0 = (unsigned)__double2hiint(f0), hx = (unsigned)__double2hiint(fxv),
                  hy = (unsigned)__double2hiint(fyv);
   const unsigned emax = max(max(h0, hx), hy) >> 20;
@@ -161,9 +159,7 @@ __device__ __forceinline__ double combine_fast(double f0, double fxv, double fyv
       fx::combine(w0, fx::align(h0, (unsigned)__double2loint(f0), emax), wx,
                   fx::align(hx, (unsigned)__double2loint(fxv), emax), wy,
                   fx::align(hy, (unsigned)__double2loint(fyv), emax));
-  top = max(top, emax);
-  ok = emax >= fx::kExpMin && fx::combine_ok(r);
-  units = fx::to_units(r, emax, eref);
+  ok = emax - fx::kExpMin <= fx::kExpMax - fx::kExpMin && fx::combine_ok(r);
   unsigned hi, lo;
   fx::to_words(r, emax, hi, lo);
   return __hiloint2double((int)hi, (int)lo);
@@ -172,12 +168,10 @@ __device__ __forceinline__ double combine_fast(double f0, double fxv, double fyv
 // The same in FP64 with the FP64 weights (integers over 2^63 keep fewer than
 // 53 bits of a weight below 2^-10, and beside a front that weight's error is
 // the result's).  A call: inlined, it would be scheduled ahead of the branch.
-__device__ __noinline__ double combine_slow(double f0, double fxv, double fyv, const double4_32a* __restrict__ coef,
-                                            unsigned eref, unsigned long long& units) {
+__device__ __noinline__ double combine_slow(double f0, double fxv, double fyv,
+                                            const double4_32a* __restrict__ coef) {
   const double4_32a co = *coef;
-  const double v = fma(co.z, fyv, fma(co.y, fxv, co.x * f0));
-  units = fx::double_to_units((unsigned)__double2hiint(v), (unsigned)__double2loint(v), eref);
-  return v;
+  return fma(co.z, fyv, fma(co.y, fxv, co.x * f0));
 }
 
 // Own and upwind values of velocity j = (jx, jy) of a cell at the edge.
@@ -227,10 +221,11 @@ __device__ __forceinline__ void prefetch_l1(const double2* p) {
 //  h: parked divided by the column's scale s (= |c_x| dt / dx), so that f~/s
 //     = f_x + (a0/s) f + (ay/s) f_y takes two FMAs; summed as integers per
 //     column, the scale applied to the column's sum.
-// eg, eh: largest exponents of g and h that the sums' units are cut for.  On
-// return they are the largest exponents seen; the sums are valid when these
-// do not exceed the ones passed in and the result is true (no lane's sum ran
-// over 63 bits).
+// eg, eh: largest exponents of f~ that the sums' units are cut for (of f~
+// itself: a neighbour may be any number of times as large when its weight is
+// small).  On return they are the largest exponents seen; the sums are valid
+// when these do not exceed the ones passed in and the result is true (no lane's
+// sum ran over 63 bits).
 template <int W, bool EDGE>
 __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables& T, const double2* __restrict__ fc,
                                                   ptrdiff_t row, const CellEdge& C, int wi,
@@ -240,8 +235,8 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
   const int lane = threadIdx.x & 31, nvx = P.nvx, nvy = P.nvy;
   const LaneMap<W> L(P, wi);
   const int h = L.row0, rpw = L.step, rows = L.rows;
-  unsigned topg = 0, over = 0;
-  int toph = 0;
+  unsigned over = 0;
+  int topg = 0, toph = 0;
   double hs = 0.0;
   const fx::i96 zero = {0u, 0u, 0u};
   fx::i96 n0 = zero, x1 = zero, x2 = zero, i1 = zero, i2 = zero;
@@ -277,21 +272,18 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
           prefetch_l1(a + offy);
         }
       }
-      u64 ug;
       bool ok;
-      ft.x = combine_fast(f0.x, fxv.x, fyv.x, rest - wy, wx, wy, (unsigned)eg, topg, ok, ug);
+      ft.x = combine_fast(f0.x, fxv.x, fyv.x, rest - wy, wx, wy, ok);
       ft.y = fma(ra.y, fyv.y, fma(ra.x, f0.y, fxv.y));
-      const bool valid = in && jr < nvy;
-      if (valid) {
-        const unsigned hh = (unsigned)__double2hiint(ft.y);
+      // rare: negative values, values near the smallest doubles, fronts steeper than the weights
+      if (!ok) ft.x = combine_slow(f0.x, fxv.x, fyv.x, T.coef + j);
+      if (in && jr < nvy) {
+        const unsigned hg = (unsigned)__double2hiint(ft.x), hh = (unsigned)__double2hiint(ft.y);
         tile[j] = ft;
-        s1 += ok ? ug : 0;
+        s1 += fx::double_to_units(hg, (unsigned)__double2loint(ft.x), (unsigned)eg);
         hsum += fx::double_to_units(hh, (unsigned)__double2loint(ft.y), (unsigned)ehc);
+        topg = max(topg, (int)(hg >> 20));
         toph = max(toph, (int)(hh >> 20) - shift);
-      }
-      if (valid && !ok) {  // rare: values near the smallest doubles, or fronts steeper than the weights
-        tile[j].x = combine_slow(f0.x, fxv.x, fyv.x, T.coef + j, (unsigned)eg, ug);
-        s1 += ug;
       }
       s2 = fx::add(s2, fx::wide(s1));
       s3 = fx::add(s3, s2);
@@ -307,7 +299,7 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
   }
   topg = __reduce_max_sync(0xffffffffu, topg);
   toph = __reduce_max_sync(0xffffffffu, toph);
-  const bool valid = (int)topg <= eg && toph <= eh && !__any_sync(0xffffffffu, (int)over < 0);
+  const bool valid = topg <= eg && toph <= eh && !__any_sync(0xffffffffu, (int)over < 0);
   if (valid) {
     // j_y of row r: A - rpw (rows - r); i1 = sum (rows - r) g, i2 = sum (rows - r)(rows - r + 1) / 2 g
     const unsigned A = (unsigned)(h + rpw * rows), B = (unsigned)rpw;
@@ -332,7 +324,7 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
     }
     if (lane == 0) sums[5] = hs;
   }
-  eg = (int)topg;
+  eg = topg;
   eh = toph;
   return valid;
 }

@@ -136,3 +136,14 @@ def test_small_time_steps(what, cfl):
     for a, b in ((st[..., 0], g1), (st[..., 1], h1)):
         assert (np.abs(a - b) <= 1e-12 * np.abs(b)).all()
     s.close()
+
+
+@pytest.mark.parametrize("tile", [1, 8])
+def test_sums_beside_a_steep_front(tile):
+    # a cell takes 1e-7 of a neighbour 1e14 times as dense: the sums keep the bits of the cell's own values
+    s, prob, g, h = pair(6, 5, 24, 20, cons=0, kinds=(2, 2, 2, 2), cfl=1e-7, tile=tile)
+    g[12:18] *= 1e14
+    h[12:18] *= 1e14
+    st, m, g1, h1, mom = run(s, prob, g, h, 1)
+    assert_moments_close(m, mom, vscale=0.05, tol=1e-14)
+    s.close()
