@@ -238,10 +238,11 @@ __device__ __forceinline__ void collide_sums(const Params& P, const Tables& T, c
 // ---- interior cells on grids that P.lane_bits maps -----------------------------
 // 2^lane_bits lanes share a velocity row; a lane takes its columns one after
 // the other, each over its rows, so that what depends on one axis is held per
-// column or read per row: lambda^{n+1} / s gathers in two FMAs per component
-// (s the column's scale, as in the forward step), the collision sums take seven
-// FP64 operations a velocity and the output three, 14 where the plain loops
-// (edge cells) take 24.
+// column or read per row: the collision sums take seven FP64 operations a
+// velocity and the output three, 16 with the gather where the plain loops (edge
+// cells) take 24.  (lambda over the column's x weight gathers in two operations
+// less; the weights then sum to one within a few roundings only, with the same
+// sign every step.)
 struct RowMap {
   int l, width, row0, step;
   __device__ __forceinline__ explicit RowMap(const Params& P) {
@@ -298,7 +299,7 @@ __device__ __forceinline__ void row_factors(const Params& P, const Tables& T, co
   }
 }
 
-// lambda^{n+1} / s into dst and the collision sums of collide_sums.
+// lambda^{n+1} into dst and the collision sums of collide_sums.
 __device__ __forceinline__ void gather_sums_rows(const Params& P, const Tables& T, const double2* __restrict__ lt,
                                                  const double2* __restrict__ f1, double2* __restrict__ dst,
                                                  const double* ex, const double* wy, double hp, double (&sum)[8]) {
@@ -309,10 +310,11 @@ __device__ __forceinline__ void gather_sums_rows(const Params& P, const Tables& 
 #pragma unroll 1
   for (int jx = L.l; jx < nvx; jx += L.width) {
     const int offx = sgn_x(T.vinfo[jx]) * P.nv;  // downwind neighbours used this value as their upwind source
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, b0 = 0.0, d0 = 0.0;
+    const double ax = T.awx[jx];
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, b0 = 0.0;
 #pragma unroll 1
     for (int j0 = L.row0; j0 < nvy; j0 += kRows * L.step) {
-      double2 l0[kRows], lx[kRows], ly[kRows], ra[kRows], f[kRows];
+      double2 l0[kRows], lx[kRows], ly[kRows], co[kRows], f[kRows];
 #pragma unroll
       for (int u = 0; u < kRows; ++u) {
         const int j = min(j0 + u * L.step, nvy - 1) * nvx + jx;
@@ -320,7 +322,7 @@ __device__ __forceinline__ void gather_sums_rows(const Params& P, const Tables& 
         l0[u] = lt[j];
         lx[u] = lt[j + offx];
         ly[u] = lt[j + offy];
-        ra[u] = T.ratio[j];
+        co[u] = T.a0y[j];
         f[u] = f1[j];
       }
 #pragma unroll
@@ -328,25 +330,24 @@ __device__ __forceinline__ void gather_sums_rows(const Params& P, const Tables& 
         const int jy = j0 + u * L.step;
         if (jy < nvy) {
           double2 l;
-          l.x = fma(ra[u].y, ly[u].x, fma(ra[u].x, l0[u].x, lx[u].x));
-          l.y = fma(ra[u].y, ly[u].y, fma(ra[u].x, l0[u].y, lx[u].y));
+          l.x = fma(co[u].y, ly[u].x, fma(ax, lx[u].x, co[u].x * l0[u].x));
+          l.y = fma(co[u].y, ly[u].y, fma(ax, lx[u].y, co[u].x * l0[u].y));
           dst[jy * nvx + jx] = l;
           const double t = fma(hp, l.y, l.x), w = wy[jy];
           a0 = fma(w, t, a0);
           a1 = fma(wy[nvy + jy], t, a1);
           a2 = fma(wy[2 * nvy + jy], t, a2);
           b0 = fma(w, l.y, b0);
-          d0 = fma(l.x, f[u].x, fma(l.y, f[u].y, d0));
+          sum[5] = fma(l.x, f[u].x, fma(l.y, f[u].y, sum[5]));
         }
       }
     }
-    const double s = T.sx[jx], es = ex[jx] * s, c = T.cx[jx], g = es * a0, cg = c * g;
+    const double x = ex[jx], c = T.cx[jx], g = x * a0, cg = c * g;
     sum[0] += g;
     sum[1] += cg;
-    sum[2] = fma(es, a1, sum[2]);
-    sum[3] += fma(es, a2, c * cg);
-    sum[4] = fma(es, b0, sum[4]);
-    sum[5] = fma(s, d0, sum[5]);
+    sum[2] = fma(x, a1, sum[2]);
+    sum[3] += fma(x, a2, c * cg);
+    sum[4] = fma(x, b0, sum[4]);
   }
 }
 
@@ -363,7 +364,7 @@ __device__ __forceinline__ void output_rows(const Params& P, const Tables& T, do
   __syncwarp();
 #pragma unroll 1
   for (int jx = L.l; jx < nvx; jx += L.width) {
-    const double c = T.cx[jx], px = fma(c, fma(B, c, A1), A0), es = e * T.sx[jx];
+    const double c = T.cx[jx], px = fma(c, fma(B, c, A1), A0);
 #pragma unroll 1
     for (int j0 = L.row0; j0 < nvy; j0 += kRows * L.step) {
       double2* p = o + j0 * nvx + jx;
@@ -374,7 +375,7 @@ __device__ __forceinline__ void output_rows(const Params& P, const Tables& T, do
 #pragma unroll
       for (int u = 0; u < kRows; ++u)
         if (j0 + u * L.step < nvy)
-          p[u * L.step * nvx] = make_double2(fma(es, l[u].x, px + qy[j0 + u * L.step]), fma(es, l[u].y, B));
+          p[u * L.step * nvx] = make_double2(fma(e, l[u].x, px + qy[j0 + u * L.step]), fma(e, l[u].y, B));
     }
   }
 }

@@ -61,8 +61,8 @@ struct bgk_solver {
   double* cx = nullptr;
   double* cy = nullptr;  // [2 nvy]: centres, then the fixed-point y weights
   uint64_t* wx = nullptr;  // [nvx] fixed-point x weights
-  double* sx = nullptr;     // [nvx] column scales
-  double2* ratio = nullptr;  // [nv]
+  double* awx = nullptr;    // [nvx] |c_x| dt / dx
+  double2* a0y = nullptr;   // [nv] (a0, ay)
   double4_32a* coef = nullptr;
   int* shift = nullptr;
   double2* cxy = nullptr;
@@ -94,8 +94,8 @@ struct bgk_solver {
     T.grid = bgk::velocity_grid(P);
     T.wx = wx;
     T.wy = y_weights();
-    T.sx = sx;
-    T.ratio = ratio;
+    T.awx = awx;
+    T.a0y = a0y;
     T.coef = coef;
     T.shift = shift;
     T.cxy = cxy;
@@ -344,7 +344,7 @@ void release(bgk_solver* s) {
   for (auto& g : s->graph)
     if (g) cudaGraphExecDestroy(g);
   void* bufs[] = {s->f[0], s->f[1], s->stage, s->mom_step, s->mom_tmp, s->flux_tmp, s->cx, s->cy,
-                  s->coef, s->shift, s->cxy, s->vinfo, s->ghost, s->emitted, s->wx, s->sx, s->ratio, s->m_coef, s->m_cx,
+                  s->coef, s->shift, s->cxy, s->vinfo, s->ghost, s->emitted, s->wx, s->awx, s->a0y, s->m_coef, s->m_cx,
                   s->m_cy, s->m_ax, s->m_ay, s->m_ghost, s->m_mabs, s->m_sums, s->m_ctr, s->err};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -537,8 +537,8 @@ bgk_status bgk_create(const bgk_config* cfg, bgk_solver** out) {
   ALLOC(cx, P.nvx);
   ALLOC(cy, 2 * (size_t)P.nvy);
   ALLOC(wx, P.nvx);
-  ALLOC(sx, P.nvx);
-  ALLOC(ratio, P.nv);
+  ALLOC(awx, P.nvx);
+  ALLOC(a0y, P.nv);
   ALLOC(coef, P.nv);
   ALLOC(shift, P.nv);
   ALLOC(cxy, P.nv);
@@ -555,7 +555,7 @@ bgk_status bgk_create(const bgk_config* cfg, bgk_solver** out) {
   if (e == cudaSuccess && s->m_ctr) e = cudaMemsetAsync(s->m_ctr, 0, 2 * sizeof(unsigned), s->stream);
   if (e == cudaSuccess)
     e = bgk::launch_build_tables(P, s->cx, s->cy, s->coef, s->shift, s->cxy, s->vinfo, s->ghost,
-                                 s->emitted, s->wx, s->y_weights(), s->sx, s->ratio, s->stream);
+                                 s->emitted, s->wx, s->y_weights(), s->awx, s->a0y, s->stream);
   if (e == cudaSuccess && s->prec != bgk::PREC_F64) e = bgk::launch_build_mixed_tables(P, s->tables(), s->mtables(), s->stream);
   if (e == cudaSuccess) e = s->prec == bgk::PREC_F64 ? bgk::prepare_step_f64(P) : bgk::prepare_step_mixed(P, s->prec);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -818,7 +818,7 @@ bgk_status bgk_sync(bgk_solver* s) {
 namespace {
 
 constexpr size_t kNoAllocScratchBytes = 384 * 1024;  // about 120 bytes per velocity
-// behind it: x weights and scales (nvy >= 2), ratios
+// behind it: x weights in both forms (nvy >= 2), (a0, ay)
 constexpr size_t kNoAllocWeightBytes = (sizeof(uint64_t) + sizeof(double)) * bgk::kMaxNv / 2 + sizeof(double2) * bgk::kMaxNv;
 constexpr int kNoAllocMaxDevices = 64;
 
@@ -867,7 +867,7 @@ extern "C" bgk_status bgk_step_noalloc(const bgk_config* cfg, const double* f_in
     return fail(BGK_ERR_INVALID_ARG, "f_in and f_out overlap");
 
   // scratch layout: tables then the error flag, each 256-byte aligned; the
-  // x weights, scales and ratios follow at kNoAllocScratchBytes
+  // fixed-point step's weights follow at kNoAllocScratchBytes
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t at = off;
@@ -909,15 +909,15 @@ extern "C" bgk_status bgk_step_noalloc(const bgk_config* cfg, const double* f_in
   int* err = (int*)(base + o_err);
   uint64_t* wx = (uint64_t*)(base + kNoAllocScratchBytes);
   uint64_t* wy = (uint64_t*)(cy + P.nvy);
-  double* sx = (double*)(wx + bgk::kMaxNv / 2);
-  double2* ratio = (double2*)(sx + bgk::kMaxNv / 2);
+  double* awx = (double*)(wx + bgk::kMaxNv / 2);
+  double2* a0y = (double2*)(awx + bgk::kMaxNv / 2);
   T.cx = cx;
   T.cy = cy;
   T.grid = bgk::velocity_grid(P);
   T.wx = wx;
   T.wy = wy;
-  T.sx = sx;
-  T.ratio = ratio;
+  T.awx = awx;
+  T.a0y = a0y;
   T.coef = coef;
   T.shift = shift;
   T.cxy = cxy;
@@ -927,7 +927,7 @@ extern "C" bgk_status bgk_step_noalloc(const bgk_config* cfg, const double* f_in
 
   cudaStream_t stream = (cudaStream_t)cfg->cuda_stream;
   e = cudaMemsetAsync(err, 0, sizeof(int), stream);
-  if (e == cudaSuccess) e = bgk::launch_build_tables(P, cx, cy, coef, shift, cxy, vinfo, ghost, emitted, wx, wy, sx, ratio, stream);
+  if (e == cudaSuccess) e = bgk::launch_build_tables(P, cx, cy, coef, shift, cxy, vinfo, ghost, emitted, wx, wy, awx, a0y, stream);
   if (e == cudaSuccess) e = bgk::prepare_step_f64(P);
   if (e == cudaSuccess)
     e = bgk::launch_step_f64(P, T, (const double2*)f_in, (double2*)f_out, (double4_32a*)mom_out, err, stream);

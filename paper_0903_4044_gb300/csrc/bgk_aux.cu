@@ -16,8 +16,8 @@ __device__ __forceinline__ double centre(double vmin, int j, double dc) {
 // instead of all (bgk_step_noalloc builds the tables on every call: 32^2 cells
 // x 16^2 velocities 73 -> 60 us).
 __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32a* coef, int* shift,
-                              double2* cxy, int* vinfo, double2* ghost, uint64_t* wx, uint64_t* wy, double* sx,
-                              double2* ratio) {
+                              double2* cxy, int* vinfo, double2* ghost, uint64_t* wx, uint64_t* wy, double* awx,
+                              double2* a0y) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= P.nv) return;
   const int jx = j % P.nvx, jy = j / P.nvx;
@@ -57,11 +57,8 @@ __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32
     const uint64_t w = __double2ull_rn(ax * one);
     if (jy == 0) wx[jx] = w < rest ? w : rest;
     if (jx == 0) wy[jy] = __double2ull_rn(ay * one) | (cyj < 0.0 ? (uint64_t)1 << 63 : 0);
-    // f~ / sx = f_upx + ratio.x f + ratio.y f_upy; where c_x = 0 the upwind
-    // value is f itself, whose weight a0 is split
-    const double s = ax > 0.0 ? ax : 0.5 * (1.0 - cy_top * P.dt / P.dy);
-    if (jy == 0) sx[jx] = s;
-    ratio[j] = make_double2((1.0 - ax - ay - (ax > 0.0 ? 0.0 : s)) / s, ay / s);
+    if (jy == 0) awx[jx] = ax;
+    a0y[j] = make_double2(1.0 - ax - ay, ay);
   } else {
     // Eq. (exact) shift by [C], then Eq. (upwind) with the remainder r
     const double C = cxj * P.dt / P.dx;
@@ -94,9 +91,9 @@ __global__ void __launch_bounds__(256) emitted_kernel(const Params P, const doub
 
 cudaError_t launch_build_tables(const Params& P, double* cx, double* cy, double4_32a* coef, int* shift,
                                 double2* cxy, int* vinfo, double2* ghost, double* emitted, uint64_t* wx,
-                                uint64_t* wy, double* sx, double2* ratio, cudaStream_t stream) {
+                                uint64_t* wy, double* awx, double2* a0y, cudaStream_t stream) {
   const dim3 grid((P.nv + 127) / 128, P.dim == 2 ? 5 : 3);
-  tables_kernel<<<grid, 128, 0, stream>>>(P, cx, cy, coef, shift, cxy, vinfo, ghost, wx, wy, sx, ratio);
+  tables_kernel<<<grid, 128, 0, stream>>>(P, cx, cy, coef, shift, cxy, vinfo, ghost, wx, wy, awx, a0y);
   emitted_kernel<<<1, 256, 0, stream>>>(P, cx, cy, ghost, emitted);
   return cudaGetLastError();
 }

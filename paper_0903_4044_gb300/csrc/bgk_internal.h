@@ -74,8 +74,8 @@ struct Tables {
   const double* emitted;  // [kFaces] sum_{c_n>0} c_n G_W(n=1) dv (diffuse)
   const uint64_t* wx;     // [nvx] 2D streaming weight |c_x| dt / dx as an integer over 2^63
   const uint64_t* wy;     // [nvy] |c_y| dt / dy likewise, top bit set for c_y < 0; wx + wy <= 2^63
-  const double* sx;       // [nvx] 2D scale of a column: |c_x| dt / dx (c_x = 0: a value below its a0)
-  const double2* ratio;   // [nv] 2D (a0 / sx, ay / sx), for c_x = 0 (a0 / sx - 1, ay / sx)
+  const double* awx;      // [nvx] 2D |c_x| dt / dx
+  const double2* a0y;     // [nv] 2D (a0, ay) of coef
 };
 
 // FP32 tables of the reduced-precision step (bgk_mixed.cu).
@@ -104,7 +104,7 @@ cudaError_t launch_step_f64(const Params& P, const Tables& T, const double2* fin
                             double4_32a* mom, int* err, cudaStream_t stream, double4_32a* par = nullptr);
 cudaError_t launch_build_tables(const Params& P, double* cx, double* cy, double4_32a* coef, int* shift,
                                 double2* cxy, int* vinfo, double2* ghost, double* emitted, uint64_t* wx,
-                                uint64_t* wy, double* sx, double2* ratio, cudaStream_t stream);
+                                uint64_t* wy, double* awx, double2* a0y, cudaStream_t stream);
 // Fills P.lane_bits (FP64) from the grid, the boundaries and the Courant number.
 void step_f64_plan(Params& P, double max_courant);
 size_t step_f64_smem_bytes(const Params& P, int tile);

@@ -218,9 +218,10 @@ __device__ __forceinline__ void prefetch_l1(const double2* p) {
 //  g: fixed point.  The running sums of first, second and third order over a
 //     column's rows give sum g, sum j_y g and sum j_y^2 g as exact integers,
 //     and times j_x the x sums.
-//  h: parked divided by the column's scale s (= |c_x| dt / dx), so that f~/s
-//     = f_x + (a0/s) f + (ay/s) f_y takes two FMAs; summed as integers per
-//     column, the scale applied to the column's sum.
+//  h: three FP64 operations, summed as an integer.  (Parked over the column's x
+//     weight it takes two, 4 % of a step; but the rounding of the quotients
+//     and the product back drift by 0.025 to 0.03 of 2^-53 a step in a uniform
+//     state, rms, where this form drifts by 0.009 to 0.017.)
 // eg, eh: largest exponents of f~ that the sums' units are cut for (of f~
 // itself: a neighbour may be any number of times as large when its weight is
 // small).  On return they are the largest exponents seen; the sums are valid
@@ -237,9 +238,8 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
   const int h = L.row0, rpw = L.step, rows = L.rows;
   unsigned over = 0;
   int topg = 0, toph = 0;
-  double hs = 0.0;
   const fx::i96 zero = {0u, 0u, 0u};
-  fx::i96 n0 = zero, x1 = zero, x2 = zero, i1 = zero, i2 = zero;
+  fx::i96 hsum = zero, n0 = zero, x1 = zero, x2 = zero, i1 = zero, i2 = zero;
 #pragma unroll 1
   for (int jl = L.l; jl - L.l < nvx; jl += L.width) {
     const bool in = jl < nvx;
@@ -247,15 +247,14 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
     const int sgx = vi_sx(T.vinfo[jx]);
     const int offx = EDGE ? sgx : -sgx * P.nv;  // upwind in x: ix - sgn c_x
     const u64 wx = T.wx[jx], rest = ((u64)1 << fx::kWeightBits) - wx;
-    const double s = T.sx[jx];
-    const int shift = 1023 - (__double2hiint(s) >> 20), ehc = eh + shift;
-    u64 s1 = 0, hsum = 0;
+    const double ax = T.awx[jx];
+    u64 s1 = 0;
     fx::i96 s2 = zero, s3 = zero;
 #pragma unroll 1
     for (int r = 0; r < rows; ++r) {
       const int jr = h + r * rpw, jy = min(jr, nvy - 1), j = jy * nvx + jx;
       const u64 wys = T.wy[jy], wy = wys & ~((u64)1 << 63);  // top bit: c_y < 0
-      const double2 ra = T.ratio[j];
+      const double2 co = T.a0y[j];
       double2 f0, fxv, fyv, ft;
       if (EDGE) {
         load_point(P, T, fc, row, C, j, jx, jy, offx, vi_sy(T.vinfo[jy * nvx]), f0, fxv, fyv);
@@ -274,28 +273,26 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
       }
       bool ok;
       ft.x = combine_fast(f0.x, fxv.x, fyv.x, rest - wy, wx, wy, ok);
-      ft.y = fma(ra.y, fyv.y, fma(ra.x, f0.y, fxv.y));
+      ft.y = fma(co.y, fyv.y, fma(ax, fxv.y, co.x * f0.y));
       // rare: negative values, values near the smallest doubles, fronts steeper than the weights
       if (!ok) ft.x = combine_slow(f0.x, fxv.x, fyv.x, T.coef + j);
       if (in && jr < nvy) {
         const unsigned hg = (unsigned)__double2hiint(ft.x), hh = (unsigned)__double2hiint(ft.y);
         tile[j] = ft;
         s1 += fx::double_to_units(hg, (unsigned)__double2loint(ft.x), (unsigned)eg);
-        hsum += fx::double_to_units(hh, (unsigned)__double2loint(ft.y), (unsigned)ehc);
+        hsum = fx::add(hsum, fx::wide(fx::double_to_units(hh, (unsigned)__double2loint(ft.y), (unsigned)eh)));
         topg = max(topg, (int)(hg >> 20));
-        toph = max(toph, (int)(hh >> 20) - shift);
+        toph = max(toph, (int)(hh >> 20));
       }
       s2 = fx::add(s2, fx::wide(s1));
       s3 = fx::add(s3, s2);
-      over |= (unsigned)((s1 | hsum) >> 32);  // an addend is at most 2^59: the top bit shows before a sum wraps
+      over |= (unsigned)(s1 >> 32);  // an addend is at most 2^59: the top bit shows before a sum wraps
     }
     n0 = fx::add(n0, fx::wide(s1));
     i1 = fx::add(i1, s2);
     i2 = fx::add(i2, s3);
     x1 = fx::add(x1, fx::mul(fx::wide(s1), (unsigned)jx));
     x2 = fx::add(x2, fx::mul(fx::wide(s1), (unsigned)(jx * jx)));
-    // the column's unit times its scale: s 2^(ehc - 1081)
-    hs = fma((double)hsum, __hiloint2double(__double2hiint(s) + (ehc - 1081) * (1 << 20), __double2loint(s)), hs);
   }
   topg = __reduce_max_sync(0xffffffffu, topg);
   toph = __reduce_max_sync(0xffffffffu, toph);
@@ -306,23 +303,16 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
     const fx::i96 b1 = fx::mul(i1, B);
     fx::i96 v[8] = {n0, x1, x2, fx::add(fx::mul(n0, A), fx::neg(b1)),
                     fx::add(fx::add(fx::mul(n0, A * A), fx::neg(fx::mul(b1, 2u * A + B))), fx::mul(i2, 2u * B * B)),
-                    zero, zero, zero};
+                    hsum, zero, zero};
     const fx::i96 t = warp_reduce8_96(v);
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) hs += __shfl_xor_sync(0xffffffffu, hs, m);
-    // from j to k = 2 j + 1 - n: lane group q holds value q of (1, j_x, j_x^2, j_y, j_y^2) sums
+    // from j to k = 2 j + 1 - n: lane group q holds value q of (1, j_x, j_x^2, j_y, j_y^2) g sums and the h sum
     const int q = lane >> 2, n = 1 - (q <= 2 ? nvx : nvy);
     const fx::i96 first = shfl96(t, 0), prev = shfl96(t, max(lane - 4, 0));
     const bool lin = q == 1 || q == 3, quad = q == 2 || q == 4;
     const fx::i96 k = lin ? fx::add(fx::mul(t, 2u), fx::muls(first, n))
                           : quad ? fx::add(fx::add(fx::mul(t, 4u), fx::muls(prev, 4 * n)), fx::mul(first, (unsigned)(n * n)))
                                  : t;
-    if ((lane & 3) == 0 && q < 5) {
-      unsigned hi, lo;
-      fx::wide_to_words(k, (unsigned)eg, hi, lo);
-      sums[q] = __hiloint2double((int)hi, (int)lo);
-    }
-    if (lane == 0) sums[5] = hs;
+    if ((lane & 3) == 0 && q < kSums) sums[q] = unit_value(k, q < 5 ? eg : eh);
   }
   eg = topg;
   eh = toph;
@@ -1017,13 +1007,12 @@ __device__ __noinline__ double relax_slow(double h, double aphi, double b, doubl
 }
 
 // The same for a cell streamed by stream_rows_fixed (rows and columns of a
-// lane as there; h parked divided by the column's scale): g in two FP64
-// operations, h on the integer pipe beside them, as two products of 63-bit
+// lane as there): g in two FP64 operations, h on the integer pipe beside them, as two products of 63-bit
 // significands aligned, added and rounded once (error half an ulp plus about
 // 2^-58).  Values that are not positive normals well inside the range take
 // FP64.
 template <int W>
-__device__ __forceinline__ void relax_rows_fixed(const Params& P, const Tables& T, int wi, double2* __restrict__ fo,
+__device__ __forceinline__ void relax_rows_fixed(const Params& P, int wi, double2* __restrict__ fo,
                                                  const double* __restrict__ px, const double* __restrict__ py,
                                                  double b, double kappa) {
   typedef unsigned long long u64;
@@ -1033,15 +1022,15 @@ __device__ __forceinline__ void relax_rows_fixed(const Params& P, const Tables& 
   const unsigned hk = (unsigned)__double2hiint(kappa);
   const u64 wk = fx::top63(hk, (unsigned)__double2loint(kappa));
   const int ek = (int)(hk >> 20) - 1022;
+  // weights as 63-bit significands and exponents; a or b not positive (Euler
+  // form, steps beyond the collision time): every value takes FP64
+  const unsigned hb = (unsigned)__double2hiint(b);
+  const bool fit = min(hb, hk) >= (400u << 20) && max(hb, hk) < (1600u << 20);
+  const u64 wb = fx::top63(hb, (unsigned)__double2loint(b));
+  const int eb = (int)(hb >> 20) - 1022;
 #pragma unroll 1
   for (int jx = L.l; jx < nvx; jx += L.width) {
-    const double xv = px[jx], bs = b * T.sx[jx];
-    // weights as 63-bit significands and exponents; a or b not positive (Euler
-    // form, steps beyond the collision time): every value takes FP64
-    const unsigned hb = (unsigned)__double2hiint(bs);
-    const bool fit = min(hb, hk) >= (400u << 20) && max(hb, hk) < (1600u << 20);
-    const u64 wb = fx::top63(hb, (unsigned)__double2loint(bs));
-    const int eb = (int)(hb >> 20) - 1022;
+    const double xv = px[jx];
 #pragma unroll 1
     for (int j0 = L.row0; j0 < nvy; j0 += kRows * rpw) {
       double2 ft[kRows];
@@ -1060,7 +1049,7 @@ __device__ __forceinline__ void relax_rows_fixed(const Params& P, const Tables& 
           unsigned hi, lo;
           fx::to_words(r, (unsigned)e, hi, lo);
           double2 o = make_double2(fma(b, ft[u].x, aphi), __hiloint2double((int)hi, (int)lo));
-          if (!fit || e < (int)fx::kExpMin || e > (int)fx::kExpMax) o.y = relax_slow(ft[u].y, aphi, bs, kappa);
+          if (!fit || e < (int)fx::kExpMin || e > (int)fx::kExpMax) o.y = relax_slow(ft[u].y, aphi, b, kappa);
           p[u * rpw * nvx] = o;
         }
       }
@@ -1068,15 +1057,7 @@ __device__ __forceinline__ void relax_rows_fixed(const Params& P, const Tables& 
   }
 }
 
-// h of rows streamed by stream_rows_fixed, back from their columns' scales.
-template <int W>
-__device__ __noinline__ void unscale_rows(const Params& P, const Tables& T, int wi, double2* __restrict__ fo) {
-  const LaneMap<W> L(P, wi);
-  for (int jx = L.l; jx < P.nvx; jx += L.width)
-    for (int jy = L.row0; jy < P.nvy; jy += L.step) fo[jy * P.nvx + jx].y *= T.sx[jx];
-}
-
-// A4 of a warp's rows in FP64, f~ unscaled.
+// A4 of a warp's rows in FP64.
 template <int W>
 __device__ __noinline__ void relax_rows_f64(const Params& P, int wi, double2* __restrict__ fo,
                                             const double* __restrict__ px, const double* __restrict__ py, double b,
@@ -1162,14 +1143,9 @@ __global__ void __launch_bounds__(256, 4)
       maxwellian_cells_fixed<G, W>(P, T, blockIdx.x * G, s_sum, s_kind, phx, phy, s_b, s_k, s_ok, mom, par, err, s_x);
   if (!live) return;
   const double *px = phx + mine * P.nvx, *py = phy + mine * P.nvy;
-  const bool ok = s_ok[mine] != 0;
-  if (kind == SUMS_INDEX && fixed && ok) {
-    relax_rows_fixed<W>(P, T, wi, tile, px, py, s_b[mine], s_k[mine]);
-    return;
-  }
-  // a failed cell keeps f^{n+1} = f~ (flagged)
-  if (kind == SUMS_INDEX) unscale_rows<W>(P, T, wi, tile);
-  if (ok) relax_rows_f64<W>(P, wi, tile, px, py, s_b[mine], s_k[mine]);
+  if (!s_ok[mine]) return;  // a failed cell keeps f^{n+1} = f~ (flagged)
+  if (kind == SUMS_INDEX && fixed) relax_rows_fixed<W>(P, wi, tile, px, py, s_b[mine], s_k[mine]);
+  else relax_rows_f64<W>(P, wi, tile, px, py, s_b[mine], s_k[mine]);
 }
 
 namespace {

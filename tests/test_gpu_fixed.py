@@ -147,3 +147,24 @@ def test_sums_beside_a_steep_front(tile):
     st, m, g1, h1, mom = run(s, prob, g, h, 1)
     assert_moments_close(m, mom, vscale=0.05, tol=1e-14)
     s.close()
+
+
+@pytest.mark.parametrize("nvx,nvy,cfl", [(32, 32, 0.5), (48, 48, 0.9), (20, 28, 0.5), (24, 24, 1.0)])
+def test_uniform_state_does_not_drift(nvx, nvy, cfl):
+    # the weights of f~ sum to one within their roundings, the same every step: without relaxation g, combined
+    # in integers, stays as it is, and h, in three FP64 operations, moves by a sixtieth of 2^-53 a step (rms) at
+    # most: most values round back.  Two roundings more a step double that
+    n, steps = 1e-20, 200
+    s = solver.Solver(B.make_config(dim=2, nx=12, ny=12, lx=10.0, ly=10.0, nvx=nvx, nvy=nvy, vx=(-5.0, 5.0), vy=(-5.0, 5.0),
+                                    cfl=cfl, conservative=0, bc=[(2, n, 0.0, 0.0, 1.0)] * 4))
+    g = n * np.exp(-8.0 * np.random.default_rng(0).random((nvy, nvx)))
+    g = np.maximum(g, g[::-1])
+    g = np.maximum(g, g[:, ::-1]).ravel()
+    f = np.tile(np.stack([g, 0.5 * g], -1), (144, 1, 1))
+    s.set_state(f)
+    s.step(steps)
+    out = s.get_state()
+    assert (out[..., 0] == f[..., 0]).all()
+    drift = (out[..., 1] / f[..., 1] - 1.0) / steps * 2.0 ** 53
+    assert np.sqrt((drift ** 2).mean()) <= 0.02
+    s.close()
