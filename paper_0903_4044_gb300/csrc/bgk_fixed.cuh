@@ -9,8 +9,9 @@
 // multiplied with 63-bit weights, and the 60-bit result is normalised and
 // rounded once.  Its error is half an ulp of the result plus about 2^-59 of
 // the largest value (three FP64 operations: up to 1.5 ulp).  The sums over
-// the velocities add the results as integers in units of 2^-57 of the cell's
-// largest exponent: exact but for one rounding per value, whatever the order.
+// the velocities add the results as 96-bit integers in a unit 2^-75 of the
+// cell's largest exponent (more on long axes): each value is rounded to that
+// unit, the additions are exact, whatever the order.
 //
 // Everything here is plain integer arithmetic and runs on the host as well.
 #pragma once
@@ -61,6 +62,17 @@ BGK_HD u64 shr64(u64 x, u32 d) {
   return r;
 #else
   return d < 64u ? x >> d : 0;
+#endif
+}
+
+// x << d for any d (0 from 32 on).
+BGK_HD u32 shl32(u32 x, u32 d) {
+#ifdef __CUDA_ARCH__
+  u32 r;
+  asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(d));  // clamped likewise
+  return r;
+#else
+  return d < 32u ? x << d : 0u;
 #endif
 }
 
@@ -138,6 +150,24 @@ BGK_HD i96 double_to_units96(u32 hi, u32 lo, u32 eref) {
   const u32 e = eref - (hi >> 20) + 2u;  // m 2^(16 - e)
   const u64 top = shr64(m, e + 16u);
   return {e >= 16u ? (u32)shr64(m, e - 16u) : (u32)m << ((16u - e) & 31u), (u32)top, (u32)(top >> 32)};
+}
+
+// sum + the same value rounded to the nearest.
+BGK_HD i96 add_units96(i96 sum, u32 hi, u32 lo, u32 eref) {
+  const u64 m = ((u64)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 8;
+  const u32 e = eref - (hi >> 20) + 2u;  // m 2^(16 - e)
+  const u64 top = shr64(m, e + 16u), low = shr64(m, e - 17u);  // low: 0 unless e >= 17
+  const u32 v0 = (u32)(low >> 1) | shl32((u32)m, 16u - e), v1 = (u32)top, v2 = (u32)(top >> 32), half = (u32)low & 1u;
+#ifdef __CUDA_ARCH__
+  i96 r;  // half + (2^32 - 1) sets the carry where half is set
+  asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %9, 0xffffffff;\n\taddc.cc.u32 %0, %3, %6;\n\taddc.cc.u32 %1, %4, %7;\n\t"
+      "addc.u32 %2, %5, %8;\n\t}"
+      : "=&r"(r.a0), "=&r"(r.a1), "=&r"(r.a2)
+      : "r"(sum.a0), "r"(sum.a1), "r"(sum.a2), "r"(v0), "r"(v1), "r"(v2), "r"(half));
+  return r;
+#else
+  return add(add(sum, {v0, v1, v2}), {half, 0u, 0u});
+#endif
 }
 
 // The double nearest to v in units of 2^(eref - 1081), |v| < 2^95 (words).

@@ -34,6 +34,7 @@ struct Params {
   int mgl;   // reduced precisions: groups of 4 velocities per lane (2, 4 or 6)
   int lane_bits;  // FP64: log2 of the lanes per velocity row of the fixed-point step
                   // (step_f64_plan); 0: FP64-only form
+  int sum_room;   // bits by which its sums' unit lies above 2^-75 of the cell's range
   int conservative, relax_exact;
   int bc_kind[kFaces];
   double dt, dx, dy, dcx, dcy, dv;

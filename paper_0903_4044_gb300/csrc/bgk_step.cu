@@ -38,8 +38,9 @@
 #include "bgk_device.cuh"
 #include "bgk_solve.cuh"
 
-namespace bgk {
+#include <algorithm>
 
+namespace bgk {
 
 namespace {
 
@@ -216,27 +217,28 @@ __device__ __forceinline__ void prefetch_l1(const double2* p) {
 // the FP64 pipe 2.64 ms, both on the integer pipe 3.18 ms, this 2.36 ms); a
 // column's weights and running sums stay in registers.
 //  g: fixed point.  The running sums of first, second and third order over a
-//     column's rows give sum g, sum j_y g and sum j_y^2 g as exact integers,
-//     and times j_x the x sums.
+//     column's rows give sum g, sum j_y g and sum j_y^2 g as integers, and
+//     times j_x the x sums.  Their unit has to lie far below the tail of a
+//     narrow distribution: weighted with the squared index its rounding is the
+//     error of the energy (59 bits below the range: 3e-15 to 1.3e-14 of theta
+//     on +-20 thermal speeds with a tail of 1e-9; here below 5e-16).
 //  h: three FP64 operations, summed as an integer.  (Parked over the column's x
 //     weight it takes two, 4 % of a step; but the rounding of the quotients
 //     and the product back drift by 0.025 to 0.03 of 2^-53 a step in a uniform
 //     state, rms, where this form drifts by 0.009 to 0.017.)
 // eg, eh: largest exponents of f~ that the sums' units are cut for (of f~
 // itself: a neighbour may be any number of times as large when its weight is
-// small).  On return they are the largest exponents seen; the sums are valid
-// when these do not exceed the ones passed in and the result is true (no lane's
-// sum ran over 63 bits).
+// small).  The sums are valid (true) when no value exceeds them; otherwise they
+// return raised to the largest exponents seen.
 template <int W, bool EDGE>
 __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables& T, const double2* __restrict__ fc,
                                                   ptrdiff_t row, const CellEdge& C, int wi,
                                                   double2* __restrict__ tile, double* __restrict__ sums, int& eg,
                                                   int& eh) {
   typedef unsigned long long u64;
-  const int lane = threadIdx.x & 31, nvx = P.nvx, nvy = P.nvy;
+  const int lane = threadIdx.x & 31, nvx = P.nvx, nvy = P.nvy, eu = eg + P.sum_room;
   const LaneMap<W> L(P, wi);
   const int h = L.row0, rpw = L.step, rows = L.rows;
-  unsigned over = 0;
   int topg = 0, toph = 0;
   const fx::i96 zero = {0u, 0u, 0u};
   fx::i96 hsum = zero, n0 = zero, x1 = zero, x2 = zero, i1 = zero, i2 = zero;
@@ -248,8 +250,7 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
     const int offx = EDGE ? sgx : -sgx * P.nv;  // upwind in x: ix - sgn c_x
     const u64 wx = T.wx[jx], rest = ((u64)1 << fx::kWeightBits) - wx;
     const double ax = T.awx[jx];
-    u64 s1 = 0;
-    fx::i96 s2 = zero, s3 = zero;
+    fx::i96 s1 = zero, s2 = zero, s3 = zero;
 #pragma unroll 1
     for (int r = 0; r < rows; ++r) {
       const int jr = h + r * rpw, jy = min(jr, nvy - 1), j = jy * nvx + jx;
@@ -279,24 +280,23 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
       if (in && jr < nvy) {
         const unsigned hg = (unsigned)__double2hiint(ft.x), hh = (unsigned)__double2hiint(ft.y);
         tile[j] = ft;
-        s1 += fx::double_to_units(hg, (unsigned)__double2loint(ft.x), (unsigned)eg);
-        hsum = fx::add(hsum, fx::wide(fx::double_to_units(hh, (unsigned)__double2loint(ft.y), (unsigned)eh)));
+        s1 = fx::add_units96(s1, hg, (unsigned)__double2loint(ft.x), (unsigned)eu);
+        hsum = fx::add(hsum, fx::double_to_units96(hh, (unsigned)__double2loint(ft.y), (unsigned)eh));
         topg = max(topg, (int)(hg >> 20));
         toph = max(toph, (int)(hh >> 20));
       }
-      s2 = fx::add(s2, fx::wide(s1));
+      s2 = fx::add(s2, s1);
       s3 = fx::add(s3, s2);
-      over |= (unsigned)(s1 >> 32);  // an addend is at most 2^59: the top bit shows before a sum wraps
     }
-    n0 = fx::add(n0, fx::wide(s1));
+    n0 = fx::add(n0, s1);
     i1 = fx::add(i1, s2);
     i2 = fx::add(i2, s3);
-    x1 = fx::add(x1, fx::mul(fx::wide(s1), (unsigned)jx));
-    x2 = fx::add(x2, fx::mul(fx::wide(s1), (unsigned)(jx * jx)));
+    x1 = fx::add(x1, fx::mul(s1, (unsigned)jx));
+    x2 = fx::add(x2, fx::mul(s1, (unsigned)(jx * jx)));
   }
   topg = __reduce_max_sync(0xffffffffu, topg);
   toph = __reduce_max_sync(0xffffffffu, toph);
-  const bool valid = topg <= eg && toph <= eh && !__any_sync(0xffffffffu, (int)over < 0);
+  const bool valid = topg <= eg && toph <= eh;
   if (valid) {
     // j_y of row r: A - rpw (rows - r); i1 = sum (rows - r) g, i2 = sum (rows - r)(rows - r + 1) / 2 g
     const unsigned A = (unsigned)(h + rpw * rows), B = (unsigned)rpw;
@@ -312,10 +312,10 @@ __device__ __forceinline__ bool stream_rows_fixed(const Params& P, const Tables&
     const fx::i96 k = lin ? fx::add(fx::mul(t, 2u), fx::muls(first, n))
                           : quad ? fx::add(fx::add(fx::mul(t, 4u), fx::muls(prev, 4 * n)), fx::mul(first, (unsigned)(n * n)))
                                  : t;
-    if ((lane & 3) == 0 && q < kSums) sums[q] = unit_value(k, q < 5 ? eg : eh);
+    if ((lane & 3) == 0 && q < kSums) sums[q] = unit_value(k, (q < 5 ? eu : eh) - 16);
   }
-  eg = topg;
-  eh = toph;
+  eg = max(eg, topg);
+  eh = max(eh, toph);
   return valid;
 }
 
@@ -374,7 +374,7 @@ __device__ __forceinline__ int stream_rows(const Params& P, const Tables& T, con
   int eg, eh;
   sample_range(fc, P.nv, eg, eh);
   const bool edge = C.xlo || C.xhi || C.ylo || C.yhi;
-  // a second pass takes the largest exponents of the first as its range
+  // a second pass takes the largest exponents of the first where they exceed the sampled ones
   for (int pass = 0; pass < 2; ++pass) {
     if (min(eg, eh) < (int)fx::kExpMin || max(eg, eh) > (int)fx::kExpMax) break;
     if (edge ? stream_rows_fixed<W, true>(P, T, fc, row, C, wi, tile, sums, eg, eh)
@@ -1374,13 +1374,21 @@ size_t step_f64_smem_bytes(const Params& P, int tile) { return step_smem(P, tile
 // Lanes per velocity row of the fixed-point kernels: the 4, 8, 16 or 32 that
 // leave the fewest lanes idle (more lanes on a tie, for wider accesses).  They
 // need weights that sum to one (Courant number at most 1), 128 velocities to
-// sample, and index sums within 95 bits (at most 512 velocities per axis).  In
-// 1D any non-zero value selects step1d_kernel.
+// sample, and sums fine enough (at most 512 velocities per axis): the sum of
+// squared indices times nv values of 75 - sum_room bits stays within 95 bits
+// (32^2: 75 bits a value, 48^2 and 64^2: 71, 8 x 512: 65).  In 1D any non-zero
+// value selects step1d_kernel.
 void step_f64_plan(Params& P, double max_courant) {
-  P.lane_bits = 0;
+  P.lane_bits = P.sum_room = 0;
   if (P.dim == 1 && P.nvx >= 8 && P.nvx <= 160 && P.bc_kind[XLO] == BC_INFLOW && P.bc_kind[XHI] == BC_INFLOW)
     P.lane_bits = 5;
   if (P.dim != 2 || P.nv < 128 || P.nvx > 512 || P.nvy > 512 || max_courant > 1.0 + 4e-15) return;
+  const auto bits = [](int n) {
+    int b = 0;
+    while (1 << b < n) ++b;
+    return b;
+  };
+  P.sum_room = std::max(0, bits(P.nv) + 2 * bits(std::max(P.nvx, P.nvy)) - 20);
   double best = 0.0;
   for (int lb = 5; lb >= 2; --lb) {
     const int lw = 1 << lb, rpw = 32 >> lb;

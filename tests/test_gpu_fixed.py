@@ -168,3 +168,36 @@ def test_uniform_state_does_not_drift(nvx, nvy, cfl):
     drift = (out[..., 1] / f[..., 1] - 1.0) / steps * 2.0 ** 53
     assert np.sqrt((drift ** 2).mean()) <= 0.02
     s.close()
+
+
+def tail_state(counts, box, ncell):
+    """A resting Maxwellian with a hot tail of 1e-9 on so many velocities per axis in +-box, the same in every cell,
+    and its n and theta in extended precision (the centres too: in FP64 each is off by an ulp of the box, up to 4e-15
+    of theta on the axis of 300)."""
+    exact = [(2 * np.arange(k) + 1 - k) * (np.longdouble(box) / k) for k in counts]
+    c = [x.astype(float) for x in exact]
+    m = [np.exp(-x * x) for x in c]
+    t = [np.exp(-x * x / 50.0) for x in c]
+    g = m[0] + 1e-9 * t[0] if len(c) == 1 else m[1][:, None] * m[0] + 1e-9 * t[1][:, None] * t[0]
+    h = (0.5 * g).ravel()
+    e = exact[0] ** 2 if len(c) == 1 else exact[1][:, None] ** 2 + exact[0] ** 2
+    G = g.astype(np.longdouble)
+    dv = np.prod([2 * np.longdouble(box) / k for k in counts])
+    theta = np.longdouble(2.0) / 3 * ((e * G).sum() + h.astype(np.longdouble).sum()) / G.sum()
+    return np.tile(g.ravel(), (ncell, 1)), np.tile(h, (ncell, 1)), float(G.sum() * dv), float(theta)
+
+
+@pytest.mark.parametrize("tile", [1, 2, 4, 8])
+@pytest.mark.parametrize("nvx,nvy,box", [(16, 16, 20.0), (32, 32, 20.0), (64, 64, 20.0), (32, 32, 10.0), (128, 32, 20.0),
+                                         (12, 300, 20.0)])
+def test_sums_of_a_tail_on_a_wide_box(nvx, nvy, box, tile):
+    # tail values 1e-9 of the peak carry most of sum c^2 g's rounding: the integer sums have to keep their low bits.
+    # Eight roundings of 2^-53 lie between the sums and theta
+    s, prob, *_ = pair(4, 3, nvx, nvy, cons=0, kinds=(2, 2, 2, 2), vx=(-box, box), vy=(-box, box), tile=tile)
+    g, h, n, theta = tail_state((nvx, nvy), box, prob.ncell)
+    s.set_state(np.ascontiguousarray(np.stack([g, h], -1)))
+    s.step(1)
+    m = s.moments(which=1)
+    assert np.abs(m[:, 0] / n - 1.0).max() <= 8 * 2.0 ** -53
+    assert np.abs(m[:, 3] / theta - 1.0).max() <= 8 * 2.0 ** -53
+    s.close()
