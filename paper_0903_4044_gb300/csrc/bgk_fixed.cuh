@@ -135,16 +135,8 @@ BGK_HD void to_words(u64 r, u32 emax, u32& hi, u32& lo) {
   hi = (u32)(m >> 32) + ((emax + 3u - lz) << 20);
 }
 
-// A positive double (words hi, lo) in the cell's unit 2^(eref - 1081), rounded;
-// at most 2^59 for an exponent field of at most eref.
-BGK_HD u64 double_to_units(u32 hi, u32 lo, u32 eref) {
-  const u64 m = (u64)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
-  const u32 d = eref - (hi >> 20);  // m 2^(6 - d)
-  return shr64(m << 8, d + 2u) + ((u32)shr64(m << 8, d + 1u) & 1u);
-}
-
-// The same in the unit 2^(eref - 1097), truncated: below 2^75 for an exponent
-// field of at most eref.
+// A positive double (words hi, lo) in the unit 2^(eref - 1097), truncated:
+// below 2^75 for an exponent field of at most eref.
 BGK_HD i96 double_to_units96(u32 hi, u32 lo, u32 eref) {
   const u64 m = ((u64)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 8;
   const u32 e = eref - (hi >> 20) + 2u;  // m 2^(16 - e)

@@ -17,14 +17,6 @@ __device__ __forceinline__ fx::i96 xor_add96(fx::i96 keep, fx::i96 send, int mas
   return fx::add(keep, got);
 }
 
-// A positive value (a sign bit counts as a large exponent) in the unit of
-// exponent eref; `top` keeps the largest of its exponent less `shift`.
-__device__ __forceinline__ unsigned long long units_of(double x, int eref, int shift, int& top) {
-  const unsigned hi = (unsigned)__double2hiint(x);
-  top = max(top, (int)(hi >> 20) - shift);
-  return fx::double_to_units(hi, (unsigned)__double2loint(x), (unsigned)eref);
-}
-
 // An integer in the unit 2^(eref - 1081) as a double.
 __device__ __forceinline__ double unit_value(fx::i96 v, int eref) {
   unsigned hi, lo;

@@ -1152,8 +1152,8 @@ namespace {
 
 // ---- 1D, inflow ends, at most 160 velocities ----------------------------------
 // One warp per cell and no barrier: f~ stays in registers (KV velocities per
-// lane), the moment sums are integers in units of the cell's largest exponent,
-// and the Gaussians and the relaxation weight come from the integer pipe, as
+// lane), the moment sums are integers in a unit 2^-72 of the cell's largest
+// exponent, and the Gaussians and the relaxation weight come from the integer pipe, as
 // in the 2D fixed-point kernels.  A cell's step is one chain of operations
 // (12 800 points give an SM one or two warps), so what counts is their number:
 // about 90 FP64 operations of 64 cycles where the FP64 form has 340.  Mach 2
@@ -1218,23 +1218,26 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
   }
   const unsigned eg = __reduce_max_sync(kAll, tg) >> 20, eh = __reduce_max_sync(kAll, th) >> 20;
   bool fit = min(eg, eh) >= fx::kExpMin && max(eg, eh) <= fx::kExpMax;
-  // A2: sums over (1, k, k^2, h), k = 2 j + 1 - nv
+  // A2: sums over (1, k, k^2, h), k = 2 j + 1 - nv: 160 values of 72 bits times
+  // 159^2 stay within 95 (59 bits left 9e-16 of theta on +-20 thermal speeds
+  // with a tail of 1e-9)
+  constexpr int kRoom = 3;
   const fx::i96 zero = {0u, 0u, 0u};
   fx::i96 v0 = zero, v1 = zero, v2 = zero, v3 = zero;
 #pragma unroll
   for (int k = 0; k < KV; ++k) {
     const int j = lane + 32 * k, kk = 2 * j + 1 - nv;
     if (j < nv) {
-      const fx::i96 g = fx::wide(fx::double_to_units((unsigned)__double2hiint(ft[k].x),
-                                                     (unsigned)__double2loint(ft[k].x), eg));
+      const fx::i96 g = fx::double_to_units96((unsigned)__double2hiint(ft[k].x), (unsigned)__double2loint(ft[k].x),
+                                              eg + kRoom);
       v0 = fx::add(v0, g);
       v1 = fx::add(v1, fx::muls(g, kk));
       v2 = fx::add(v2, fx::mul(g, (unsigned)(kk * kk)));
-      v3 = fx::add(v3, fx::wide(fx::double_to_units((unsigned)__double2hiint(ft[k].y),
-                                                    (unsigned)__double2loint(ft[k].y), eh)));
+      v3 = fx::add(v3, fx::double_to_units96((unsigned)__double2hiint(ft[k].y), (unsigned)__double2loint(ft[k].y),
+                                             eh + kRoom));
     }
   }
-  const double t = unit_value(warp_reduce4_96(v0, v1, v2, v3), (int)(lane < 24 ? eg : eh));
+  const double t = unit_value(warp_reduce4_96(v0, v1, v2, v3), (int)(lane < 24 ? eg : eh) + kRoom - 16);
   const double s0 = __shfl_sync(kAll, t, 0), s1 = __shfl_sync(kAll, t, 8), s2 = __shfl_sync(kAll, t, 16),
                sh = __shfl_sync(kAll, t, 24);
   // A3, every lane alike: moments about the box centre

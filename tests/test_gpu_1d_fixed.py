@@ -9,6 +9,7 @@ import oracle
 from paper_0903_4044_gb300 import bgk as B
 from paper_0903_4044_gb300 import build, solver
 from paper_0903_4044_gb300 import workloads as W
+from test_gpu_fixed import tail_state
 from test_gpu_parity import assert_moments_close, assert_state_close
 
 pytestmark = pytest.mark.gpu
@@ -84,4 +85,20 @@ def test_states_out_of_range(what):
         if what != "negative":
             assert (np.abs(a - b) <= 1e-12 * np.abs(b)).all()
     assert_moments_close(m, mom, vscale=1.0)
+    s.close()
+
+
+@pytest.mark.parametrize("nvx", [32, 64, 96, 160])
+def test_sums_of_a_tail_on_a_wide_box(nvx):
+    # as in test_gpu_fixed.py, in the cells that the ends do not reach
+    box, nx = 20.0, 12
+    rest = (1.0, 0.0, 0.0, 1.0)
+    s = solver.Solver(B.make_config(dim=1, nx=nx, lx=6.0, nvx=nvx, vx=(-box, box), cfl=0.5, conservative=0,
+                                    bc=[(B.BGK_BC_INFLOW, *rest)] * 2))
+    g, h, n, theta = tail_state((nvx,), box, nx)
+    s.set_state(np.ascontiguousarray(np.stack([g, h], -1)))
+    s.step(1)
+    m = s.moments(which=1)[2:-2]
+    assert np.abs(m[:, 0] / n - 1.0).max() <= 8 * 2.0 ** -53
+    assert np.abs(m[:, 3] / theta - 1.0).max() <= 8 * 2.0 ** -53
     s.close()
