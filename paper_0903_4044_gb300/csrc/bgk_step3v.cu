@@ -671,7 +671,7 @@ void plan3v(Params3v& P) {
   for (int a = 0; a < 3; ++a) {
     P.half[a] = 0.5 * P.dc[a];
     P.inv_half[a] = 1.0 / P.half[a];
-    P.mid[a] = P.vmin[a] + n3[a] * P.half[a];
+    P.mid[a] = std::fma((double)n3[a], P.half[a], P.vmin[a]);  // see velocity_grid
   }
   P.lane_bits = P.zw_bits = 0;
   if (P.nvx > 64 || P.nvy > 64 || P.nvz > 64) return;

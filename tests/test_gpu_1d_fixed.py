@@ -2,6 +2,8 @@
 every number of velocities per lane and its remainders, grids it leaves to the
 FP64-only kernel, shifts, options, and states out of its range.  Tolerances as
 in test_gpu_fixed.py."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -101,4 +103,18 @@ def test_sums_of_a_tail_on_a_wide_box(nvx):
     m = s.moments(which=1)[2:-2]
     assert np.abs(m[:, 0] / n - 1.0).max() <= 8 * 2.0 ** -53
     assert np.abs(m[:, 3] / theta - 1.0).max() <= 8 * 2.0 ** -53
+    s.close()
+
+@pytest.mark.parametrize("nvx", [32, 49])
+def test_symmetric_state_has_the_velocity_of_the_box_centre(nvx):
+    # as in test_gpu_fixed.py; the streaming weights are mirrored within a rounding only
+    rest = (1.0, 0.0, 0.0, 1.0)
+    s = solver.Solver(B.make_config(dim=1, nx=12, lx=6.0, nvx=nvx, vx=(-4.0, 4.0), cfl=0.5, conservative=0,
+                                    bc=[(B.BGK_BC_INFLOW, *rest)] * 2))
+    c = -4.0 + (np.arange(nvx) + 0.5) * (8.0 / nvx)
+    g = np.exp(-np.maximum(np.abs(c), np.abs(c[::-1])) ** 2)
+    s.set_state(np.tile(np.stack([g, 0.5 * g], -1), (12, 1, 1)))
+    s.step(1)
+    mid = float(Fraction(-4) + nvx * Fraction(8.0 / nvx) / 2)
+    assert np.abs(s.moments(which=1)[2:-2, 1] - mid).max() <= 2.0 ** -54
     s.close()

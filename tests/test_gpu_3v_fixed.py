@@ -3,6 +3,8 @@ oracle where it can go wrong: velocity counts that fill neither lanes nor
 warps, more columns than lanes, shifts beyond the domain, grids it leaves to
 the FP64 kernel, and states out of its range.  Tolerances as in
 test_gpu_fixed.py."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -70,3 +72,18 @@ def test_states_out_of_range(what):
     else:
         f[4, 3] += 20 * f.max()  # above the sampled range; more would leave theta a difference of large terms
     check(s, prob, f, 1, what == "negative")
+
+@pytest.mark.parametrize("nv", [(16, 16, 16), (49, 16, 16), (16, 49, 16), (14, 16, 49)])
+def test_symmetric_state_has_the_velocity_of_the_box_centre(nv):
+    # as in test_gpu_fixed.py: f2 - f1 = 0 in a uniform state, so f~ = f exactly
+    rest = (1.0, 0.0, 0.0, 0.0, 1.0)
+    s = solver.Solver3v(B.make_config3v(nx=8, lx=4.0, nv=nv, vmin=(-4.0,) * 3, vmax=(4.0,) * 3, cfl=0.5, conservative=0,
+                                        inflow=(rest, rest)))
+    c = [-4.0 + (np.arange(n) + 0.5) * (8.0 / n) for n in nv]
+    x, y, z = (np.exp(-np.maximum(np.abs(a), np.abs(a[::-1])) ** 2) for a in c)
+    f = (z[:, None, None] * y[:, None] * x).ravel()
+    s.set_state(np.tile(f, (8, 1)))
+    s.step(1)
+    mid = np.array([float(Fraction(-4) + n * Fraction(8.0 / n) / 2) for n in nv])
+    assert np.abs(s.moments(which=1)[2:-2, 1:4] - mid).max() <= 2.0 ** -54
+    s.close()

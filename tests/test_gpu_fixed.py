@@ -9,6 +9,8 @@ Tolerances as in test_gpu_parity.py: 1e-13 of the largest value and 1e-12 of
 each value per step.  Each rounds at most five times a step (streaming 2,
 relaxation 1, parameters), each to half an ulp of a sum of positive terms.
 """
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -200,4 +202,25 @@ def test_sums_of_a_tail_on_a_wide_box(nvx, nvy, box, tile):
     m = s.moments(which=1)
     assert np.abs(m[:, 0] / n - 1.0).max() <= 8 * 2.0 ** -53
     assert np.abs(m[:, 3] / theta - 1.0).max() <= 8 * 2.0 ** -53
+    s.close()
+
+@pytest.mark.parametrize("tile", [1, 2, 4, 8])
+@pytest.mark.parametrize("nvx,nvy,broad", [(32, 32, False), (49, 16, False), (16, 49, False), (64, 64, True), (12, 300, True)])
+def test_symmetric_state_has_the_velocity_of_the_box_centre(nvx, nvy, broad, tile):
+    # g mirrored in both axes: the integer sums over the indices cancel exactly whatever their order (sums in FP64
+    # do not) where one warp has the cell (tile 8), else within a rounding of the warps' sums.  What is left is the
+    # centre of the tabulated velocities -4 + (j + 1/2) dc, 3e-16 for 49.  broad: all values alike, the largest sums
+    # a lane can meet
+    s, prob, *_ = pair(4, 3, nvx, nvy, cons=0, kinds=(2, 2, 2, 2), vx=(-4.0, 4.0), vy=(-4.0, 4.0), tile=tile)
+    c = [-4.0 + (np.arange(n) + 0.5) * (8.0 / n) for n in (nvx, nvy)]
+    g = 0.5 + 0.5 * np.random.default_rng(1).random((nvy, nvx)) * (1 if broad else np.exp(-c[1][:, None] ** 2 - c[0] ** 2))
+    g = np.maximum(g, g[::-1])
+    g = np.maximum(g, g[:, ::-1]).ravel()
+    f = np.tile(np.stack([g, 0.5 * g], -1), (prob.ncell, 1, 1))
+    s.set_state(np.ascontiguousarray(f))
+    s.step(1)
+    m = s.moments(which=1)
+    for u, n in ((m[:, 1], nvx), (m[:, 2], nvy)):
+        mid = float(Fraction(-4) + n * Fraction(8.0 / n) / 2)
+        assert np.abs(u - mid).max() <= 2.0 ** -51 * abs(mid) + (0.0 if tile == 8 else 2.0 ** -53)
     s.close()
