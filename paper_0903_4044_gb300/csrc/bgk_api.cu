@@ -291,7 +291,7 @@ bgk_status validate(const bgk_config* c, bgk::Params* P, double* max_courant) {
         return fail(BGK_ERR_INVALID_ARG, "face %d: unknown boundary kind %d", face, b.kind);
     }
   }
-  if (c->precision == BGK_F64) bgk::step_f64_plan(p, *max_courant);
+  if (c->precision == BGK_F64) bgk::step_f64_plan(p, *max_courant, my * p.dt / p.dy);
   if (c->dim == 2 && *max_courant > 1.0 + 1e-12)
     return fail(BGK_ERR_UNSUPPORTED, "2D donor cell needs (max|cx|/dx + max|cy|/dy) dt <= 1 (got %.6g)",
                 *max_courant);

@@ -111,8 +111,9 @@ cudaError_t launch_step_f64(const Params& P, const Tables& T, const double2* fin
 cudaError_t launch_build_tables(const Params& P, double* cx, double* cy, double4_32a* coef, int* shift,
                                 double2* cxy, int* vinfo, double2* ghost, double* emitted, uint64_t* wx,
                                 uint64_t* wy, double* awx, double2* a0y, cudaStream_t stream);
-// Fills P.lane_bits (FP64) from the grid, the boundaries and the Courant number.
-void step_f64_plan(Params& P, double max_courant);
+// Fills P.lane_bits and P.sum_room (FP64) from the grid, the boundaries and the
+// Courant number (max_courant_y: its y part).
+void step_f64_plan(Params& P, double max_courant, double max_courant_y);
 size_t step_f64_smem_bytes(const Params& P, int tile);
 cudaError_t prepare_step_f64(const Params& P);
 cudaError_t launch_init_step(const Params& P, double2* f, double x_split, const double left[4],

@@ -1376,16 +1376,20 @@ size_t step_f64_smem_bytes(const Params& P, int tile) { return step_smem(P, tile
 
 // Lanes per velocity row of the fixed-point kernels: the 4, 8, 16 or 32 that
 // leave the fewest lanes idle (more lanes on a tie, for wider accesses).  They
-// need weights that sum to one (Courant number at most 1), 128 velocities to
+// need weights that sum to one (Courant number at most 1), y weights below one
+// (their top bit is the sign of c_y; the margin covers host and device
+// rounding: with it the x part is at most 2^-40 of one), 128 velocities to
 // sample, and sums fine enough (at most 512 velocities per axis): the sum of
 // squared indices times nv values of 75 - sum_room bits stays within 95 bits
 // (32^2: 75 bits a value, 48^2 and 64^2: 71, 8 x 512: 65).  In 1D any non-zero
 // value selects step1d_kernel.
-void step_f64_plan(Params& P, double max_courant) {
+void step_f64_plan(Params& P, double max_courant, double max_courant_y) {
   P.lane_bits = P.sum_room = 0;
   if (P.dim == 1 && P.nvx >= 8 && P.nvx <= 160 && P.bc_kind[XLO] == BC_INFLOW && P.bc_kind[XHI] == BC_INFLOW)
     P.lane_bits = 5;
-  if (P.dim != 2 || P.nv < 128 || P.nvx > 512 || P.nvy > 512 || max_courant > 1.0 + 4e-15) return;
+  if (P.dim != 2 || P.nv < 128 || P.nvx > 512 || P.nvy > 512 || max_courant > 1.0 + 4e-15 ||
+      max_courant_y > 1.0 - 0x1p-40)
+    return;
   const auto bits = [](int n) {
     int b = 0;
     while (1 << b < n) ++b;

@@ -31,9 +31,9 @@ def _lib():
 
 
 def pair(nx, ny, nvx, nvy, *, tile=0, vx=(-4.0, 4.0), vy=(-4.5, 4.5), cfl=0.6, cons=1, exact=1, kinds=(1, 1, 1, 1),
-         omega=0.5, n=1.0, length=0.5):
+         omega=0.5, n=1.0, length=0.5, lx=None, ly=None):
     rest, lid = (n, 0.0, 0.0, 1.0), (n, 0.05, 0.0, 1.0)
-    kw = dict(dim=2, nx=nx, ny=ny, lx=nx * length, ly=ny * length, nvx=nvx, nvy=nvy, vx=vx, vy=vy, cfl=cfl,
+    kw = dict(dim=2, nx=nx, ny=ny, lx=lx or nx * length, ly=ly or ny * length, nvx=nvx, nvy=nvy, vx=vx, vy=vy, cfl=cfl,
               conservative=cons, relax_exact=exact, omega=omega)
     cfg = B.make_config(**kw, bc=[(k, *s) for k, s in zip(kinds, (rest, rest, rest, lid))], tile_cells=tile)
     prob = oracle.Problem(oracle.make_config(**kw, bc_kind=kinds, bc_state=(rest, rest, rest, lid)))
@@ -223,4 +223,27 @@ def test_symmetric_state_has_the_velocity_of_the_box_centre(nvx, nvy, broad, til
     for u, n in ((m[:, 1], nvx), (m[:, 2], nvy)):
         mid = float(Fraction(-4) + n * Fraction(8.0 / n) / 2)
         assert np.abs(u - mid).max() <= 2.0 ** -51 * abs(mid) + (0.0 if tile == 8 else 2.0 ** -53)
+    s.close()
+
+
+def test_time_step_of_the_order_of_the_smallest_numbers():
+    # an infinity stays one
+    s, prob, g, h = pair(6, 5, 24, 20, cfl=1e-85, cons=0)
+    h[9, 5] = np.inf
+    s.set_state(np.ascontiguousarray(np.stack([g, h], -1)))
+    s.step(1)
+    with pytest.raises(B.BgkError) as e:
+        s.sync()
+    assert e.value.status == B.BGK_ERR_NUMERIC
+    s.close()
+
+
+@pytest.mark.parametrize("nvx", [21, 20])
+@pytest.mark.parametrize("sides", [dict(lx=1e22), dict(ly=1e22)])
+def test_courant_number_of_one_axis(sides, nvx):
+    # cells 1e22 times as long as high or as high as long: the fastest velocity's weight along one axis is one
+    s, prob, g, h = pair(6, 5, nvx, 16, cfl=1.0, vy=(-4.0, 4.0), **sides)
+    st, m, g1, h1, mom = run(s, prob, g, h, 1)
+    assert_state_close(st, g1, h1)
+    assert_moments_close(m, mom, vscale=0.05)
     s.close()
