@@ -253,12 +253,12 @@ BGK_HD u64 relax(u32 hi, u32 lo, u64 wb, int eb, u64 mphi, int ephi, int& e) {
   return mulhi(shr64(m, (u32)(e - e1)), wb) + shr64(mphi, (u32)(e - ephi) + 2u) + 1u;
 }
 
-// A double (words) with |x| < 32 in units of 2^-58, rounded.
+// A double (words) with |x| < 32 in units of 2^-58, rounded (0 below half of one).
 BGK_HD int64_t to_fix58(u32 hi, u32 lo) {
   const u32 e = (hi >> 20) & 0x7ffu;
   const u64 m = ((u64)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 10;  // m 2^(e - 1027)
-  const u32 d = 1027u - e, t = d < 63u ? d : 63u;
-  const u64 r = t ? (m >> t) + ((m >> (t - 1u)) & 1u) : m;
+  const u32 d = 1027u - e;
+  const u64 r = shr64(m, d) + ((u32)shr64(m, d - 1u) & 1u);
   return (hi >> 31) ? -(int64_t)r : (int64_t)r;
 }
 

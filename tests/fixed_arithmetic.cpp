@@ -25,10 +25,18 @@ static const u64 kTable[32] = BGK_EXP2_TABLE;
 int main() {
   std::mt19937_64 g(1);
   std::uniform_real_distribution<double> U(0, 1);
-  long double worst[6] = {0, 0, 0, 0, 0, 0};
+  long double worst[7] = {0, 0, 0, 0, 0, 0, 0};
   auto keep = [&](int k, long double got, long double want) {
     worst[k] = std::fmax(worst[k], std::fabs((got - want) / want));
   };
+  // to_fix58 over all exponents, zeros and subnormals
+  for (int t = 0; t < 100000; ++t) {
+    const double edge[] = {0.0, -0.0, 0x1p-59, -0x1p-59, 0x1p-60, -0x1p-60, 0x1.8p-59, 0x1.fffffffffffffp-60, 5e-324, 1e-300, 0x1.fffffffffffffp4};
+    const double x = t < 11 ? edge[t] : std::ldexp(2 * U(g) - 1, (int)(110 * U(g)) - 105);
+    u32 a, b;
+    words(x, a, b);
+    worst[6] = std::fmax(worst[6], std::fabs(to_fix58(a, b) - std::ldexp((long double)x, 58)));
+  }
   for (int t = 0; t < 300000; ++t) {
     u32 a, b, c, d, e, f, hi, lo, n;
     // donor-cell combination

@@ -11,7 +11,7 @@ def test_error_bounds(tmp_path):
     exe = str(tmp_path / "fixed")
     subprocess.run(["g++", "-O2", "-std=c++17", "-I", os.path.join(HERE, "..", "paper_0903_4044_gb300", "csrc"), "-x",
                     "c++", os.path.join(HERE, "fixed_arithmetic.cpp"), "-o", exe], check=True)
-    combine, units96, gauss, relax, wide, add96 = map(float, subprocess.run([exe], check=True, capture_output=True,
+    combine, units96, gauss, relax, wide, add96, fix58 = map(float, subprocess.run([exe], check=True, capture_output=True,
                                                                    text=True).stdout.split())
     half = 2.0 ** -53
     assert combine <= half + 2.0 ** -54   # the sum keeps at least 54 bits above three truncations of 2^-60
@@ -20,3 +20,4 @@ def test_error_bounds(tmp_path):
     assert wide <= half + 2.0 ** -60
     assert units96 == 0.0  # truncated
     assert add96 <= 0.5  # rounded
+    assert fix58 <= 0.5
