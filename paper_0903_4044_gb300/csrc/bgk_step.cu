@@ -784,7 +784,7 @@ struct FixedSolve {
   double ith, isq;
   double iq0, iq3, ivs;  // 1 / n, 1 / theta, 1 / sqrt(theta) of q
   int it;
-  bool conv, fail;
+  bool conv, out;  // out: parameters beyond the range of the FP32 starts, or no convergence (the FP64 path decides)
 };
 
 // Publishes the base point of a cell; false when it or a velocity lies too
@@ -836,9 +836,9 @@ __device__ __forceinline__ void eff_update(const VelocityGrid& V, const double (
     r = max(r, abs_hi(delta * (k == 0 ? E.iq0 : k == 3 ? E.iq3 : E.ivs)));
   }
   // the high words of kEffTol = 1e-13, sqrt(kEffTol / 100) = 3.16e-8 and kEffFail = 1e-9
-  if (!in_range(E.p[0]) || !in_range(E.p[3]) || r >= 0x7ff00000u) E.fail = true;
+  if (!in_range(E.p[0]) || !in_range(E.p[3]) || r >= 0x7ff00000u) E.out = true;
   else if (r < 0x3d3c25c2u || (E.it == 1 && r < 0x3e60fa33u)) E.conv = true;
-  else if (E.it >= kEffMaxIt) (r < 0x3e112e0bu ? E.conv : E.fail) = true;
+  else if (E.it >= kEffMaxIt) (r < 0x3e112e0bu ? E.conv : E.out) = true;
   E.isq = rsqrt3(E.p[3]);
   E.ith = E.isq * E.isq;
 }
@@ -917,7 +917,7 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
     E.iq0 = rcp3(E.q[0]);
     E.it = 0;
     E.conv = P.conservative == 0 || !ok;
-    E.fail = false;
+    E.out = false;
     if (wr) {
       const bool reach = publish_base(P, V, E, c, X);
       fit = fit && (reach || !ok);
@@ -938,16 +938,16 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
     __syncthreads();
     if (solving) {
       bool fit = true;
-      if (!E.conv && !E.fail) {
+      if (!E.conv) {
         double M[2][3];
         central_sums(X.sums[c][0], X.base[c][0].k0, V.half_x, V.mid_x, E.p[1], M[0]);
         central_sums(X.sums[c][1], X.base[c][1].k0, V.half_y, V.mid_y, E.p[2], M[1]);
         eff_update(V, M[0], M[1], E);
-        if (wr) fit = publish_base(P, V, E, c, X) || E.fail;
+        if (wr) fit = !E.out && publish_base(P, V, E, c, X);
       }
-      if (wr) X.need[c] = !E.conv && !E.fail;
+      if (wr) X.need[c] = !E.conv;
       const bool all = __all_sync(0xffffffffu, fit);
-      const bool any = __any_sync(0xffffffffu, wr && !E.conv && !E.fail);
+      const bool any = __any_sync(0xffffffffu, wr && !E.conv);
       if (lane == 0) X.go = !all ? -1 : any ? 1 : 0;
     }
     __syncthreads();
@@ -958,7 +958,6 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
     return false;
   }
   if (solving) {
-    if (E.fail) ok = false;
     if (!weighted) relax_weights_fixed(P, E, a, b);
     if (wr) {
       X.ap[c] = a * (E.p[0] * E.ith) * 0.31830988618379067;  // 1 / pi
@@ -968,7 +967,7 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
       if (live) {
         store4(mom + cell, qm[0], qm[1], qm[2], qm[3]);
         if (par) store4(par + cell, E.p[0], E.p[1], E.p[2], E.p[3]);
-        if (!ok) atomicOr(err, E.fail ? ERR_EFFECTIVE : ERR_MOMENT);
+        if (!ok) atomicOr(err, ERR_MOMENT);
       }
     }
   }
@@ -1254,7 +1253,6 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
     isq = rsqrt3(q[2]);
     fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, q[1], isq * 1.2011224087864498, B);
   }
-  bool fail = false;
   double a = 0.0, b = 0.0;
   if (fit) {
 #pragma unroll
@@ -1291,10 +1289,10 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
         p[2] += e2;
         const unsigned r = max(max(abs_hi(e0 * iq0), abs_hi(e1 * ivs)), abs_hi(e2 * iq2));
         // the high words of kEffTol = 1e-13, sqrt(kEffTol / 100) = 3.16e-8 and kEffFail = 1e-9
-        fail = !in_range(p[0]) || !in_range(p[2]) || r >= 0x7ff00000u;
         const bool conv = r < 0x3d3c25c2u || (it == 1 && r < 0x3e60fa33u) || (it >= kEffMaxIt && r < 0x3e112e0bu);
-        if (!fail && !conv && it >= kEffMaxIt) fail = true;
-        if (fail) break;
+        // beyond the range of the FP32 starts, or no convergence: the FP64 path decides
+        fit = in_range(p[0]) && in_range(p[2]) && r < 0x7ff00000u && (conv || it < kEffMaxIt);
+        if (!fit) break;
         isq = rsqrt3(p[2]);
         fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, p[1], isq * 1.2011224087864498, B);
         if (conv || !fit) break;
@@ -1309,23 +1307,18 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
   if (lane == 0) {
     store4(mom + cell, q[0], q[1], 0.0, q[2]);
     if (par) store4(par + cell, p[0], p[1], 0.0, p[2]);
-    if (fail) atomicOr(err, ERR_EFFECTIVE);
   }
-  // A4 (a failed cell keeps f~)
+  // A4
   const double ap = a * p[0] * isq * 0.5641895835477563;
 #pragma unroll
   for (int k = 0; k < KV; ++k) {
     const int j = lane + 32 * k;
     if (j < nv) {
-      if (!fail) {
-        unsigned n2, hi, lo;
-        const unsigned long long g = fx::gauss(B.a * (2 * j + 1 - nv) - B.c, (const fx::u64*)kExp2, n2);
-        fx::gauss_words(g, n2, hi, lo);
-        const double aphi = ap * __hiloint2double((int)hi, (int)lo);
-        ft[k].x = fma(b, ft[k].x, aphi);
-        ft[k].y = fma(b, ft[k].y, p[2] * aphi);
-      }
-      fo[j] = ft[k];
+      unsigned n2, hi, lo;
+      const unsigned long long g = fx::gauss(B.a * (2 * j + 1 - nv) - B.c, (const fx::u64*)kExp2, n2);
+      fx::gauss_words(g, n2, hi, lo);
+      const double aphi = ap * __hiloint2double((int)hi, (int)lo);
+      fo[j] = make_double2(fma(b, ft[k].x, aphi), fma(b, ft[k].y, p[2] * aphi));
     }
   }
 }

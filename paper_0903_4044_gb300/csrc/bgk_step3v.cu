@@ -364,8 +364,7 @@ __device__ __forceinline__ int sample3v(const Params3v& P, const double* __restr
 __device__ __forceinline__ void bar_solve() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
 
 // The cell's parameters on warps 0 to 3, from the totals in S.tot.  Leaves
-// S.ok, S.ab, the factors in fac and returns true, or false (S.ok = -1) when
-// the cell needs FP64.
+// S.go = 0, S.ab and the factors in fac, or S.go = -1 when the cell needs FP64.
 __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v& S, double* fac,
                                               double* __restrict__ mom, int* __restrict__ err) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -377,7 +376,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
     mid[a] = P.mid[a];
   }
   double q[5], p[5], ith = 1.0, isq = 1.0, iq0 = 1.0, iq4 = 1.0, ivs = 1.0;
-  bool ok = false, conv = true, fail = false;
+  bool conv = true;
   if (warp == 0) {  // all lanes alike
     const double* t = S.tot;
     bool fit = in_range(t[0]);
@@ -394,7 +393,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
       uu += u;
     }
     q[4] = (2.0 / 3.0) * e;
-    ok = q[0] > 0.0 && q[4] > 0.0 && isfinite(q[0]) && isfinite(q[4]) && isfinite(uu);
+    const bool ok = q[0] > 0.0 && q[4] > 0.0 && isfinite(q[0]) && isfinite(q[4]) && isfinite(uu);
     fit = fit && ok && in_range(q[0]) && in_range(q[4]);
     if (fit) {
       ivs = isq = rsqrt3(q[4]);
@@ -459,11 +458,10 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
       // the high words of kEffTol = 1e-13 and kEffFail = 1e-9 (no early stop: on
       // coarse grids, 16^3 on the paper's box, the contraction is 20 times the
       // first update, and the skipped one would show at 1e-14)
-      if (!in_range(p[0]) || !in_range(p[4]) || r >= 0x7ff00000u) fail = true;
-      else if (r < 0x3d3c25c2u) conv = true;
-      else if (it >= kEffMaxIt) (r < 0x3e112e0bu ? conv : fail) = true;
-      bool fit = true;
-      if (!fail) {
+      conv = r < 0x3d3c25c2u || (it >= kEffMaxIt && r < 0x3e112e0bu);
+      // beyond the range of the FP32 starts, or no convergence: the FP64 path decides
+      bool fit = in_range(p[0]) && in_range(p[4]) && r < 0x7ff00000u && (conv || it < kEffMaxIt);
+      if (fit) {
         isq = rsqrt3(p[4]);
         ith = isq * isq;
 #pragma unroll
@@ -473,19 +471,16 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
           if (lane == 0) S.base[a] = B;
         }
       }
-      if (lane == 0) S.go = !fit ? -1 : conv || fail ? 0 : 1;
+      if (lane == 0) S.go = !fit ? -1 : conv ? 0 : 1;
     }
     bar_solve();
   }
   if (S.go < 0) return;
   bar_solve();  // the weights of warp 3, when there was no round
   if (warp == 0) {
-    if (fail) ok = false;
     if (lane == 0) {
-      S.ok = ok ? 1 : 0;
       S.tot[6] = S.ab[0] * p[0] * (ith * isq) * (1.0 / 5.568327996831708);
       for (int k = 0; k < 5; ++k) mom[(size_t)i * 5 + k] = q[k];
-      if (!ok) atomicOr(err, fail ? ERR_EFFECTIVE : ERR_MOMENT);
     }
   }
   bar_solve();
@@ -539,7 +534,6 @@ __global__ void __launch_bounds__(kT, 4) step3v_fixed_kernel(const Params3v P, c
     cell3v_f64(P, T, fin, fout, mom, err, i, fac, S);
     return;
   }
-  if (!S.ok) return;  // a failed cell keeps f~ (flagged)
   // pass 2: f^{n+1} = b f~ + a Phi on the rows of pass 1
   const Map3v L(P);
   const int nvx = P.nvx, nvy = P.nvy, ys = L.ystep * nvx;

@@ -87,3 +87,20 @@ def test_symmetric_state_has_the_velocity_of_the_box_centre(nv):
     mid = np.array([float(Fraction(-4) + n * Fraction(8.0 / n) / 2) for n in nv])
     assert np.abs(s.moments(which=1)[2:-2, 1:4] - mid).max() <= 2.0 ** -54
     s.close()
+
+
+def test_effective_parameters_at_the_range_end():
+    # as in test_gpu_1d_fixed.py (the other end is the sums' own, which lie further out)
+    n = 2.0 ** 97 * 0.99
+    c = -8.0 + (np.arange(12) + 0.5) * (16.0 / 12)
+    e = np.exp(-c * c)
+    f = (e[:, None, None] * e[:, None] * e).ravel()
+    f *= n / (f.sum() * (16.0 / 12) ** 3)
+    end = (n, 0.0, 0.0, 0.0, 1.0)
+    s = solver.Solver3v(B.make_config3v(nx=8, lx=4.0, nv=(12,) * 3, vmin=(-8.0,) * 3, vmax=(8.0,) * 3, cfl=0.5, omega=1.0,
+                                        inflow=(end, end)))
+    s.set_state(np.tile(f, (8, 1)))
+    s.step(1)
+    s.sync()
+    assert np.abs(s.moments(which=1)[2:-2, 0] / n - 1.0).max() <= 1e-12
+    s.close()
