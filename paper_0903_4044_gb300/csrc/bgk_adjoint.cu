@@ -265,7 +265,7 @@ __device__ __forceinline__ void row_factors(const Params& P, const Tables& T, co
   double ith, pref;
   if (fit) {
     const double isq = rsqrt3(p.w), gamma = isq * 1.2011224087864498;  // sqrt(log2 e)
-    ith = isq * isq;
+    ith = rcp3(p.w);
     pref = p.x * ith * 0.31830988618379067;
     fit = axis_base(nvx, V.half_x, V.inv_half_x, V.mid_x, p.y, gamma, A) &&
           axis_base(nvy, V.half_y, V.inv_half_y, V.mid_y, p.z, gamma, B);

@@ -54,23 +54,33 @@ __device__ __forceinline__ bool in_range(double x) {
 }
 __device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
-// 2^-t for 0 <= t < 32 on the integer pipe.
-__device__ __forceinline__ double exp2_neg_fixed(double t) {
-  const unsigned long long f = (unsigned long long)fx::to_fix58((unsigned)__double2hiint(t), (unsigned)__double2loint(t));
+// 2^-t, t in units of 2^-58 below 2^63, times 2^up.
+__device__ __forceinline__ double exp2_neg_fixed(unsigned long long t, unsigned up) {
   unsigned hi, lo;
-  fx::gauss_words(fx::exp2_neg(f << 6, (const fx::u64*)kExp2), (unsigned)(f >> 58), hi, lo);
+  fx::gauss_words(fx::exp2_neg(t << 6, (const fx::u64*)kExp2), (unsigned)(t >> 58) - up, hi, lo);
   return __hiloint2double((int)hi, (int)lo);
 }
-// e^-x; the argument's rounding is that of the product with log2 e.
+// e^-x.  The product with log2 e is taken to 2^-57 (rounded to a double it
+// cost 14 times 2^-53 of e^-x at x = 20).
 __device__ __forceinline__ double exp_neg_fixed(double x) {
-  const double t = x * 1.4426950408889634;  // log2 e
-  return t >= 0.0 && t < 32.0 ? exp2_neg_fixed(t) : exp(-x);
+  const unsigned h = (unsigned)__double2hiint(x);
+  if (h >= 0x40360000u) return exp(-x);  // 22 and more, negative, NaN
+  const unsigned long long u = (unsigned long long)fx::to_fix58(h, (unsigned)__double2loint(x)) << 1;
+  return exp2_neg_fixed(fx::mulhi(u, 0xb8aa3b295c17f0bcull), 0u);  // 2^63 log2 e
 }
-// x^y as 2^(y log2 x): one third of pow's FP64 operations, as accurate (1.5e-16)
-// while the exponent's magnitude is below one.
+// x^y as 2^(y log2 x), the product as an integer: one third of pow's FP64
+// operations.  Error 2^-53 of log2 x and the last rounding while the exponent's
+// magnitude is below one.
 __device__ __forceinline__ double pow_fixed(double x, double y) {
-  const double e = y * log2(x);
-  return fabs(e) < 1.0 ? 2.0 * exp2_neg_fixed(1.0 - e) : pow(x, y);
+  const double l = log2(x);
+  const unsigned hl = (unsigned)__double2hiint(l), hy = (unsigned)__double2hiint(y);
+  if (max(hl & 0x7fffffffu, hy & 0x7fffffffu) >= 0x40400000u) return pow(x, y);  // 32 and more, NaN
+  const long long a = fx::to_fix58(hl, (unsigned)__double2loint(l)), b = fx::to_fix58(hy, (unsigned)__double2loint(y));
+  const unsigned long long ua = (unsigned long long)(a < 0 ? -a : a), ub = (unsigned long long)(b < 0 ? -b : b);
+  const unsigned long long top = __umul64hi(ua, ub);
+  if (top >= 1ull << 52) return pow(x, y);  // one and more
+  const long long e = (long long)(top << 6 | (ua * ub) >> 58);
+  return exp2_neg_fixed((unsigned long long)((1ll << 58) - ((a ^ b) < 0 ? -e : e)), 1u);
 }
 
 // One axis of a cell's Gaussians at a base point: (c_k - u) sqrt(log2 e /

@@ -840,7 +840,7 @@ __device__ __forceinline__ void eff_update(const VelocityGrid& V, const double (
   else if (r < 0x3d3c25c2u || (E.it == 1 && r < 0x3e60fa33u)) E.conv = true;
   else if (E.it >= kEffMaxIt) (r < 0x3e112e0bu ? E.conv : E.out) = true;
   E.isq = rsqrt3(E.p[3]);
-  E.ith = E.isq * E.isq;
+  E.ith = rcp3(E.p[3]);
 }
 
 // Which axis of its cell a warp works on, with which lane of how many: half a
@@ -913,7 +913,7 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
 #pragma unroll
     for (int k = 0; k < 4; ++k) E.q[k] = E.p[k] = ok && fit ? qm[k] : (k == 0 || k == 3) ? 1.0 : 0.0;
     E.ivs = E.isq = rsqrt3(E.q[3]);
-    E.iq3 = E.ith = E.isq * E.isq;
+    E.iq3 = E.ith = rcp3(E.q[3]);
     E.iq0 = rcp3(E.q[0]);
     E.it = 0;
     E.conv = P.conservative == 0 || !ok;

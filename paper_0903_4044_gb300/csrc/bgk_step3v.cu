@@ -397,7 +397,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
     fit = fit && ok && in_range(q[0]) && in_range(q[4]);
     if (fit) {
       ivs = isq = rsqrt3(q[4]);
-      iq4 = ith = isq * isq;
+      iq4 = ith = rcp3(q[4]);
       iq0 = rcp3(q[0]);
     }
 #pragma unroll
@@ -463,7 +463,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
       bool fit = in_range(p[0]) && in_range(p[4]) && r < 0x7ff00000u && (conv || it < kEffMaxIt);
       if (fit) {
         isq = rsqrt3(p[4]);
-        ith = isq * isq;
+        ith = rcp3(p[4]);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
           AxisBase B;
