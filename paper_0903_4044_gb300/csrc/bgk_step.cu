@@ -785,21 +785,16 @@ struct FixedSolve {
   double iq0, iq3, ivs;  // 1 / n, 1 / theta, 1 / sqrt(theta) of q
   int it;
   bool conv, out;  // out: parameters beyond the range of the FP32 starts, or no convergence (the FP64 path decides)
-  // n / (pi theta), the same in D(p) and in Phi: a constant rounded one way in
-  // one and another way in the other is a density that changes with every step
-  __device__ __forceinline__ double prefactor() const {
-    const double t = p[0] * ith;
-    return fma(t, 0.31830988618379067, t * -1.9678676675182486e-17);  // 1 / pi
-  }
 };
 
 // Publishes the base point of a cell; false when it or a velocity lies too
 // far out for the fixed-point Gaussian.
 template <int G>
 __device__ __forceinline__ bool publish_base(const Params& P, const VelocityGrid& V, const FixedSolve& E, int c, CellSolve<G>& X) {
+  const double gamma = E.isq * 1.2011224087864498;  // sqrt(log2 e)
   AxisBase x, y;
-  const bool fx = axis_base(P.nvx, V.half_x, V.inv_half_x, V.mid_x, E.p[1], E.isq, x);
-  const bool fy = axis_base(P.nvy, V.half_y, V.inv_half_y, V.mid_y, E.p[2], E.isq, y);
+  const bool fx = axis_base(P.nvx, V.half_x, V.inv_half_x, V.mid_x, E.p[1], gamma, x);
+  const bool fy = axis_base(P.nvy, V.half_y, V.inv_half_y, V.mid_y, E.p[2], gamma, y);
   X.base[c][0] = x;
   X.base[c][1] = y;
   return fx && fy;
@@ -821,14 +816,14 @@ __device__ __forceinline__ void relax_weights_fixed(const Params& P, const Fixed
 
 // One update p <- p + (q - D(p)) (A3) from the central sums M_m of both axes
 // at p, with the stopping rules of eff_iterate.
-__device__ __forceinline__ void eff_update(double dv, const double (&Mx)[3], const double (&My)[3],
+__device__ __forceinline__ void eff_update(const VelocityGrid& V, const double (&Mx)[3], const double (&My)[3],
                                            FixedSolve& E) {
   ++E.it;
   const double rxy = rcp3(Mx[0] * My[0]);
   const double rx = My[0] * rxy, ry = Mx[0] * rxy;
   const double mux = Mx[1] * rx, muy = My[1] * ry;
   double d[4];
-  d[0] = E.prefactor() * dv * (Mx[0] * My[0]);
+  d[0] = (E.p[0] * E.ith) * V.dv_pi * (Mx[0] * My[0]);
   d[1] = E.p[1] + mux;
   d[2] = E.p[2] + muy;
   const double var = fma(Mx[2], rx, -mux * mux) + fma(My[2], ry, -muy * muy);
@@ -947,7 +942,7 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
         double M[2][3];
         central_sums(X.sums[c][0], X.base[c][0].k0, V.half_x, V.mid_x, E.p[1], M[0]);
         central_sums(X.sums[c][1], X.base[c][1].k0, V.half_y, V.mid_y, E.p[2], M[1]);
-        eff_update(P.dv, M[0], M[1], E);
+        eff_update(V, M[0], M[1], E);
         if (wr) fit = !E.out && publish_base(P, V, E, c, X);
       }
       if (wr) X.need[c] = !E.conv;
@@ -965,7 +960,7 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
   if (solving) {
     if (!weighted) relax_weights_fixed(P, E, a, b);
     if (wr) {
-      X.ap[c] = a * E.prefactor();
+      X.ap[c] = a * (E.p[0] * E.ith) * 0.31830988618379067;  // 1 / pi
       sb[c] = b;
       sk[c] = 0.5 * E.p[3];
       sok[c] = ok ? 1 : 0;
@@ -1256,7 +1251,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
   double isq = 1.0;
   if (fit) {
     isq = rsqrt3(q[2]);
-    fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, q[1], isq, B);
+    fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, q[1], isq * 1.2011224087864498, B);
   }
   double a = 0.0, b = 0.0;
   if (fit) {
@@ -1286,7 +1281,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
         double M[3];
         central_sums(ks, B.k0, V.half_x, V.mid_x, p[1], M);
         const double r0 = rcp3(M[0]), mu = M[1] * r0;
-        const double d0 = p[0] * isq * 0.5641895835477563 * P.dv * M[0];  // 1 / sqrt(pi); prefactor as in A4
+        const double d0 = p[0] * isq * (P.dv * 0.5641895835477563) * M[0];  // 1 / sqrt(pi)
         const double d2 = (2.0 / 3.0) * (fma(M[2], r0, -mu * mu) + p[2]);
         const double e0 = q[0] - d0, e1 = q[1] - (p[1] + mu), e2 = q[2] - d2;
         p[0] += e0;
@@ -1299,7 +1294,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
         fit = in_range(p[0]) && in_range(p[2]) && r < 0x7ff00000u && (conv || it < kEffMaxIt);
         if (!fit) break;
         isq = rsqrt3(p[2]);
-        fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, p[1], isq, B);
+        fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, p[1], isq * 1.2011224087864498, B);
         if (conv || !fit) break;
       }
     }
@@ -1314,7 +1309,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
     if (par) store4(par + cell, p[0], p[1], 0.0, p[2]);
   }
   // A4
-  const double ap = a * (p[0] * isq * 0.5641895835477563);
+  const double ap = a * p[0] * isq * 0.5641895835477563;
 #pragma unroll
   for (int k = 0; k < KV; ++k) {
     const int j = lane + 32 * k;
