@@ -47,7 +47,7 @@ struct Params {
 // Numbers of the velocity grid that the fixed-point step uses (FP64).
 struct VelocityGrid {
   double half_x, half_y, inv_half_x, inv_half_y;  // half velocity steps and their reciprocals
-  double mid_x, mid_y, dv_pi;                     // box centres, dv / pi
+  double mid_x, mid_y;                            // box centres
 };
 // The centres are those of the tabulated velocities min + (j + 1/2) dc, to the
 // last bit of dc (by an fma, whether or not the host compiler contracts): the
@@ -61,7 +61,6 @@ inline VelocityGrid velocity_grid(const Params& P) {
   g.inv_half_y = 1.0 / g.half_y;
   g.mid_x = std::fma((double)P.nvx, g.half_x, P.vx_min);
   g.mid_y = std::fma((double)P.nvy, g.half_y, P.vy_min);
-  g.dv_pi = P.dv / 3.14159265358979323846;
   return g;
 }
 

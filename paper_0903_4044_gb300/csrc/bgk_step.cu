@@ -785,6 +785,12 @@ struct FixedSolve {
   double iq0, iq3, ivs;  // 1 / n, 1 / theta, 1 / sqrt(theta) of q
   int it;
   bool conv, out;  // out: parameters beyond the range of the FP32 starts, or no convergence (the FP64 path decides)
+  // n / (pi theta), the same in D(p) and in Phi: a constant rounded one way in
+  // one and another way in the other is a density that changes with every step
+  __device__ __forceinline__ double prefactor() const {
+    const double t = p[0] * ith;
+    return fma(t, 0.31830988618379067, t * -1.9678676675182486e-17);  // 1 / pi
+  }
 };
 
 // Publishes the base point of a cell; false when it or a velocity lies too
@@ -816,14 +822,14 @@ __device__ __forceinline__ void relax_weights_fixed(const Params& P, const Fixed
 
 // One update p <- p + (q - D(p)) (A3) from the central sums M_m of both axes
 // at p, with the stopping rules of eff_iterate.
-__device__ __forceinline__ void eff_update(const VelocityGrid& V, const double (&Mx)[3], const double (&My)[3],
+__device__ __forceinline__ void eff_update(double dv, const double (&Mx)[3], const double (&My)[3],
                                            FixedSolve& E) {
   ++E.it;
   const double rxy = rcp3(Mx[0] * My[0]);
   const double rx = My[0] * rxy, ry = Mx[0] * rxy;
   const double mux = Mx[1] * rx, muy = My[1] * ry;
   double d[4];
-  d[0] = (E.p[0] * E.ith) * V.dv_pi * (Mx[0] * My[0]);
+  d[0] = E.prefactor() * dv * (Mx[0] * My[0]);
   d[1] = E.p[1] + mux;
   d[2] = E.p[2] + muy;
   const double var = fma(Mx[2], rx, -mux * mux) + fma(My[2], ry, -muy * muy);
@@ -942,7 +948,7 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
         double M[2][3];
         central_sums(X.sums[c][0], X.base[c][0].k0, V.half_x, V.mid_x, E.p[1], M[0]);
         central_sums(X.sums[c][1], X.base[c][1].k0, V.half_y, V.mid_y, E.p[2], M[1]);
-        eff_update(V, M[0], M[1], E);
+        eff_update(P.dv, M[0], M[1], E);
         if (wr) fit = !E.out && publish_base(P, V, E, c, X);
       }
       if (wr) X.need[c] = !E.conv;
@@ -960,7 +966,7 @@ __device__ __forceinline__ bool maxwellian_cells_fixed(const Params& P, const Ta
   if (solving) {
     if (!weighted) relax_weights_fixed(P, E, a, b);
     if (wr) {
-      X.ap[c] = a * (E.p[0] * E.ith) * 0.31830988618379067;  // 1 / pi
+      X.ap[c] = a * E.prefactor();
       sb[c] = b;
       sk[c] = 0.5 * E.p[3];
       sok[c] = ok ? 1 : 0;
@@ -1281,7 +1287,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
         double M[3];
         central_sums(ks, B.k0, V.half_x, V.mid_x, p[1], M);
         const double r0 = rcp3(M[0]), mu = M[1] * r0;
-        const double d0 = p[0] * isq * (P.dv * 0.5641895835477563) * M[0];  // 1 / sqrt(pi)
+        const double d0 = p[0] * isq * 0.5641895835477563 * P.dv * M[0];  // 1 / sqrt(pi); prefactor as in A4
         const double d2 = (2.0 / 3.0) * (fma(M[2], r0, -mu * mu) + p[2]);
         const double e0 = q[0] - d0, e1 = q[1] - (p[1] + mu), e2 = q[2] - d2;
         p[0] += e0;
@@ -1309,7 +1315,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
     if (par) store4(par + cell, p[0], p[1], 0.0, p[2]);
   }
   // A4
-  const double ap = a * p[0] * isq * 0.5641895835477563;
+  const double ap = a * (p[0] * isq * 0.5641895835477563);
 #pragma unroll
   for (int k = 0; k < KV; ++k) {
     const int j = lane + 32 * k;

@@ -360,6 +360,8 @@ __device__ __forceinline__ int sample3v(const Params3v& P, const double* __restr
   return (int)((__reduce_max_sync(0xffffffffu, m) >> 20) + fx::kHeadroom);
 }
 
+constexpr double kPi15 = 0.17958712212516656;  // pi^(-3/2); the prefactor is the same in D(p) and in Phi
+
 // Warps 0 to 2 (an axis each) and 3 (the relaxation weight).
 __device__ __forceinline__ void bar_solve() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
 
@@ -438,8 +440,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
       double M[3][3], d[5];
 #pragma unroll
       for (int a = 0; a < 3; ++a) central_sums(S.ax[a], S.base[a].k0, half[a], mid[a], p[1 + a], M[a]);
-      const double pi15 = 5.568327996831708;  // pi^(3/2)
-      d[0] = p[0] * (ith * isq) * (P.dv / pi15) * (M[0][0] * M[1][0] * M[2][0]);
+      d[0] = p[0] * (ith * isq) * kPi15 * P.dv * (M[0][0] * M[1][0] * M[2][0]);
       double var = 0.0;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -479,7 +480,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
   bar_solve();  // the weights of warp 3, when there was no round
   if (warp == 0) {
     if (lane == 0) {
-      S.tot[6] = S.ab[0] * p[0] * (ith * isq) * (1.0 / 5.568327996831708);
+      S.tot[6] = S.ab[0] * (p[0] * (ith * isq) * kPi15);
       for (int k = 0; k < 5; ++k) mom[(size_t)i * 5 + k] = q[k];
     }
   }

@@ -134,3 +134,23 @@ def test_effective_parameters_at_the_range_ends(n, nvx):
     s.sync()
     assert np.abs(s.moments(which=1)[2:-2, 0] / n - 1.0).max() <= 1e-12
     s.close()
+
+
+def test_collisions_keep_density_and_temperature():
+    # as in test_gpu_fixed.py, in cells that the ends do not reach (FP64-only form: 0.058 and 0.046)
+    drift = []
+    for box in (5.6, 5.7, 5.83, 6.0, 6.1, 6.25):
+        for n, theta in ((24, 1.0), (28, 0.93), (31, 1.07)):
+            s = solver.Solver(B.make_config(dim=1, nx=220, lx=8800.0, nvx=n, vx=(-box, box), cfl=0.5,
+                                            bc=[(B.BGK_BC_INFLOW, 1.0, 0.0, 0.0, theta)] * 2))
+            c = -box + (np.arange(n) + 0.5) * (2 * box / n)
+            for density in np.linspace(1.0, 1.9, 10):
+                g = density * np.exp(-c * c / theta) / np.sqrt(np.pi * theta)
+                s.set_state(np.tile(np.stack([g, theta * g], -1), (220, 1, 1)))
+                s.step(1)
+                m0 = s.moments(which=1)[105:115]
+                s.step(100)
+                drift.append((s.moments(which=1)[105:115, [0, 3]] / m0[:, [0, 3]] - 1.0).mean(0) / 100 * 2.0 ** 53)
+            s.close()
+    rms = np.sqrt((np.array(drift) ** 2).mean(0))
+    assert (rms <= 0.12).all(), rms
