@@ -264,11 +264,11 @@ __device__ __forceinline__ void row_factors(const Params& P, const Tables& T, co
   bool fit = in_range(p.x) && in_range(p.w);
   double ith, pref;
   if (fit) {
-    const double isq = rsqrt3(p.w), gamma = isq * 1.2011224087864498;  // sqrt(log2 e)
+    const double isq = rsqrt3(p.w);
     ith = rcp3(p.w);
     pref = p.x * ith * 0.31830988618379067;
-    fit = axis_base(nvx, V.half_x, V.inv_half_x, V.mid_x, p.y, gamma, A) &&
-          axis_base(nvy, V.half_y, V.inv_half_y, V.mid_y, p.z, gamma, B);
+    fit = axis_base(nvx, V.half_x, V.inv_half_x, V.mid_x, p.y, isq, A) &&
+          axis_base(nvy, V.half_y, V.inv_half_y, V.mid_y, p.z, isq, B);
   } else {
     ith = 1.0 / p.w;
     pref = p.x / (kPi() * p.w);

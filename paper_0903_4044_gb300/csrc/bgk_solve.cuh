@@ -92,20 +92,28 @@ struct AxisBase {
 };
 constexpr int kMaxIndexShift = 1024;  // |k0|: keeps sum k'^2 e within 95 bits
 
+// x sqrt(log2 e), rounded, |x| below 2^62 (a double's sqrt(log2 e) is 0.22 of
+// 2^-53 too small: twice that in the width of every Gaussian, with one sign).
+__device__ __forceinline__ long long times_sqrt_log2e(long long x) {
+  const unsigned long long k = 0x99be610c1d827eefull;  // 2^63 sqrt(log2 e)
+  const unsigned long long u = (unsigned long long)(x < 0 ? -x : x) << 1;
+  const long long r = (long long)(__umul64hi(u, k) + ((u * k) >> 63));
+  return x < 0 ? -r : r;
+}
 
 // The base of an axis of n velocity cells of half width `half`, centre `mid`,
-// at mean u; gamma = sqrt(log2 e / theta).  False when a velocity lies too far
-// out for the fixed-point Gaussian.
-__device__ __forceinline__ bool axis_base(int n, double half, double inv_half, double mid, double u, double gamma,
+// at mean u; isq = 1 / sqrt(theta).  False when a velocity lies too far out for
+// the fixed-point Gaussian.
+__device__ __forceinline__ bool axis_base(int n, double half, double inv_half, double mid, double u, double isq,
                                           AxisBase& B) {
-  const double off = u - mid, a = half * gamma, s = off * gamma;
+  const double off = u - mid, a = half * isq, s = off * isq;
   const double r = fma(off, inv_half, 6755399441055744.0);  // 1.5 2^52: rounds to an integer
   const double reach = fma(a, (double)n, fabs(s));
   B.k0 = __double2loint(r);
-  B.a = fx::to_fix58((unsigned)__double2hiint(a), (unsigned)__double2loint(a));
-  B.c = fx::to_fix58((unsigned)__double2hiint(s), (unsigned)__double2loint(s));
-  // |s| + a n < 31.9, |off| below kMaxIndexShift half steps (words: the exponent decides)
-  return abs_hi(reach) < 0x403fe666u && abs_hi(r) == 0x43380000u - (B.k0 < 0 ? 1u : 0u) &&
+  B.a = times_sqrt_log2e(fx::to_fix58((unsigned)__double2hiint(a), (unsigned)__double2loint(a)));
+  B.c = times_sqrt_log2e(fx::to_fix58((unsigned)__double2hiint(s), (unsigned)__double2loint(s)));
+  // |s| + a n < 26.55, times sqrt(log2 e) 31.9; |off| below kMaxIndexShift half steps (words: the exponent decides)
+  return abs_hi(reach) < 0x403a8cccu && abs_hi(r) == 0x43380000u - (B.k0 < 0 ? 1u : 0u) &&
          (unsigned)(B.k0 + kMaxIndexShift) < 2u * kMaxIndexShift;
 }
 

@@ -797,10 +797,9 @@ struct FixedSolve {
 // far out for the fixed-point Gaussian.
 template <int G>
 __device__ __forceinline__ bool publish_base(const Params& P, const VelocityGrid& V, const FixedSolve& E, int c, CellSolve<G>& X) {
-  const double gamma = E.isq * 1.2011224087864498;  // sqrt(log2 e)
   AxisBase x, y;
-  const bool fx = axis_base(P.nvx, V.half_x, V.inv_half_x, V.mid_x, E.p[1], gamma, x);
-  const bool fy = axis_base(P.nvy, V.half_y, V.inv_half_y, V.mid_y, E.p[2], gamma, y);
+  const bool fx = axis_base(P.nvx, V.half_x, V.inv_half_x, V.mid_x, E.p[1], E.isq, x);
+  const bool fy = axis_base(P.nvy, V.half_y, V.inv_half_y, V.mid_y, E.p[2], E.isq, y);
   X.base[c][0] = x;
   X.base[c][1] = y;
   return fx && fy;
@@ -1257,7 +1256,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
   double isq = 1.0;
   if (fit) {
     isq = rsqrt3(q[2]);
-    fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, q[1], isq * 1.2011224087864498, B);
+    fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, q[1], isq, B);
   }
   double a = 0.0, b = 0.0;
   if (fit) {
@@ -1300,7 +1299,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const double2* __restrict__
         fit = in_range(p[0]) && in_range(p[2]) && r < 0x7ff00000u && (conv || it < kEffMaxIt);
         if (!fit) break;
         isq = rsqrt3(p[2]);
-        fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, p[1], isq * 1.2011224087864498, B);
+        fit = axis_base(nv, V.half_x, V.inv_half_x, V.mid_x, p[1], isq, B);
         if (conv || !fit) break;
       }
     }

@@ -408,7 +408,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         AxisBase B;
-        fit = axis_base(n3[a], half[a], P.inv_half[a], mid[a], p[1 + a], isq * 1.2011224087864498, B) && fit;
+        fit = axis_base(n3[a], half[a], P.inv_half[a], mid[a], p[1 + a], isq, B) && fit;
         if (lane == 0) S.base[a] = B;
       }
     }
@@ -468,7 +468,7 @@ __device__ __forceinline__ void solve3v_fixed(const Params3v& P, int i, Shared3v
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
           AxisBase B;
-          fit = axis_base(n3[a], half[a], P.inv_half[a], mid[a], p[1 + a], isq * 1.2011224087864498, B) && fit;
+          fit = axis_base(n3[a], half[a], P.inv_half[a], mid[a], p[1 + a], isq, B) && fit;
           if (lane == 0) S.base[a] = B;
         }
       }

@@ -279,4 +279,4 @@ def test_collisions_keep_density_and_temperature():
                 drift.append((s.moments(which=1)[:, [0, 3]] / m0[:, [0, 3]] - 1.0).mean(0) / 100 * 2.0 ** 53)
             s.close()
     rms = np.sqrt((np.array(drift) ** 2).mean(0))
-    assert (rms <= 0.3).all(), rms
+    assert (rms <= 0.16).all(), rms
