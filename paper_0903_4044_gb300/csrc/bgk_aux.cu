@@ -47,7 +47,7 @@ __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32
     // unsplit donor cell: f~ = (1 - |Cx| - |Cy|) f + |Cx| f_upx + |Cy| f_upy
     const double ax = fabs(cxj) * P.dt / P.dx;
     const double ay = fabs(cyj) * P.dt / P.dy;
-    coef[j] = make_double4_32a(1.0 - ax - ay, ax, ay, c2);
+    store4(coef + j, 1.0 - ax - ay, ax, ay, c2);
     shift[j] = 0;
     // the weights as integers over 2^63, rounded; where that would make a sum
     // of two exceed one (Courant number 1), the x weight gives way
@@ -64,7 +64,7 @@ __global__ void tables_kernel(const Params P, double* cx, double* cy, double4_32
     const double C = cxj * P.dt / P.dx;
     const int s = (int)C;
     const double r = fabs(C - s);
-    coef[j] = make_double4_32a(1.0 - r, r, 0.0, c2);
+    store4(coef + j, 1.0 - r, r, 0.0, c2);
     shift[j] = s;
   }
 }
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(256) moments_kernel(const Params P, const Tabl
   if (threadIdx.x == 0) {
     double q[4];
     moments_from_sums(tot[0], tot[1], tot[2], tot[3], P.dv, q);
-    mom[cell] = make_double4_32a(q[0], q[1], q[2], q[3]);
+    store4(mom + cell, q[0], q[1], q[2], q[3]);
   }
 }
 
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(256) wall_flux_kernel(const Params P, const Ta
     e = fma(cn, fma(T.coef[j].w, F.x, F.y), e);
   }
   block_reduce4<256>(m, s, pn, e, red, tot);
-  if (threadIdx.x == 0) out[k] = make_double4_32a(tot[0] * P.dv, tot[1] * P.dv, tot[2] * P.dv, tot[3] * P.dv);
+  if (threadIdx.x == 0) store4(out + k, tot[0] * P.dv, tot[1] * P.dv, tot[2] * P.dv, tot[3] * P.dv);
 }
 
 cudaError_t launch_wall_fluxes(const Params& P, const Tables& T, const double2* f, int face,

@@ -8,6 +8,17 @@ namespace bgk {
 
 __device__ __forceinline__ double kPi() { return 3.14159265358979323846; }
 
+// Four doubles as two 16-byte stores, for every double4_32a in memory.  As one
+// 32-byte assignment in a function that is called (the FP64 path of the 1D step),
+// nvcc 13.0.88 stored the first value and three zeros while the same function
+// went on to use the right ones; inlined, or in halves as here, all four arrive
+// (test_gpu_1d_fixed.py, states out of range).
+__device__ __forceinline__ void store4(double4_32a* p, double x, double y, double z, double w) {
+  double2* q = reinterpret_cast<double2*>(p);
+  q[0] = make_double2(x, y);
+  q[1] = make_double2(z, w);
+}
+
 // ---------------------------------------------------------------------------
 // Reductions.  FP64 adds run on the (slow) FP64 pipe of sm_103, so sums of
 // several values use recursive halving: at each xor level a lane keeps half

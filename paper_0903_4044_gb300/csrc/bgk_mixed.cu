@@ -1220,7 +1220,7 @@ __global__ void msum_moments_kernel(const Params P, const MixedTables M, int pre
   }
   double q[4];
   moments_from_sums(s[0], s[1], s[2], s[3], P.dv, q);
-  mom[cell] = make_double4_32a(q[0], q[1], q[2], q[3]);
+  store4(mom + cell, q[0], q[1], q[2], q[3]);
 }
 
 cudaError_t launch_msum_moments(const Params& P, int prec, const MixedTables& M, const float2* msum,

@@ -49,15 +49,6 @@ __device__ __forceinline__ int vi_jy(int vi) { return (vi >> 12) & 0xfff; }
 __device__ __forceinline__ int vi_sx(int vi) { return ((vi >> 24) & 3) - 1; }
 __device__ __forceinline__ int vi_sy(int vi) { return ((vi >> 26) & 3) - 1; }
 
-// Four doubles as two 16-byte stores: the 32-byte store that nvcc 13.0 makes of
-// a double4_32a assignment lost its last three values in step1d_kernel's
-// out-of-range path (a test checks those moments).
-__device__ __forceinline__ void store4(double4_32a* p, double x, double y, double z, double w) {
-  double2* q = reinterpret_cast<double2*>(p);
-  q[0] = make_double2(x, y);
-  q[1] = make_double2(z, w);
-}
-
 // Boundary value at velocity j (components jx, jy) for a face of the cell
 // whose state starts at fc.
 __device__ __forceinline__ double2 ghost_at(const Params& P, const Tables& T, int face, int j, int jx,
@@ -1165,15 +1156,12 @@ namespace {
 
 // Sum over the warp of four 96-bit values per lane: lane L ends with value
 // (L >> 3) & 3 (recursive halving, as warp_reduce4).
-__device__ __forceinline__ fx::i96 pick96(bool c, fx::i96 x, fx::i96 y) {
-  return {c ? x.a0 : y.a0, c ? x.a1 : y.a1, c ? x.a2 : y.a2};
-}
 __device__ __forceinline__ fx::i96 warp_reduce4_96(fx::i96 v0, fx::i96 v1, fx::i96 v2, fx::i96 v3) {
   const int lane = threadIdx.x & 31;
   const bool b4 = lane & 16, b3 = lane & 8;
-  const fx::i96 a = xor_add96(pick96(b4, v2, v0), pick96(b4, v0, v2), 16);
-  const fx::i96 b = xor_add96(pick96(b4, v3, v1), pick96(b4, v1, v3), 16);
-  fx::i96 x = xor_add96(pick96(b3, b, a), pick96(b3, a, b), 8);
+  const fx::i96 a = xor_add96(pick(b4, v2, v0), pick(b4, v0, v2), 16);
+  const fx::i96 b = xor_add96(pick(b4, v3, v1), pick(b4, v1, v3), 16);
+  fx::i96 x = xor_add96(pick(b3, b, a), pick(b3, a, b), 8);
   x = xor_add96(x, x, 4);
   x = xor_add96(x, x, 2);
   return xor_add96(x, x, 1);
