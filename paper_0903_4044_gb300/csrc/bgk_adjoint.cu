@@ -392,8 +392,9 @@ __device__ __forceinline__ double rcp_any(double x) { return in_range(x) ? rcp3(
 //   collide = 0: out = lambda^{n+1} (the last launch, giving lambda^0).
 // dghost, demit: d/dU_W of the lid's unit Maxwellian and of its emitted flux.
 // The per-cell coefficients are computed cells-in-lanes by warp 0.  24 warps
-// per SM at 80 registers.  128^2 x 32^2: 0.84 -> 0.60 ms a step; the FP64 pipe
-// stays the bound (17.4 operations per velocity, 98 % of its measured rate).
+// per SM at 80 registers.  128^2 x 32^2: 0.84 -> 0.62 ms a step; the FP64 pipe
+// stays the bound (19.6 operations issued per velocity instead of 23.4, all of
+// its measured rate).
 template <int G>
 __global__ void __launch_bounds__(32 * G, 24 / G) adj_step_kernel(const Params P, const Tables T,
                                                           const double2* __restrict__ fn1,

@@ -59,8 +59,9 @@ struct bgk_solver {
   double4_32a* mom_tmp = nullptr;   // scratch for bgk_moments(which = 0)
   double4_32a* flux_tmp = nullptr;  // scratch for bgk_wall_fluxes
   double* cx = nullptr;
-  double* cy = nullptr;  // [2 nvy]: centres, then the fixed-point y weights
-  uint64_t* wx = nullptr;  // [nvx] fixed-point x weights
+  double* cy = nullptr;
+  uint64_t* wx = nullptr;   // [nvx] fixed-point x weights
+  uint64_t* wy = nullptr;   // [nvy] fixed-point y weights
   double* awx = nullptr;    // [nvx] |c_x| dt / dx
   double2* a0y = nullptr;   // [nv] (a0, ay)
   double4_32a* coef = nullptr;
@@ -86,14 +87,13 @@ struct bgk_solver {
   int64_t device_bytes = 0;
   double max_courant = 0.0;
 
-  uint64_t* y_weights() const { return reinterpret_cast<uint64_t*>(cy + P.nvy); }
   bgk::Tables tables() const {
     bgk::Tables T;
     T.cx = cx;
     T.cy = cy;
     T.grid = bgk::velocity_grid(P);
     T.wx = wx;
-    T.wy = y_weights();
+    T.wy = wy;
     T.awx = awx;
     T.a0y = a0y;
     T.coef = coef;
@@ -303,12 +303,14 @@ bgk_status validate(const bgk_config* c, bgk::Params* P, double* max_courant) {
 // Largest tile (cells per CTA) that keeps two CTAs' shared memory within an
 // SM and still gives every SM at least two CTAs.  The fixed-point FP64 step
 // runs 8 warps per CTA at every tile: 8 cells share one scalar solve, 4 or 2
-// cells split each over 2 or 4 warps.  Measured us per step (2 / 4 / 8 cells):
-// 16^2 x 16^2 19 / 21 / 25, 32^2 x 32^2 53 / 49 / 63, 64^2 x 32^2 130 / 105 /
-// 108, 64^2 x 48^2 233 / 211 / 244, 96^2 x 20^2 221 / 140 / 107, 128^2 x 32^2
-// 424 / 332 / 316, 256^2 x 48^2 3020 / 2630 / 2360: 8 from three full waves
-// (4 CTAs per SM) on, and from 40 cells per SM on grids of few velocities,
-// where the solve weighs more.
+// cells split each over 2 or 4 warps.  Measured us per step of a run (2 / 4 / 8
+// cells): 16^2 x 16^2 19 / 21 / 25, 26^2 x 32^2 46 / 51 / 67, 28^2 x 16^2 25 / 24 /
+// 25, 28^2 x 48^2 80 / 97 / 127, 32^2 x 32^2 53 / 50 / 69, 64^2 x 32^2 135 / 109 /
+// 112, 64^2 x 48^2 241 / 219 / 252, 80^2 x 20^2 162 / 106 / 89, 96^2 x 20^2 222 /
+// 144 / 112, 110^2 x 32^2 337 / 266 / 259, 128^2 x 32^2 443 / 345 / 331, 128^2 x
+// 48^2 757 / 670 / 683, 256^2 x 48^2 2860 / 2410 / 2330: 4 from 5 cells per SM (28^2
+// on 152 SMs) on, 8 from three full waves (4 CTAs per SM) on, and from 40 cells
+// per SM on grids of few velocities, where the solve weighs more.
 int auto_tile(const bgk::Params& P, int prec, int sms) {
   const long long ncell = (long long)P.nx * P.ny;
   if (prec == BGK_F64 && P.dim == 2 && P.lane_bits) {
@@ -344,7 +346,7 @@ void release(bgk_solver* s) {
   for (auto& g : s->graph)
     if (g) cudaGraphExecDestroy(g);
   void* bufs[] = {s->f[0], s->f[1], s->stage, s->mom_step, s->mom_tmp, s->flux_tmp, s->cx, s->cy,
-                  s->coef, s->shift, s->cxy, s->vinfo, s->ghost, s->emitted, s->wx, s->awx, s->a0y, s->m_coef, s->m_cx,
+                  s->coef, s->shift, s->cxy, s->vinfo, s->ghost, s->emitted, s->wx, s->wy, s->awx, s->a0y, s->m_coef, s->m_cx,
                   s->m_cy, s->m_ax, s->m_ay, s->m_ghost, s->m_mabs, s->m_sums, s->m_ctr, s->err};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -535,8 +537,9 @@ bgk_status bgk_create(const bgk_config* cfg, bgk_solver** out) {
   ALLOC(mom_tmp, ncell);
   ALLOC(flux_tmp, nfc);
   ALLOC(cx, P.nvx);
-  ALLOC(cy, 2 * (size_t)P.nvy);
+  ALLOC(cy, P.nvy);
   ALLOC(wx, P.nvx);
+  ALLOC(wy, P.nvy);
   ALLOC(awx, P.nvx);
   ALLOC(a0y, P.nv);
   ALLOC(coef, P.nv);
@@ -555,7 +558,7 @@ bgk_status bgk_create(const bgk_config* cfg, bgk_solver** out) {
   if (e == cudaSuccess && s->m_ctr) e = cudaMemsetAsync(s->m_ctr, 0, 2 * sizeof(unsigned), s->stream);
   if (e == cudaSuccess)
     e = bgk::launch_build_tables(P, s->cx, s->cy, s->coef, s->shift, s->cxy, s->vinfo, s->ghost,
-                                 s->emitted, s->wx, s->y_weights(), s->awx, s->a0y, s->stream);
+                                 s->emitted, s->wx, s->wy, s->awx, s->a0y, s->stream);
   if (e == cudaSuccess && s->prec != bgk::PREC_F64) e = bgk::launch_build_mixed_tables(P, s->tables(), s->mtables(), s->stream);
   if (e == cudaSuccess) e = s->prec == bgk::PREC_F64 ? bgk::prepare_step_f64(P) : bgk::prepare_step_mixed(P, s->prec);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -908,7 +911,7 @@ extern "C" bgk_status bgk_step_noalloc(const bgk_config* cfg, const double* f_in
   double* emitted = (double*)(base + o_emit);
   int* err = (int*)(base + o_err);
   uint64_t* wx = (uint64_t*)(base + kNoAllocScratchBytes);
-  uint64_t* wy = (uint64_t*)(cy + P.nvy);
+  uint64_t* wy = (uint64_t*)(base + o_cy + sizeof(double) * P.nvy);
   double* awx = (double*)(wx + bgk::kMaxNv / 2);
   double2* a0y = (double2*)(awx + bgk::kMaxNv / 2);
   T.cx = cx;

@@ -24,14 +24,15 @@
 // nearly all of its per-cell work to the integer pipe as fixed-point
 // arithmetic (bgk_fixed.cuh) that rounds less than the FP64 form: g streams
 // and h relaxes on the integer pipe while h streams and g relaxes on the FP64
-// pipe (2 FP64 operations per velocity and phase), the moment sums are exact
-// integers, and the Gaussians are evaluated directly; 5 FP64 operations per
-// velocity in all instead of 15 to 19.  Measured against the FP64-only form:
-// 256^2 x 48^2 4.11 -> 2.36 ms, 64^2 x 32^2 167 -> 105 us, 157 x 83 cells x 20
-// x 28 velocities 320 -> 185 us a step; error of a 20-step run against exact
-// 64-bit sums 8.8e-16 -> 2.9e-16.  What bounds it now: 300 instructions per
-// warp and velocity (46 % of the issue slots), upwind loads and the parked f~
-// that L2 does not hold (82 B of DRAM traffic per update).
+// pipe (3 and 2 FP64 operations per velocity), the moment sums are integers of
+// 65 to 75 bits a value, and the Gaussians are evaluated directly; 5.6 FP64
+// operations per velocity in all instead of 15 to 19.  Measured against the
+// FP64-only form, state in and moments out included: 20 steps of 256^2 x 48^2
+// 85.4 -> 49.7 ms, 100 of 64^2 x 32^2 16.9 -> 11.2 ms, 50 of 157 x 83 cells x 20
+// x 28 velocities 16.3 -> 9.4 ms; error of the 20 steps against 64-bit sums
+// 8.8e-16 -> 4.6e-16.  What bounds it now: 332 thread instructions per update
+// (50 % of the issue slots), upwind loads and the parked f~ that L2 does not
+// hold (75.5 B of DRAM traffic per update, 128^2 x 48^2).
 //
 // step1d_kernel is the same for 1D grids; step_f64_kernel is the FP64-only
 // form, for the grids that step_f64_plan leaves to it.
@@ -196,27 +197,29 @@ struct LaneMap {
 };
 
 // Rows ahead that a lane asks into L1: with 8 warps per sub-partition at 64
-// registers the next row's values cannot wait in registers (256^2 x 48^2:
-// 2.57 ms without, 2.36 ms with 1 to 4 rows).
+// registers the next row's values cannot wait in registers (20 steps of 256^2 x
+// 48^2: 51.3 ms without, 47.1 ms with 1 to 4 rows, before the sums of 65 to 75
+// bits and h's third operation).
 constexpr int kAhead = 2;
 __device__ __forceinline__ void prefetch_l1(const double2* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
 // A1 + A2 of a warp's rows of a 2D cell, g on the integer pipe and h on the
-// FP64 pipe, which run side by side (measured per 256^2 x 48^2 step: both on
-// the FP64 pipe 2.64 ms, both on the integer pipe 3.18 ms, this 2.36 ms); a
-// column's weights and running sums stay in registers.
+// FP64 pipe, which run side by side (20 steps of 256^2 x 48^2, before the sums
+// of 65 to 75 bits and h's third operation: both on the FP64 pipe 52.7 ms, both
+// on the integer pipe 58.7 ms, this 47.1 ms); a column's weights and running
+// sums stay in registers.
 //  g: fixed point.  The running sums of first, second and third order over a
 //     column's rows give sum g, sum j_y g and sum j_y^2 g as integers, and
 //     times j_x the x sums.  Their unit has to lie far below the tail of a
 //     narrow distribution: weighted with the squared index its rounding is the
 //     error of the energy (59 bits below the range: 3e-15 to 1.3e-14 of theta
-//     on +-20 thermal speeds with a tail of 1e-9; here below 5e-16).
+//     on +-20 thermal speeds with a tail of 1e-9; here below 9e-16).
 //  h: three FP64 operations, summed as an integer.  (Parked over the column's x
-//     weight it takes two, 4 % of a step; but the rounding of the quotients
-//     and the product back drift by 0.025 to 0.03 of 2^-53 a step in a uniform
-//     state, rms, where this form drifts by 0.009 to 0.017.)
+//     weight it takes two, 4 % of the time; but with the rounding of the
+//     quotients and of the product back h of a uniform state drifts by 0.024 to
+//     0.031 of 2^-53 a step, rms, here by 0.009 to 0.017.)
 // eg, eh: largest exponents of f~ that the sums' units are cut for (of f~
 // itself: a neighbour may be any number of times as large when its weight is
 // small).  The sums are valid (true) when no value exceeds them; otherwise they
@@ -1152,7 +1155,8 @@ namespace {
 // in the 2D fixed-point kernels.  A cell's step is one chain of operations
 // (12 800 points give an SM one or two warps), so what counts is their number:
 // about 90 FP64 operations of 64 cycles where the FP64 form has 340.  Mach 2
-// shock, 200 cells x 64 velocities: 11.6 -> 7.1 us a step.
+// shock, 200 cells x 64 velocities, 200 steps with state in and moments out:
+// 2396 -> 1445 us.
 
 // Sum over the warp of four 96-bit values per lane: lane L ends with value
 // (L >> 3) & 3 (recursive halving, as warp_reduce4).

@@ -220,10 +220,12 @@ namespace {
 // ---- fixed-point kernel -------------------------------------------------------
 // The FP64 pipe takes 64 to 76 cycles per warp instruction and bounded the
 // step (12.1 operations per velocity).  Here four remain, two to stream and
-// two to relax; the moment sums are exact integers, the Gaussians and the
-// relaxation weight come from the integer pipe.  2048 x 30^3: 1.24 -> 0.65 ms a
-// step, 512 x 16^3: 126 -> 51 us.  What bounds it now: pass 1 (half of the
-// time) by its loads, each lane's column comes from another cell (8 of each 32
+// two to relax; the moment sums are integers of 75 bits a value, the Gaussians
+// and the relaxation weight come from the integer pipe.  With state in and
+// moments out: 10 steps of 2048 x 30^3 13.2 -> 7.3 ms, 20 of 512 x 16^3 2.61 ->
+// 1.06 ms.  What bounds it now: the FP64 pipe at 97 % of its measured rate on
+// 608 x 30^3 (5.0 operations issued per velocity, idle lanes and solve
+// included); in pass 1 each lane's column comes from another cell (8 of each 32
 // bytes are used); the solve of a 16^3 cell takes as long as its passes.
 //
 // 2^lane_bits lanes share a velocity row (fixed jy, jz); the 8 warps split z
@@ -263,8 +265,8 @@ __device__ __forceinline__ void axis_weights(fx::i96 r0, fx::i96 r1, fx::i96 r2,
                fx::mul(r2, (unsigned)(2 * B * B)));
 }
 
-// Rows whose values are loaded together (2048 x 30^3: 0.77 ms a step with 4,
-// 0.71 with 8).
+// Rows whose values are loaded together (2048 x 30^3, a step, at the time the
+// line was drawn: 0.77 ms with 4, 0.71 with 8; 0.65 since).
 constexpr int kAhead3 = 8;
 
 // Pass 1 of the warp's rows: f~ into fo, the sums of (1, k_x, k_x^2,
@@ -660,7 +662,12 @@ cudaError_t launch_init3v(const Params3v& P, const Tables3v& T, double x_split, 
 // a step on 100 cells and 342 on 600, 58 and 121 with one column of 16 rows.  More
 // lanes per row, then more warps along z, unless the gain is above 3 %.  The
 // fixed-point kernel takes at most 64 velocities per axis (its squared indices
-// and sums then stay within 95 bits).
+// and sums then stay within 95 bits), and no plan that leaves more than 70 % of
+// the lanes idle: a few dozen velocities or an axis just past a power of two.  On
+// 600 cells, us a step fixed / FP64: 3 x 20 x 1 (23 % in use) 38 / 29, 9 x 17 x 1
+// (30 %) 33 / 22, 33 x 3 x 3 (29 %) 38 / 37, 5^3 (24 %) 33 / 34, 4^3 (25 %) 24 / 33,
+// 9^3 (28 %) 29 / 41; above the line 5 x 33 x 1 (32 %) 35 / 35, 34 x 5 x 5 (33 %) 43
+// / 39, 10^3 (39 %) 30 / 43, 6^3 (42 %) 23 / 35, 8^3 25 / 37.
 void plan3v(Params3v& P) {
   const int n3[3] = {P.nvx, P.nvy, P.nvz};
   for (int a = 0; a < 3; ++a) {

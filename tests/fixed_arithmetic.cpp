@@ -42,7 +42,9 @@ int main() {
     // donor-cell combination
     const double f0 = std::pow(10.0, -30 * U(g)) * (0.1 + U(g));
     const double fx = f0 * std::exp(4 * (U(g) - 0.5)), fy = f0 * std::exp(4 * (U(g) - 0.5));
-    const u64 wx = (u64)(U(g) * 0.6 * 0x1p63), wy = (u64)(U(g) * 0.4 * 0x1p63), w0 = ((u64)1 << 63) - wx - wy;
+    // every third pair of weights is spread over 60 powers of two
+    const double small = t % 3 ? 1.0 : std::ldexp(1.0, -(int)(60 * U(g)));
+    const u64 wx = (u64)(U(g) * 0.6 * small * 0x1p63), wy = (u64)(U(g) * 0.4 * small * 0x1p63), w0 = ((u64)1 << 63) - wx - wy;
     words(f0, a, b);
     words(fx, c, d);
     words(fy, e, f);
@@ -65,7 +67,7 @@ int main() {
     words(x, a, b);
     const u64 qx = gauss(to_fix58(a, b), kTable, n);
     gauss_words(qx, n, hi, lo);
-    if (std::fabs(x) < 3) keep(2, value(hi, lo), std::exp2(-(long double)x * x));
+    keep(2, value(hi, lo), std::exp2(-(long double)x * x));
     const double p = std::exp2(-x * x - y * y), bw = t % 3 ? 1 - 0.3 * U(g) : std::ldexp(U(g) + 0.1, -(int)(40 * U(g)));
     const double ka = 0.1 + U(g), ft = p * std::exp(4 * (U(g) - 0.5));
     words(p, a, b);

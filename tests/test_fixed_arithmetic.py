@@ -15,7 +15,7 @@ def test_error_bounds(tmp_path):
                                                                    text=True).stdout.split())
     half = 2.0 ** -53
     assert combine <= half + 2.0 ** -54   # the sum keeps at least 54 bits above three truncations of 2^-60
-    assert gauss <= half + 2.0 ** -56 + 18 * 2.0 ** -58  # 2^-56.6 of the series, 2 w dw of the argument (w < 3)
+    assert gauss <= half + 2.0 ** -56 + 6 * 2.0 ** -58  # 2^-56.6 of the series, 2 w dw ln 2 of the argument (w < 8, dw 2^-59)
     assert relax <= half + 2.0 ** -55
     assert wide <= half + 2.0 ** -60
     assert units96 == 0.0  # truncated

@@ -6,7 +6,7 @@ zero values, steep fronts, densities far from one, relaxation weights beyond
 one), for which the kernels fall back to FP64.
 
 Tolerances as in test_gpu_parity.py: 1e-13 of the largest value and 1e-12 of
-each value per step.  Each rounds at most five times a step (streaming 2,
+each value per step.  Each rounds at most five times a step (streaming 3,
 relaxation 1, parameters), each to half an ulp of a sum of positive terms.
 """
 from fractions import Fraction
