@@ -65,20 +65,23 @@ CAVITY256_200 = "cavity_kn0.05_ma0.05_256x256_v48x48_200steps"
 # and the kernel name must match, else traffic is reported as null.  The
 # capture commands sit with the ncu summaries under profiles/.
 MEASURED_TRAFFIC = {
-    # captured on 128^2 x 48^2 (2.858 GB per launch, 75.7 B per update: the parked
+    # captured on 128^2 x 48^2 (2.852 GB per launch, 75.5 B per update: the parked
     # f~ of the resident cells exceeds L2 at 48^2 velocities) and scaled by the 4x
-    # updates of a 256^2 x 48^2 launch
+    # updates of a 256^2 x 48^2 launch; the reduced forms on 192^2 x 48^2 (1.440 and
+    # 0.642 GB), by 16 / 9
     (CAVITY256_200, "f64"): {
-        "bytes": 4 * 2.858e9,
+        "bytes": 4 * 2.852e9,
         "sources": ("csrc/bgk_step.cu", "csrc/bgk_fixed.cuh", "csrc/bgk_solve.cuh", "csrc/bgk_device.cuh"),
-        "sha1": "42e95ff1f5618e6ea5c37cba9eeaadb991a6651d", "kernel": "bgk::step_fixed_kernel",
+        "sha1": "0f71d175ff6db07ad85460a015fb9baccfdeca78", "kernel": "bgk::step_fixed_kernel",
         "note": "captured on 128^2 x 48^2 cells x velocities, scaled by updates"},
     (CAVITY256_200, "f32"): {
-        "bytes": 2.544e9, "sources": ("csrc/bgk_mixed.cu", "csrc/bgk_device.cuh"),
-        "sha1": "b79fe2943df7966e824c40d48003f385d010c245", "kernel": "bgk::step_mixed_pipe_kernel"},
+        "bytes": 2.560e9, "sources": ("csrc/bgk_mixed.cu", "csrc/bgk_device.cuh"),
+        "sha1": "33cd522e76338868e309a6858e436105d4d54fb6", "kernel": "bgk::step_mixed_pipe_kernel",
+        "note": "captured on 192^2 x 48^2 cells x velocities, scaled by updates"},
     (CAVITY256_200, "bf16"): {
-        "bytes": 1.171e9, "sources": ("csrc/bgk_mixed.cu", "csrc/bgk_device.cuh"),
-        "sha1": "b79fe2943df7966e824c40d48003f385d010c245", "kernel": "bgk::step_mixed_kernel"},
+        "bytes": 1.142e9, "sources": ("csrc/bgk_mixed.cu", "csrc/bgk_device.cuh"),
+        "sha1": "33cd522e76338868e309a6858e436105d4d54fb6", "kernel": "bgk::step_mixed_kernel",
+        "note": "captured on 192^2 x 48^2 cells x velocities, scaled by updates"},
 }
 
 
